@@ -1,6 +1,7 @@
 // Dense contractions on CUDA cores: grouped GEMM and valid 3x3 convolutions as
 // implicit GEMMs.  These are the plain FP32 path of the update (and, in FP64,
-// the reference-precision kernels the layer-level gradient checks use).
+// the reference-precision kernels the layer-level gradient checks use).  FP32 GEMMs whose
+// operands have a unit stride run in sq_gemm_f32.cu; the kernel here takes FP64 and the rest.
 //
 // Tile: 64 x 64 outputs x 16 reduction steps per stage, 256 threads, 4 x 4
 // outputs per thread, operands staged in shared memory k-major.
@@ -108,6 +109,7 @@ __global__ void __launch_bounds__(NT) gemm_kernel(GemmBatch gb) {
 
 template <typename T>
 void launch_gemm(const GemmProblem* probs, int n_probs, GemmLayout layout, cudaStream_t s) {
+    if (std::is_same<T, float>::value && launch_gemm_f32(probs, n_probs, s)) return;
     for (int base = 0; base < n_probs; base += kMaxProbs) {
         GemmBatch gb{};
         gb.n = std::min(kMaxProbs, n_probs - base);

@@ -79,6 +79,9 @@ struct GemmProblem {
 enum GemmLayout { kKK = 0, kKN = 1, kMN = 2 };
 template <typename T>
 void launch_gemm(const GemmProblem* probs, int n_probs, GemmLayout layout, cudaStream_t s);
+// The FP32 problems whose operands each have a unit stride (the same one in every problem
+// of the call); false, and nothing launched, for any other.
+bool launch_gemm_f32(const GemmProblem* probs, int n_probs, cudaStream_t s);
 
 // Valid 3x3 convolution (NCHW), implicit GEMM on CUDA cores.
 struct ConvShape {
