@@ -543,6 +543,8 @@ template <typename T>
 void launch_conv_fwd(const ConvShape& sh, const T* x, const T* w, const T* b, T* y, bool relu, cudaStream_t s) {
     const int M = sh.nimg * sh.OH * sh.OW;
     if (M == 0) return;
+    if constexpr (std::is_same<T, float>::value)
+        if (launch_conv_fwd_f32(sh, x, w, b, y, relu, s)) return;
     dim3 grid((M + CBM - 1) / CBM, (sh.Cout + CBN - 1) / CBN);
     launch_k(conv_fwd_kernel<T>, dim3(grid), dim3(NT), 0, s, sh, x, w, b, y, relu ? 1 : 0);
 }
@@ -550,6 +552,8 @@ template <typename T>
 void launch_conv_dgrad(const ConvShape& sh, const T* dy, const T* w, T* dx, const T* mask, cudaStream_t s) {
     const int M = sh.nimg * sh.H * sh.W;
     if (M == 0) return;
+    if constexpr (std::is_same<T, float>::value)
+        if (launch_conv_dgrad_f32(sh, dy, w, dx, mask, s)) return;
     dim3 grid((M + CBM - 1) / CBM, (sh.Cin + CBN - 1) / CBN);
     launch_k(conv_dgrad_kernel<T>, dim3(grid), dim3(NT), 0, s, sh, dy, w, dx, mask);
 }
@@ -562,10 +566,18 @@ void launch_conv_wgrad(const ConvShape& sh, const T* dy, const T* x, T* dw, T* d
     const int splits = wgrad_splits(sh);
     const int chunk = (P + splits - 1) / splits;
     const int N = sh.Cin * 9 + 1;
-    if (std::is_same<T, float>::value && sh.Cout == 32 && N <= 32)
-        launch_k(conv_wgrad_c32_kernel<false>, dim3(splits), dim3(128), 0, s, sh, (const void*)dy, (const float*)x,
-                 (float*)work, chunk);
-    else
+    bool done = false;
+    if constexpr (std::is_same<T, float>::value) {
+        // the encoder's first layer: 21 us here, 37 us in sq_conv_f32.cu (512 images, 3 x 32 x 32, stride 2)
+        if (sh.Cout == 32 && N <= 32) {
+            launch_k(conv_wgrad_c32_kernel<false>, dim3(splits), dim3(128), 0, s, sh, (const void*)dy, (const float*)x,
+                     (float*)work, chunk);
+            done = true;
+        } else {
+            done = launch_conv_wgrad_partials_f32(sh, dy, x, work, splits, chunk, s);
+        }
+    }
+    if (!done)
         launch_k(conv_wgrad_kernel<T>, dim3((N + WBN - 1) / WBN, (sh.Cout + WBM - 1) / WBM, splits), dim3(NT), 0, s,
                  sh, dy, x, work, chunk);
     const int tot = sh.Cout * N;

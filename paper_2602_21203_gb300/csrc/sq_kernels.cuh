@@ -105,6 +105,15 @@ template <typename T>
 void launch_conv_dgrad(const ConvShape& sh, const T* dy, const T* w, T* dx, const T* mask, cudaStream_t s);
 // dw, db from dy and x; workspace of conv_wgrad_workspace(sh) elements of T.
 int64_t conv_wgrad_workspace(const ConvShape& sh);
+// The FP32 forms (sq_conv_f32.cu); false, and nothing launched, for a shape whose tile of
+// pixels reads more than fits in shared memory.  The weight gradient writes the partial
+// sums of `splits` chunks of pixels, [splits][Cout][Cin * 9 + 1] (the last column the bias).
+bool launch_conv_fwd_f32(const ConvShape& sh, const float* x, const float* w, const float* b, float* y, bool relu,
+                         cudaStream_t s);
+bool launch_conv_dgrad_f32(const ConvShape& sh, const float* dy, const float* w, float* dx, const float* mask,
+                           cudaStream_t s);
+bool launch_conv_wgrad_partials_f32(const ConvShape& sh, const float* dy, const float* x, float* work, int splits,
+                                    int chunk, cudaStream_t s);
 template <typename T>
 void launch_conv_wgrad(const ConvShape& sh, const T* dy, const T* x, T* dw, T* db, T* work, cudaStream_t s);
 // The same for a 32-output layer with Cin * 9 + 1 <= 32 whose output gradient is the
