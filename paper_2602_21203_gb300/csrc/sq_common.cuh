@@ -200,6 +200,21 @@ __device__ __forceinline__ bool bulk_load_wait(uint64_t* bar, uint32_t parity) {
     }
 }
 
+// One lane of the (converged) calling warp, the same one at every call.  Issue loops branch on
+// the warp (made uniform by warp_uniform) and then on this predicate: descriptors and loop
+// counters then stay in uniform registers, where a branch on the thread index moves every
+// operand of every MMA there first.  One thread's chain of M = 128, K = 16 MMAs issued that way
+// takes 46 / 54 / 70 cycles an MMA at N = 32 / 64 / 128 (what their shared-memory operands
+// take); in a branch on the thread index 82 with descriptors advanced by addition, 213 when
+// each is formed anew.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+    return p != 0;
+}
+template <typename T>
+__device__ __forceinline__ T warp_uniform(T v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 template <typename T> __device__ __forceinline__ T ld(const T* p) { return *p; }
 
 __device__ __forceinline__ float to_f(float x) { return x; }

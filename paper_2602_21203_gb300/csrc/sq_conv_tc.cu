@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kConvThreads) conv32_tc_kernel(const __grid_co
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 10);
     const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + 2), tfull0 = smem_u32(bars + 4),
                    tempty0 = smem_u32(bars + 6), done_bar = smem_u32(bars + 8);
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_uniform((int)threadIdx.x / 32), lane = threadIdx.x % 32;
     const int n_local = (int)blockIdx.x < a.nimg ? (a.nimg - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     const uint32_t cols = 2 * (uint32_t)a.tmem_cols;
 
@@ -167,11 +167,11 @@ __global__ void __launch_bounds__(kConvThreads) conv32_tc_kernel(const __grid_co
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = warp_uniform(*tmem_slot);
     const uint32_t w_u = smem_u32(w_s);
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             // producer: the filter with the first image, then image i into buffer i % 2 once
             // the MMAs of image i - 2 have read it
             int issued = 0;
@@ -192,24 +192,24 @@ __global__ void __launch_bounds__(kConvThreads) conv32_tc_kernel(const __grid_co
                 mbar_wait(full0 + 8 * (i & 1), (i >> 1) & 1, a.err, 14);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = idesc_bf16(128, kCh, false, false);
             for (int i = 0; i < n_local; ++i) {
                 const int b = i & 1;
                 if (!mbar_wait(full0 + 8 * b, (i >> 1) & 1, a.err, 11)) break;
                 if (i >= 2 && !mbar_wait(tempty0 + 8 * b, ((i - 2) >> 1) & 1, a.err, 15)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t img_u = smem_u32(smem) + b * ibytes;
+                // descriptors of the first tap; starts move in 16-byte units within the 14-bit field
+                const uint64_t a0 = plain_desc(smem_u32(smem) + b * ibytes + a.off0 * 16, plane, 128);
+                const uint64_t b0 = plain_desc(w_u, 512, 128);
                 const uint32_t acc = tmem + b * (uint32_t)a.tmem_cols;
                 for (int t = 0; t < a.n_tiles; ++t)
-                    for (int tap = 0; tap < 9; ++tap) {
-                        const int row0 = t * 128 + a.off0 + (tap / 3) * a.Wp + (tap % 3);
-                        for (int kc = 0; kc < 2; ++kc) {
-                            const uint64_t ad = plain_desc(img_u + 2 * kc * plane + row0 * 16, plane, 128);
-                            const uint64_t bd = plain_desc(w_u + tap * 2048 + 2 * kc * 512, 512, 128);
-                            mma_bf16(acc + t * kCh, ad, bd, idesc, (tap | kc) ? 1u : 0u);
-                        }
-                    }
+#pragma unroll
+                    for (int tap = 0; tap < 9; ++tap)
+#pragma unroll
+                        for (int kc = 0; kc < 2; ++kc)
+                            mma_bf16(acc + t * kCh, a0 + (uint64_t)(kc * (plane / 8) + t * 128 + (tap / 3) * a.Wp + tap % 3),
+                                     b0 + (uint64_t)(tap * 128 + kc * 64), idesc, (tap | kc) ? 1u : 0u);
                 mma_commit(empty0 + 8 * b);
                 mma_commit(tfull0 + 8 * b);
             }
@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(128) wgrad32_tc_kernel(const __grid_constant__
     const uint32_t tma_bar[2] = {smem_u32(bars), smem_u32(bars + 1)};
     const uint32_t mma_bar[2] = {smem_u32(bars + 2), smem_u32(bars + 3)};
     const uint32_t done_bar = smem_u32(bars + 4);
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_uniform((int)threadIdx.x / 32), lane = threadIdx.x % 32;
     const int i0 = blockIdx.x * a.per_cta, i1 = min(a.nimg, i0 + a.per_cta);
 
     if (warp == 0) tmem_alloc(smem_u32(tmem_slot), 512);
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(128) wgrad32_tc_kernel(const __grid_constant__
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = warp_uniform(*tmem_slot);
     const int wpo = a.out_w + 4;
     const int64_t dy_img = (int64_t)(a.out_h + 4) * wpo * kCh;
     float bsum[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(128) wgrad32_tc_kernel(const __grid_constant__
     for (int i = i0; i < i1; ++i) {
         const int li = i - i0, b = li & 1;
         if (li >= 2 && !mbar_wait(mma_bar[b], ((li - 2) >> 1) & 1, a.err, 21)) ok = false;
-        if (threadIdx.x == 0 && ok) {
+        if (warp == 0 && elect_one() && ok) {
             const int boxes = a.slot_rows / a.box_rows;
             const int row0 = i * a.in_rows + 2 * a.Wp + 2;
             mbar_expect_tx(tma_bar[b], xbytes);
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(128) wgrad32_tc_kernel(const __grid_constant__
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
-        if (threadIdx.x == 32) {
+        if (warp == 1 && elect_one()) {
             if (!ok || !mbar_wait(tma_bar[b], (li >> 1) & 1, a.err, 22)) {
                 ok = false;
             } else {
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(128) wgrad32_tc_kernel(const __grid_constant__
         }
         __syncwarp();
     }
-    if (threadIdx.x == 32) mma_commit(done_bar);
+    if (warp == 1 && elect_one()) mma_commit(done_bar);
     __syncwarp();
     const bool have = mbar_wait(done_bar, 0, a.err, 23) && ok && i1 > i0;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -616,7 +616,7 @@ __global__ void __launch_bounds__(128, PL == 4 ? 5 : 2) conv0_tc_kernel(const __
     uint64_t* bars = reinterpret_cast<uint64_t*>(bias_s + kCh);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2);
     const uint32_t a_u = smem_u32(smem), b_u = smem_u32(b_s), bar0 = smem_u32(bars);
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_uniform((int)threadIdx.x / 32);
     const ConvShape& sh = a.sh;
     const int opix = sh.OH * sh.OW;
 
@@ -644,7 +644,7 @@ __global__ void __launch_bounds__(128, PL == 4 ? 5 : 2) conv0_tc_kernel(const __
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = warp_uniform(*tmem_slot);
     const int n_local = (int)blockIdx.x < a.n_tiles ? (a.n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     const int hw = sh.H * sh.W;
     bool ok = true;
@@ -726,12 +726,12 @@ __global__ void __launch_bounds__(128, PL == 4 ? 5 : 2) conv0_tc_kernel(const __
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (warp == 0 && elect_one()) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint64_t a0 = plain_desc(a_u + b * kTile, 2048, 128), b0 = plain_desc(b_u, 512, 128);
 #pragma unroll
             for (int kc = 0; kc < PL / 2; ++kc)
-                mma_bf16(tmem + (uint32_t)b * kCh, plain_desc(a_u + b * kTile + kc * 4096, 2048, 128),
-                         plain_desc(b_u + kc * 1024, 512, 128), idesc, kc > 0 ? 1u : 0u);
+                mma_bf16(tmem + (uint32_t)b * kCh, a0 + (uint64_t)(kc * 256), b0 + (uint64_t)(kc * 64), idesc, kc > 0 ? 1u : 0u);
             mma_commit(bar0 + 8 * b);
         }
         __syncwarp();
@@ -748,6 +748,261 @@ __global__ void __launch_bounds__(128, PL == 4 ? 5 : 2) conv0_tc_kernel(const __
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         tmem_dealloc(tmem, 64);
+    }
+}
+
+// ---------------------------------------------------------------- the whole encoder forward
+// Every layer of a 32-channel encoder (a first layer of at most 3 input channels and any
+// stride, then stride-1 layers) in one launch: an image's activations go from layer to layer
+// in shared memory, and only what is read later leaves it (the padded-HWC outputs of the first
+// n_save images, the features of all).
+//
+// A CTA runs kEncGroups images at a time, each by a group of four warps with its own two
+// activation buffers and tensor-memory columns: the group gathers the first layer's operand,
+// and per layer one of its threads issues the layer's MMAs, all wait for them, and each thread
+// takes its pixels out of tensor memory (bias, ReLU, BF16) into the other buffer.  The groups
+// share nothing but the filters, which stay in shared memory, so one group's MMAs run under
+// the others' epilogues.  Between the layers a plane holds its pixels densely, so an output
+// grid is as wide as its input (fewer 128-row tiles than the padded rows: the last layer of a
+// 32 x 32 input takes one instead of two).  The MMAs of an output and their order are those of
+// conv0_tc_kernel and conv32_tc_kernel: the same bits.
+//
+// Bound by the shared-memory path that the MMAs' operands (5 KB an M = 128, N = 32 MMA, 94 of
+// them an image at 32 x 32, 38 cycles each with four groups issuing) share with the gather and
+// the epilogues: without the inner MMAs 4,096 images of 3 x 32 x 32 take 51 us, with them 84;
+// 8 images 9.4 us, 1,024 with 512 saved 29 us.  The four launches it replaces: 207 us (act of
+// 4,096 rows), 59 us (the update's 1,024 images).  Three groups measured 107 us, four 99, six
+// (without the staged input) 93, before the issue loops became warp-uniform (103 -> 84).
+constexpr int kEncGroups = 4;      // at most
+constexpr int kEncMaxInner = 4;
+constexpr int kEncTiles = 4;
+// A layer's output grid: w columns computed (its input's width), of which ow and oh rows are
+// real; 128-pixel tiles; 2^20 / w rounded up, which divides pixel numbers below 512 by w.
+struct EncLayer { int w, oh, ow, tiles, inv; };
+struct EncArgs {
+    ConvShape sh;
+    const float* x;
+    const float* w0;
+    const float* bias[kEncMaxInner + 1];
+    const __nv_bfloat16* w[kEncMaxInner];     // layer l + 1, layout [tap][plane][out ch][8]
+    EncLayer l[kEncMaxInner + 1];
+    __nv_bfloat16* save[kEncMaxInner];        // padded-HWC output of layer l < n_inner (null: not kept)
+    float* z;                                 // optional features [nimg, 32 oh ow], FP32 and BF16
+    __nv_bfloat16* z_bf;
+    int nimg, n_save, n_inner, K, groups, group_cols, cols;   // cols: all groups', a power of two
+    uint32_t xbytes, ybytes, ibytes;   // of a group: the two activation buffers, an input image
+    int* err;
+};
+
+// Inputs k = 16 HALF .. + 15, k = (ci, ky, kx), of first-layer output pixels tg, tg + 128, ... of
+// the image at `in`, rounded to BF16, into planes of 8 k-values at `dst`.
+template <int HALF>
+__device__ __forceinline__ void gather_conv0(const EncArgs& a, const float* in, int tg, int hw, int opix, uint8_t* dst,
+                                             uint32_t plane) {
+    const ConvShape& sh = a.sh;
+    for (int p = tg; p < opix; p += 128) {   // the last tile's other rows read what is there and are dropped
+        const int oy = p * a.l[0].inv >> 20, ox = p - oy * sh.OW;
+        const float* src = in + (oy * sh.stride) * sh.W + ox * sh.stride;
+        float v[16];
+#pragma unroll
+        for (int kk = 0; kk < 16; ++kk) {
+            const int k = 16 * HALF + kk, ci = k / 9, tap = k % 9;
+            v[kk] = k < a.K ? src[ci * hw + (tap / 3) * sh.W + tap % 3] : 0.f;
+        }
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+            *reinterpret_cast<uint4*>(dst + (2 * HALF + c) * plane + p * 16) =
+                make_uint4(pack2_bf16(v[8 * c], v[8 * c + 1]), pack2_bf16(v[8 * c + 2], v[8 * c + 3]),
+                           pack2_bf16(v[8 * c + 4], v[8 * c + 5]), pack2_bf16(v[8 * c + 6], v[8 * c + 7]));
+    }
+}
+
+__global__ void __launch_bounds__(128 * kEncGroups, 1) encoder_tc_kernel(const __grid_constant__ EncArgs a) {
+    SQ_KERNEL_ENTRY();
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
+    const uint32_t group_bytes = a.xbytes + a.ybytes + a.ibytes;
+    uint8_t* w_s = smem + a.groups * group_bytes;          // inner filters (reads past a buffer's planes end here)
+    uint8_t* w0_s = w_s + a.n_inner * kWBytes;               // first filter: 4 planes of 32 rows x 16 B
+    float* bias_s = reinterpret_cast<float*>(w0_s + 2048);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(bias_s + (kEncMaxInner + 1) * kCh);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + a.groups * (kEncTiles + 1) + 1);
+    const int warp = warp_uniform((int)threadIdx.x / 32), g = warp / 4, quarter = warp % 4, tg = threadIdx.x % 128;
+    const uint32_t bar = smem_u32(bars + g * (kEncTiles + 1)), ibar = bar + 8 * kEncTiles,
+                   wbar = smem_u32(bars + a.groups * (kEncTiles + 1));
+    const ConvShape& sh = a.sh;
+    const int opix = sh.OH * sh.OW, hw = sh.H * sh.W;
+
+    if (warp == 0) tmem_alloc(smem_u32(tmem_slot), a.cols);
+    if (threadIdx.x == 0) {
+        for (int b = 0; b <= a.groups * (kEncTiles + 1); ++b) mbar_init(smem_u32(bars + b), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        mbar_expect_tx(wbar, a.n_inner * kWBytes);
+        for (int l = 0; l < a.n_inner; ++l) bulk_load(smem_u32(w_s) + l * kWBytes, a.w[l], kWBytes, wbar);
+    }
+    for (int e = threadIdx.x; e < 32 * 4; e += (int)blockDim.x) {
+        const int co = e / 4, c = e % 4;
+        __align__(16) __nv_bfloat16 hb[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int k = 8 * c + j;
+            hb[j] = __float2bfloat16_rn(k < a.K ? a.w0[(int64_t)co * a.K + k] : 0.f);
+        }
+        *reinterpret_cast<uint4*>(w0_s + c * 512 + co * 16) = *reinterpret_cast<const uint4*>(hb);
+    }
+    for (int e = threadIdx.x; e < (a.n_inner + 1) * kCh; e += (int)blockDim.x) bias_s[e] = a.bias[e / kCh][e % kCh];
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t acc = warp_uniform(*tmem_slot) + (uint32_t)(g * a.group_cols);
+    uint8_t* const bx = smem + g * group_bytes;
+    uint8_t* const by = bx + a.xbytes;
+    uint8_t* const bi = by + a.ybytes;
+    const uint32_t plane0 = (uint32_t)opix * 16;
+    constexpr uint32_t idesc = idesc_bf16(128, kCh, false, false);
+    bool ok = mbar_wait(wbar, 0, a.err, 41);
+    uint32_t phase = 0;   // bit t: parity of the barrier of tile t
+
+    // the group's shared-memory writes and tensor-memory reads before the next MMAs
+    auto group_sync = [&] {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        asm volatile("bar.sync %0, 128;" ::"r"(g + 1) : "memory");
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    };
+    // one thread's bulk copy of an image's input, and all threads' first-layer operand from it
+    auto fetch = [&](int img) {
+        mbar_expect_tx(ibar, a.ibytes);
+        bulk_load(smem_u32(bi), a.x + (int64_t)img * sh.x_img_stride, a.ibytes, ibar);
+    };
+    uint32_t iphase = 0;
+    auto gather = [&] {
+        if (!mbar_wait(ibar, iphase, a.err, 44)) ok = false;
+        iphase ^= 1;
+        gather_conv0<0>(a, reinterpret_cast<const float*>(bi), tg, hw, opix, bx, plane0);
+        gather_conv0<1>(a, reinterpret_cast<const float*>(bi), tg, hw, opix, bx, plane0);
+    };
+    // this thread's pixels of a layer's output, tile by tile as the MMAs complete: bias, ReLU,
+    // BF16, into `dst` (planes of oh ow pixels; unused for the last layer) and to global memory.
+    // A wait that gives up stops this thread's further issue only (the commits go on, so
+    // nobody waits for what was not issued).
+    auto drain = [&](int img, int layer, uint8_t* dst, bool last) {
+        const EncLayer& L = a.l[layer];
+        const float4* bias = reinterpret_cast<const float4*>(bias_s + layer * kCh);
+        for (int t = 0; t < L.tiles; ++t) {
+            if (!mbar_wait(bar + 8 * t, (phase >> t) & 1, a.err, 42)) ok = false;
+            phase ^= 1u << t;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int q = t * 128 + tg, y = q * L.inv >> 20, x = q - y * L.w;
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {   // 16 channels at a time
+                uint32_t r[16];
+                tmem_ld16(acc + ((uint32_t)(quarter * 32) << 16) + t * kCh + 16 * half, r);
+                if (y < L.oh && x < L.ow) {
+                    float v[16];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float4 b = bias[4 * half + j];
+                        v[4 * j] = fmaxf(__uint_as_float(r[4 * j]) + b.x, 0.f);
+                        v[4 * j + 1] = fmaxf(__uint_as_float(r[4 * j + 1]) + b.y, 0.f);
+                        v[4 * j + 2] = fmaxf(__uint_as_float(r[4 * j + 2]) + b.z, 0.f);
+                        v[4 * j + 3] = fmaxf(__uint_as_float(r[4 * j + 3]) + b.w, 0.f);
+                    }
+                    const int px = L.oh * L.ow, row = y * L.ow + x;
+                    if (!last) {
+                        uint4 h[2];
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            h[c] = make_uint4(pack2_bf16(v[8 * c], v[8 * c + 1]), pack2_bf16(v[8 * c + 2], v[8 * c + 3]),
+                                              pack2_bf16(v[8 * c + 4], v[8 * c + 5]), pack2_bf16(v[8 * c + 6], v[8 * c + 7]));
+                            *reinterpret_cast<uint4*>(dst + ((2 * half + c) * px + row) * 16) = h[c];
+                        }
+                        if (img < a.n_save && a.save[layer]) {
+                            uint4* out = reinterpret_cast<uint4*>(
+                                a.save[layer] + (((int64_t)img * (L.oh + 4) + y + 2) * (L.ow + 4) + x + 2) * kCh + 16 * half);
+                            out[0] = h[0];
+                            out[1] = h[1];
+                        }
+                    } else {
+                        const int64_t base = ((int64_t)img * kCh + 16 * half) * px + row;
+                        if (a.z) {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) a.z[base + j * px] = v[j];
+                        }
+                        if (a.z_bf) {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) a.z_bf[base + j * px] = __float2bfloat16_rn(v[j]);
+                        }
+                    }
+            }
+            }
+            __syncwarp();
+        }
+    };
+
+    // images in turn over the CTAs, then over a CTA's groups
+    const int step = (int)gridDim.x * a.groups;
+    int img = (int)blockIdx.x + (int)gridDim.x * g;
+    if (img < a.nimg) {
+        if (quarter == 0 && elect_one()) fetch(img);
+        __syncwarp();
+        gather();
+    }
+    for (; img < a.nimg; img += step) {
+        group_sync();   // (the input image has been read)
+        if (quarter == 0 && elect_one()) {
+            if (img + step < a.nimg) fetch(img + step);
+            const uint64_t a0 = plain_desc(smem_u32(bx), plane0, 128), b0 = plain_desc(smem_u32(w0_s), 512, 128);
+            for (int t = 0; t < a.l[0].tiles; ++t) {
+                if (ok)
+#pragma unroll
+                    for (int kc = 0; kc < 2; ++kc)
+                        mma_bf16(acc + t * kCh, a0 + (uint64_t)(2 * kc * (plane0 / 16) + t * 128), b0 + (uint64_t)(kc * 64),
+                                 idesc, kc);
+                mma_commit(bar + 8 * t);
+            }
+        }
+        __syncwarp();
+        drain(img, 0, by, false);
+        for (int l = 1; l <= a.n_inner; ++l) {
+            const EncLayer& L = a.l[l];
+            const uint32_t plane = (uint32_t)(a.l[l - 1].oh * L.w) * 16;
+            const bool last = l == a.n_inner;
+            group_sync();
+            if (quarter == 0 && elect_one()) {
+                // descriptors of the first tap; starts move in 16-byte units within the 14-bit field
+                const uint64_t a0 = plain_desc(smem_u32(l % 2 ? by : bx), plane, 128);
+                const uint64_t b0 = plain_desc(smem_u32(w_s) + (l - 1) * kWBytes, 512, 128);
+                for (int t = 0; t < L.tiles; ++t) {
+                    if (ok)
+#pragma unroll
+                        for (int tap = 0; tap < 9; ++tap)
+#pragma unroll
+                            for (int kc = 0; kc < 2; ++kc)
+                                mma_bf16(acc + t * kCh,
+                                         a0 + (uint64_t)(2 * kc * (plane / 16) + t * 128 + (tap / 3) * L.w + tap % 3),
+                                         b0 + (uint64_t)(tap * 128 + kc * 64), idesc, (tap | kc) ? 1u : 0u);
+                    mma_commit(bar + 8 * t);
+                }
+            }
+            __syncwarp();
+            // the next image's operand while the last layer multiplies, where that reads the other buffer
+            if (last && l % 2 == 1 && img + step < a.nimg) gather();
+            drain(img, l, l % 2 ? bx : by, last);
+            if (last && l % 2 == 0 && img + step < a.nimg) gather();
+        }
+    }
+    if (quarter == 0 && elect_one()) {   // every MMA this group issued has completed before the tensor memory is freed
+        mma_commit(bar);
+        mbar_wait(bar, phase & 1, a.err, 43);
+    }
+    __syncwarp();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        tmem_dealloc(*tmem_slot, a.cols);
     }
 }
 
@@ -827,6 +1082,7 @@ bool plane_map(CUtensorMap* m, const __nv_bfloat16* base, int64_t rows, int box_
 int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
 size_t conv_smem(int load_rows) { return 1024 + 2 * 4 * (size_t)load_rows * 16 + kWBytes + 10 * 8 + 16; }
+constexpr int kEncSmem = 227 * 1024;
 constexpr int kConvCtasPerSm = 2;   // resident CTAs per SM of the persistent convolution
 int g_num_sms = 152;                 // set by conv_tc_prepare
 size_t wgrad_smem(int slot_rows, int kq) {
@@ -907,6 +1163,7 @@ void conv_tc_prepare() {
         g_num_sms = sms;
     cudaFuncSetAttribute(conv32_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(wgrad32_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+    cudaFuncSetAttribute(encoder_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncSmem);
     cudaFuncSetAttribute(conv0_tc_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
     cudaFuncSetAttribute(conv0_tc_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
     cudaFuncSetAttribute(conv0_tc_kernel<18>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
@@ -956,6 +1213,67 @@ int launch_conv0_tc(const ConvShape& sh, const float* x, const float* w, const f
     if (K <= 32) conv0_tc_go<4>(a, s);
     else if (K <= 64) conv0_tc_go<8>(a, s);
     else conv0_tc_go<18>(a, s);
+    return 0;
+}
+
+namespace {
+// The kernel's arguments and shared memory; false outside its range.
+bool encoder_plan(const EncoderTc& c, EncArgs& a, size_t& smem) {
+    const ConvShape& sh = c.sh;
+    const int K = sh.Cin * 9;
+    if (sh.Cout != kCh || K > 32 || c.n_inner < 1 || c.n_inner > kEncMaxInner || sh.nimg < 0) return false;
+    std::memset(&a, 0, sizeof(a));
+    a.sh = sh; a.x = c.x; a.w0 = c.w0; a.nimg = sh.nimg; a.n_save = c.n_save; a.n_inner = c.n_inner; a.K = K;
+    a.z = c.z; a.z_bf = c.z_bf;
+    auto layer = [](int w, int oh, int ow) { return EncLayer{w, oh, ow, (oh * w + 127) / 128, ((1 << 20) + w - 1) / w}; };
+    a.l[0] = layer(sh.OW, sh.OH, sh.OW);
+    a.xbytes = a.ybytes = (uint32_t)(sh.OH * sh.OW) * 64;
+    a.ibytes = (uint32_t)(sh.Cin * sh.H * sh.W) * 4;
+    if (sh.x_img_stride * 4 != (int64_t)a.ibytes || a.ibytes % 16 || (reinterpret_cast<uintptr_t>(c.x) & 15)) return false;
+    a.bias[0] = c.bias[0];
+    for (int l = 1; l <= c.n_inner; ++l) {
+        const EncLayer& p = a.l[l - 1];
+        if (p.oh < 3 || p.ow < 3 || (reinterpret_cast<uintptr_t>(c.w[l - 1]) & 15) || (reinterpret_cast<uintptr_t>(c.save[l - 1]) & 15))
+            return false;
+        a.l[l] = layer(p.ow, p.oh - 2, p.ow - 2);
+        if (a.l[l].oh * (p.ow + 4) > 512) return false;   // a layer launch_conv32_tc refuses
+        // layer l writes X for odd l, Y for even l; the last one leaves shared memory
+        uint32_t& buf = l % 2 ? a.xbytes : a.ybytes;
+        if (l < c.n_inner) buf = std::max(buf, (uint32_t)(a.l[l].oh * a.l[l].ow) * 64);
+        a.w[l - 1] = c.w[l - 1]; a.bias[l] = c.bias[l]; a.save[l - 1] = c.save[l - 1];
+    }
+    const int tiles = a.l[0].tiles;   // the most of any layer
+    // an MMA reads whole 128-row tiles at every tap: past the last plane it must end inside the filters
+    if (tiles > kEncTiles || (tiles * 128 + 2 * sh.OW + 2) * 16 > kWBytes) return false;
+    a.group_cols = kCh * tiles;
+    const size_t fixed = 128 + (size_t)c.n_inner * kWBytes + 2048 + (kEncMaxInner + 1) * kCh * 4 + 8 + 16;
+    const size_t group = a.xbytes + a.ybytes + a.ibytes + (kEncTiles + 1) * 8;
+    if (fixed + group > kEncSmem) return false;
+    a.groups = (int)std::min<size_t>(kEncGroups, (kEncSmem - fixed) / group);
+    a.groups = std::min(a.groups, 512 / a.group_cols);
+    // no more groups than the rounds of images need
+    const int rounds = (sh.nimg + g_num_sms * a.groups - 1) / (g_num_sms * a.groups);
+    while (a.groups > 1 && (sh.nimg + g_num_sms * (a.groups - 1) - 1) / (g_num_sms * (a.groups - 1)) == rounds) --a.groups;
+    a.cols = 32;   // a power of two from 32 to 512
+    while (a.cols < a.groups * a.group_cols) a.cols *= 2;
+    smem = fixed + a.groups * group;
+    return true;
+}
+}  // namespace
+
+bool encoder_tc_fits(const EncoderTc& c) {
+    EncArgs a;
+    size_t smem;
+    return encoder_plan(c, a, smem);
+}
+
+int launch_encoder_tc(const EncoderTc& c, int* err, cudaStream_t s) {
+    EncArgs a;
+    size_t smem;
+    if (!encoder_plan(c, a, smem)) return -1;
+    if (c.sh.nimg == 0) return 0;
+    a.err = err;
+    launch_k(encoder_tc_kernel, dim3(std::min(c.sh.nimg, g_num_sms)), dim3(128 * a.groups), smem, s, a);
     return 0;
 }
 

@@ -1070,6 +1070,27 @@ void squint_handle::record_update(int j, int k, cudaStream_t s, bool debug) {
         const ConvL& c0 = L.conv[0];
         const int64_t img0 = (int64_t)c.obs_c * c0.h * c0.w;
         ConvShape sh{n, c0.cin, c0.h, c0.w, c0.cout, c0.s, c0.oh, c0.ow, img0, (int64_t)c0.cout * c0.oh * c0.ow};
+        if (upto == nconv - 1) {
+            // the whole forward in one launch, keeping what the backward reads: the o_t images'
+            // activations (none when they are recomputed there)
+            EncoderTc e{};
+            e.sh = sh; e.x = x2 + (int64_t)i0 * img0; e.w0 = W + c0.wo; e.n_inner = nconv - 1;
+            double flops = 0.0;
+            for (int l = 0; l < nconv; ++l) {
+                e.bias[l] = W + L.conv[l].bo;
+                if (l > 0) e.w[l - 1] = wconv_fwd[l];
+                if (l < nconv - 1) e.save[l] = act_p[l];
+                flops += conv_flops(L.conv[l], n);
+            }
+            e.n_save = rc_chunk ? 0 : B;
+            e.z = conv_out[nconv - 1] + (int64_t)i0 * F;
+            e.z_bf = z_h + (int64_t)i0 * F;
+            if (encoder_tc_fits(e)) {
+                ProfScope ps(this, st, "conv_tc_fwd", flops, 0);
+                if (launch_encoder_tc(e, d_err, st) != 0) launch_failed = true;
+                return;
+            }
+        }
         {
             // first layer on tensor cores (CUDA cores outside that kernel's range), written
             // straight into the padded-HWC input of layer 1

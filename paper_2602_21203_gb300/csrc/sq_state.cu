@@ -280,7 +280,23 @@ int squint_handle::act(sq::ActArena& a, const squint_act_request* reqs, int n_re
     // is independent of the other rows of the batch)
     const bool tc = bf16 && tc_conv;
     const float* in = ax;
-    for (size_t l = 0; l < L.conv.size(); ++l) {
+    bool encoded = false;
+    if (tc) {   // the whole encoder in one launch; FP32 features only where the heads read them
+        const ConvL& c0 = L.conv[0];
+        EncoderTc e{};
+        e.sh = ConvShape{rows, c0.cin, c0.h, c0.w, c0.cout, c0.s, c0.oh, c0.ow, (int64_t)c0.cin * c0.h * c0.w,
+                         (int64_t)c0.cout * c0.oh * c0.ow};
+        e.x = ax; e.w0 = Wp + c0.wo; e.n_inner = (int)L.conv.size() - 1;
+        for (size_t l = 0; l < L.conv.size(); ++l) {
+            e.bias[l] = Wp + L.conv[l].bo;
+            if (l > 0) e.w[l - 1] = policy_wconv[pi] + (l - 1) * 9 * 32 * 32;
+        }
+        e.z = Dd > 0 ? nullptr : aconv.back();
+        e.z_bf = az_h;
+        encoded = launch_encoder_tc(e, d_err, s) == 0;
+        if (encoded) in = aconv.back();
+    }
+    for (size_t l = 0; l < L.conv.size() && !encoded; ++l) {
         const ConvL& cv = L.conv[l];
         if (tc && l > 0) {
             ConvTc ct{};

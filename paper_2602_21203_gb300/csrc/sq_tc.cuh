@@ -2,6 +2,7 @@
 #pragma once
 
 #include "sq_common.cuh"
+#include "sq_kernels.cuh"
 
 namespace sq {
 
@@ -108,6 +109,26 @@ struct ConvTc {
     __nv_bfloat16* out_chw_bf;
 };
 int launch_conv32_tc(const ConvTc& c, int* err, cudaStream_t s);
+// A whole 32-channel encoder forward in one launch: the first layer (sh: Cin <= 3, any stride,
+// NCHW FP32 input, FP32 filter w0), then n_inner stride-1 layers (filters in the forward layout,
+// biases bias[0 .. n_inner]), ReLU after each.  save[l] (layer l < n_inner, null: not kept)
+// receives the padded-HWC outputs of images [0, n_save); z and z_bf (either may be null) the
+// last layer's outputs of all images as CHW rows.  The results are those of launch_conv0_tc and
+// launch_conv32_tc bit for bit.  0, or < 0, and nothing launched, for a shape outside its range.
+struct EncoderTc {
+    ConvShape sh;
+    const float* x;
+    const float* w0;
+    int n_inner;
+    const __nv_bfloat16* w[8];
+    const float* bias[8];
+    __nv_bfloat16* save[8];
+    int n_save;
+    float* z;
+    __nv_bfloat16* z_bf;
+};
+int launch_encoder_tc(const EncoderTc& c, int* err, cudaStream_t s);
+bool encoder_tc_fits(const EncoderTc& c);
 // Weight gradient: x = padded layer input (Wp = W+4), dy = padded gradient at the
 // layer's pre-activation (out_h x out_w); dw [32, 32, 3, 3] and db [32] written.
 struct WgradTc {
