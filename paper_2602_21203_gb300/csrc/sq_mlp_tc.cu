@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
     const int rank = CL > 1 ? (int)cluster_rank() : 0;
     const int m0 = ((int)blockIdx.x - P.cta0) / CL * BM;
     const int M = P.M;
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_uniform((int)threadIdx.x / 32), lane = threadIdx.x % 32;
     const long long wlim = a.wait_limit;
     int* err = a.err;
     const int hslabs = (H + SLAB - 1) / SLAB;
@@ -320,14 +320,15 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = slot[0];
+    const uint32_t tmem = warp_uniform(slot[0]);
 
     if (warp == 4) {
         // ---------------------------------------------------------------- TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             mbar_expect_tx(x_full, (uint32_t)(P.nk0 * SLAB_BYTES));
             for (int kb = 0; kb < P.nk0; ++kb) tma_load_2d(a_base + kb * SLAB_BYTES, &P.tx, kb * SLAB, m0, x_full);
-            int it = 0;
+            int it = 0, s = 0;
+            uint32_t ph = 1;   // parity of the stage's previous release (none in the first round)
             bool ok = true;
             for (int l = 0; l <= nh && ok; ++l) {
                 const bool last = l == nh;
@@ -335,10 +336,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
                 const int row0 = last ? 0 : rank * NS;
                 const int kcol0 = (last && CL > 1) ? rank * NS : 0;
                 for (int kb = 0; kb < nk(l); ++kb, ++it) {
-                    const int s = it % S;
-                    if (it >= S && !mbar_wait(empty(s), ((it / S) - 1) & 1, err, 30, wlim)) { ok = false; break; }
+                    if (it >= S && !mbar_wait(empty(s), ph, err, 30, wlim)) { ok = false; break; }
                     mbar_expect_tx(full(s), bytes);
                     tma_load_2d(ring + s * a.stage_bytes, &P.tw[l], kcol0 + kb * SLAB, row0, full(s));
+                    if (++s == S) { s = 0; ph ^= 1; }
                 }
             }
             slot[1] = it;
@@ -362,12 +363,13 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
         float* const p_out = P.out;
         const int64_t p_ldo = P.ldo;
         float* stg_w = stg + warp * 32 * STG_LD;
-        int it = 0;                                      // weight slab sequence (issuer)
+        int it0 = 0;                                     // weight slabs of the layers before
         bool dead = false;                               // the issuer gave up on a wait
         for (int l = 0; l <= nh; ++l) {
             const bool last = l == nh;
             // ---------------------------------------------------------------- MMA issue
-            if (threadIdx.x == 0) {
+            if (warp == 0 && elect_one()) {
+                const bool gave_up = dead;
                 if (!dead) {
                     if (l == 0) dead = !mbar_wait(x_full, 0, err, 31, wlim);
                     else dead = !mbar_wait<true>(a_ready, (l - 1) & 1, err, 32, wlim);
@@ -375,21 +377,23 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t idesc = idesc_bf16_kk(BM, last ? nop : NS);
                 const int nkl = nk(l);
-                for (int kb = 0; kb < nkl && !dead; ++kb) {
-                    const int s = it % S;
-                    if (!mbar_wait(full(s), (it / S) & 1, err, 33, wlim)) { dead = true; break; }
+                int kb = 0, s = it0 % S;
+                uint32_t ph = (uint32_t)(it0 / S) & 1;
+                for (; kb < nkl && !dead; ++kb) {
+                    if (!mbar_wait(full(s), ph, err, 33, wlim)) { dead = true; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t as = a_base + kb * SLAB_BYTES, bs = ring + s * a.stage_bytes;
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk)
                         mma_bf16(tmem, sw128_desc(as + kk * 32), sw128_desc(bs + kk * 32), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
                     mma_commit(empty(s));
-                    ++it;
+                    if (++s == S) { s = 0; ph ^= 1; }
                 }
-                slot[2] = it;
+                if (!gave_up) slot[2] = it0 + kb;
                 mma_commit(acc_full);
             }
             __syncwarp();
+            it0 += nk(l);
             mbar_wait(acc_full, l & 1, err, 34, wlim);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (l == 0) epi_bar();   // the staged parameter slices
@@ -742,7 +746,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
     const int m0 = ((int)blockIdx.x - P.cta0) / CL * BM;
     const int rb = m0 / BM;
     const int M = P.M;
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_uniform((int)threadIdx.x / 32), lane = threadIdx.x % 32;
     const long long wlim = a.wait_limit;
     int* err = a.err;
     const int hslabs = (H + SLAB - 1) / SLAB;
@@ -786,14 +790,15 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = slot[0];
+    const uint32_t tmem = warp_uniform(slot[0]);
 
     if (warp == 4) {
         // ---------------------------------------------------------------- TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             mbar_expect_tx(a0_full, (uint32_t)(a.nko * SLAB_BYTES));
             for (int kb = 0; kb < a.nko; ++kb) tma_load_2d(a_base + kb * SLAB_BYTES, &P.tdo, kb * SLAB, m0, a0_full);
-            int it = 0;
+            int it = 0, s = 0;
+            uint32_t ph = 1;   // parity of the stage's previous release (none in the first round)
             bool ok = true;
             for (int st = 0; st < nsteps && ok; ++st) {
                 const bool fin = st == nh;
@@ -802,11 +807,11 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
                 const int n0 = fin ? (ksplit ? a.c0 : a.c0 + rank * nfin) : rank * NS;
                 const int k0 = (fin && ksplit) ? rank * NS : 0;
                 for (int kb = 0; kb < nk(st); ++kb, ++it) {
-                    const int s = it % S;
-                    if (it >= S && !mbar_wait(empty(s), ((it / S) - 1) & 1, err, 40, wlim)) { ok = false; break; }
+                    if (it >= S && !mbar_wait(empty(s), ph, err, 40, wlim)) { ok = false; break; }
                     mbar_expect_tx(full(s), (uint32_t)(N * 128));
                     for (int j = 0; j < N / 64; ++j)
                         tma_load_2d(ring + s * a.stage_bytes + j * 8192, &P.tw[wl], n0 + 64 * j, k0 + kb * SLAB, full(s));
+                    if (++s == S) { s = 0; ph ^= 1; }
                 }
             }
             slot[1] = it;
@@ -823,7 +828,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
             }
         float* const p_dx = P.dx;
         const int64_t p_lddx = P.lddx;
-        int it = 0;
+        int it0 = 0;                                     // weight slabs of the steps before
         bool dead = false;
         for (int st = 0; st < nsteps; ++st) {
             const bool fin = st == nh;
@@ -840,16 +845,18 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
                 }
             }
             // ---------------------------------------------------------------- MMA issue
-            if (threadIdx.x == 0) {
+            if (warp == 0 && elect_one()) {
+                const bool gave_up = dead;
                 if (!dead) {
                     if (st == 0) dead = !mbar_wait(a0_full, 0, err, 41, wlim);
                     else dead = !mbar_wait<true>(a_ready, (st - 1) & 1, err, 42, wlim);
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t idesc = idesc_bf16_kn(BM, fin ? nfin : NS);
-                for (int kb = 0; kb < nk(st) && !dead; ++kb) {
-                    const int s = it % S;
-                    if (!mbar_wait(full(s), (it / S) & 1, err, 43, wlim)) { dead = true; break; }
+                int kb = 0, s = it0 % S;
+                uint32_t ph = (uint32_t)(it0 / S) & 1;
+                for (; kb < nk(st) && !dead; ++kb) {
+                    if (!mbar_wait(full(s), ph, err, 43, wlim)) { dead = true; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t as = a_base + kb * SLAB_BYTES, bs = ring + s * a.stage_bytes;
 #pragma unroll
@@ -857,12 +864,13 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
                         mma_bf16(tmem, sw128_desc(as + kk * 32), sw128_desc_mn(bs + kk * 2048), idesc,
                                  (kb > 0 || kk > 0) ? 1u : 0u);
                     mma_commit(empty(s));
-                    ++it;
+                    if (++s == S) { s = 0; ph ^= 1; }
                 }
-                slot[2] = it;
+                if (!gave_up) slot[2] = it0 + kb;
                 mma_commit(acc_full);
             }
             __syncwarp();
+            it0 += nk(st);
             mbar_wait(acc_full, st & 1, err, 44, wlim);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (st == 0) epi_bar();   // the staged g slices

@@ -281,16 +281,15 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
     const int crank = (int)cluster_rank();
     const int t = cta / gb.splits, split = gb.ln ? 0 : crank;   // K split rank (0 in LayerNorm mode)
     const int m0 = (t / tiles_n) * BM, n0 = (t % tiles_n) * BN;
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_uniform((int)threadIdx.x / 32), lane = threadIdx.x % 32;
     const uint32_t base = smem_u32(smem);
     const int nkb = (pK + BKE - 1) / BKE;
     // this CTA's share of the (pair, K slab) iterations
     const int it0 = (int)((int64_t)nkb * n_pairs * split / gb.splits);
     const int total = (int)((int64_t)nkb * n_pairs * (split + 1) / gb.splits) - it0;
-    const bool producer = warp == 1 && lane == 0, issuer = warp == 0 && lane == 0;
+    const bool producer = warp == 1 && elect_one(), issuer = warp == 0 && elect_one();
     const long long wlim = gb.wait_limit;
-    auto load_stage = [&](int i) {
-        const int s = i % STAGES;
+    auto load_stage = [&](int i, int s) {   // slab i of this CTA into stage s = i mod STAGES
         const int pr = (it0 + i) / nkb, kb = (it0 + i) % nkb;
         const uint32_t st = base + s * STAGE_BYTES;
         mbar_expect_tx(full0 + 8 * s, STAGE_BYTES + (MX ? 2 * SF_ATOM : 0));
@@ -323,7 +322,7 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
     SQ_KERNEL_ENTRY();
     const int pre = gb.stall ? 0 : (total < STAGES ? total : STAGES);
     if (producer)
-        for (int i = 0; i < pre; ++i) load_stage(i);   // first stages: no slot to wait for
+        for (int i = 0; i < pre; ++i) load_stage(i, i);   // first stages: no slot to wait for
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(TMEM_COLS));
@@ -332,7 +331,7 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = warp_uniform(*tmem_slot);
     // the bias is first read in the epilogue, after the cluster barrier
     if (warp >= 2) {
         for (int j = threadIdx.x - 64; j < BN; j += 64) bias_s[j] = (p_bias && n0 + j < pN) ? p_bias[n0 + j] : 0.f;
@@ -345,21 +344,22 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
 
     if (producer) {
         int issued = pre;
-        for (int i = pre; i < total && !gb.stall; ++i) {
-            const int s = i % STAGES;
-            if (!mbar_wait(empty0 + 8 * s, ((i / STAGES) - 1) & 1, gb.err, 1, wlim)) break;
-            load_stage(i);
+        uint32_t ph = 0;
+        for (int i = pre, s = 0; i < total && !gb.stall; ++i) {   // (pre = STAGES if the loop runs at all)
+            if (!mbar_wait(empty0 + 8 * s, ph, gb.err, 1, wlim)) break;
+            load_stage(i, s);
             issued = i + 1;
+            if (++s == STAGES) { s = 0; ph ^= 1; }
         }
         tmem_slot[1] = issued;
     } else if (issuer) {
         // MMA issuer
         constexpr uint32_t idesc = F8 ? idesc_e4m3(BM, BN, A_MN, B_MN) : idesc_bf16(BM, BN, A_MN, B_MN);
         if constexpr (MX) {
-            int i = 0;
+            int i = 0, s = 0;
+            uint32_t ph = 0;
             for (; i < total; ++i) {
-                const int s = i % STAGES;
-                if (!mbar_wait(full0 + 8 * s, (i / STAGES) & 1, gb.err, 2, wlim)) break;
+                if (!mbar_wait(full0 + 8 * s, ph, gb.err, 2, wlim)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t st = base + s * STAGE_BYTES;
                 const uint32_t sf = base + SF_OFF + s * 2 * SF_ATOM;
@@ -372,14 +372,15 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
                     mma_mx(tmem, operand_desc<false>(st, kk), operand_desc<false>(st + TILE_BYTES, kk),
                            idesc_mx(BM, BN, (uint32_t)kk), sfa_t, sfb_t, (i > 0 || kk > 0) ? 1u : 0u);
                 mma_commit(empty0 + 8 * s);
+                if (++s == STAGES) { s = 0; ph ^= 1; }
             }
             tmem_slot[2] = i;
             mma_commit(done_bar);
         } else {
-            int i = 0;
+            int i = 0, s = 0;
+            uint32_t ph = 0;
             for (; i < total; ++i) {
-                const int s = i % STAGES;
-                if (!mbar_wait(full0 + 8 * s, (i / STAGES) & 1, gb.err, 2, wlim)) break;
+                if (!mbar_wait(full0 + 8 * s, ph, gb.err, 2, wlim)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t st = base + s * STAGE_BYTES;
 #pragma unroll
@@ -391,6 +392,7 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
                         mma_bf16(tmem, operand_desc<A_MN>(st, kk), operand_desc<B_MN>(st + TILE_BYTES, kk), idesc,
                                  (i > 0 || kk > 0) ? 1u : 0u);
                 mma_commit(empty0 + 8 * s);
+                if (++s == STAGES) { s = 0; ph ^= 1; }
             }
             tmem_slot[2] = i;
             mma_commit(done_bar);
