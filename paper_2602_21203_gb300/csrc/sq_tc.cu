@@ -234,6 +234,101 @@ __device__ __forceinline__ void load_operand(uint32_t dst, const CUtensorMap* ma
     }
 }
 
+// Where a tile's values go: zeroed where mask <= 0, then stored or added as FP32 and stored as BF16.
+struct TcOut {
+    const float* mask; int64_t ldmask;
+    float* c; int64_t ldc;
+    __nv_bfloat16* cbf; int64_t ldcbf;
+    bool accumulate;
+};
+// Entry i < rows_ok of acc is the nv (<= 4) values from column col on of row row0 + 4 i; each
+// output runs as its own loop, so that a lane's loads are in flight together.
+__device__ __forceinline__ void finish_rows(float4 (&acc)[8], int rows_ok, int row0, int col, int nv, const TcOut& o) {
+    const bool cvec = nv == 4 && (o.ldc & 3) == 0 && ((reinterpret_cast<uintptr_t>(o.c) & 15) == 0);
+    const bool hvec = nv == 4 && (o.ldcbf & 3) == 0 && ((reinterpret_cast<uintptr_t>(o.cbf) & 7) == 0);
+    const bool mvec = nv == 4 && (o.ldmask & 3) == 0 && ((reinterpret_cast<uintptr_t>(o.mask) & 15) == 0);
+    if (o.mask) {
+        if (mvec) {
+            float4 mk[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (i < rows_ok) mk[i] = *reinterpret_cast<const float4*>(o.mask + (int64_t)(row0 + 4 * i) * o.ldmask + col);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (i < rows_ok) {
+                    if (!(mk[i].x > 0.f)) acc[i].x = 0.f;
+                    if (!(mk[i].y > 0.f)) acc[i].y = 0.f;
+                    if (!(mk[i].z > 0.f)) acc[i].z = 0.f;
+                    if (!(mk[i].w > 0.f)) acc[i].w = 0.f;
+                }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (i < rows_ok) {
+                    const float* mk = o.mask + (int64_t)(row0 + 4 * i) * o.ldmask + col;
+                    if (!(mk[0] > 0.f)) acc[i].x = 0.f;
+                    if (nv > 1 && !(mk[1] > 0.f)) acc[i].y = 0.f;
+                    if (nv > 2 && !(mk[2] > 0.f)) acc[i].z = 0.f;
+                    if (nv > 3 && !(mk[3] > 0.f)) acc[i].w = 0.f;
+                }
+        }
+    }
+    if (o.c) {
+        if (cvec) {
+            if (o.accumulate) {
+                float4 old[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (i < rows_ok) old[i] = *reinterpret_cast<const float4*>(o.c + (int64_t)(row0 + 4 * i) * o.ldc + col);
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (i < rows_ok) {
+                        acc[i].x += old[i].x; acc[i].y += old[i].y; acc[i].z += old[i].z; acc[i].w += old[i].w;
+                    }
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (i < rows_ok) *reinterpret_cast<float4*>(o.c + (int64_t)(row0 + 4 * i) * o.ldc + col) = acc[i];
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (i < rows_ok) {
+                    float* dst = o.c + (int64_t)(row0 + 4 * i) * o.ldc + col;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float v = j == 0 ? acc[i].x : j == 1 ? acc[i].y : j == 2 ? acc[i].z : acc[i].w;
+                        if (j < nv) dst[j] = o.accumulate ? dst[j] + v : v;
+                    }
+                }
+        }
+    }
+    if (o.cbf) {
+        if (hvec) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (i < rows_ok) {
+                    __nv_bfloat162 lo = __floats2bfloat162_rn(acc[i].x, acc[i].y);
+                    __nv_bfloat162 hi = __floats2bfloat162_rn(acc[i].z, acc[i].w);
+                    uint2 u;
+                    u.x = *reinterpret_cast<uint32_t*>(&lo);
+                    u.y = *reinterpret_cast<uint32_t*>(&hi);
+                    *reinterpret_cast<uint2*>(o.cbf + (int64_t)(row0 + 4 * i) * o.ldcbf + col) = u;
+                }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (i < rows_ok) {
+                    __nv_bfloat16* dst = o.cbf + (int64_t)(row0 + 4 * i) * o.ldcbf + col;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float v = j == 0 ? acc[i].x : j == 1 ? acc[i].y : j == 2 ? acc[i].z : acc[i].w;
+                        if (j < nv) dst[j] = __float2bfloat16_rn(v);
+                    }
+                }
+        }
+    }
+}
+
 // F8 = 1: e4m3 operands, 128-element (128-byte) K slabs, kind::f8f6f4 MMAs with K = 32,
 // and the per-tensor scales applied in the epilogue.  The K step of a slab is 32 bytes in
 // both types, so the shared-memory descriptors are the same.  F8 = 2 (MX-FP8): the same
@@ -268,13 +363,7 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
     // through a generic pointer, which the compiler would otherwise re-read after every store
     const int pM = P.M, pN = P.N, pK = P.K, n_pairs = P.n_pairs, tiles_n = P.tiles_n;
     const float* const p_bias = P.bias;
-    float* const p_c = P.c;
-    const int64_t p_ldc = P.ldc;
-    __nv_bfloat16* const p_cbf = P.cbf;
-    const int64_t p_ldcbf = P.ldcbf;
-    const float* const p_mask = P.mask;
-    const int64_t p_ldmask = P.ldmask;
-    const bool p_acc = P.accumulate != 0;
+    const TcOut out{P.mask, P.ldmask, P.c, P.ldc, P.cbf, P.ldcbf, P.accumulate != 0};
     const float* const p_sa = P.scale_a;
     const float* const p_sb = P.scale_b;
     const int cta = blockIdx.x - P.tile_start;
@@ -490,9 +579,6 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
         const int col = n0 + cq;
         const int nv = col < pN ? min(4, pN - col) : 0;   // valid columns of this lane
         const int nrows = rb1 - rb0 > warp ? (rb1 - rb0 - warp + 3) / 4 : 0;
-        const bool cvec = nv == 4 && (p_ldc & 3) == 0 && ((reinterpret_cast<uintptr_t>(p_c) & 15) == 0);
-        const bool hvec = nv == 4 && (p_ldcbf & 3) == 0 && ((reinterpret_cast<uintptr_t>(p_cbf) & 7) == 0);
-        const bool mvec = nv == 4 && (p_ldmask & 3) == 0 && ((reinterpret_cast<uintptr_t>(p_mask) & 15) == 0);
         float bias4[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) bias4[j] = bias_s[cq + j];
@@ -546,86 +632,7 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
             }
             const int row0 = m0 + rb0 + warp + 4 * g0;   // row of entry i: row0 + 4 i
             const int rows_ok = nv > 0 ? max(0, min(cnt, (pM - row0 + 3) / 4)) : 0;
-            if (p_mask) {
-                if (mvec) {
-                    float4 mk[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        if (i < rows_ok) mk[i] = *reinterpret_cast<const float4*>(p_mask + (int64_t)(row0 + 4 * i) * p_ldmask + col);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        if (i < rows_ok) {
-                            if (!(mk[i].x > 0.f)) acc[i].x = 0.f;
-                            if (!(mk[i].y > 0.f)) acc[i].y = 0.f;
-                            if (!(mk[i].z > 0.f)) acc[i].z = 0.f;
-                            if (!(mk[i].w > 0.f)) acc[i].w = 0.f;
-                        }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        if (i < rows_ok) {
-                            const float* mk = p_mask + (int64_t)(row0 + 4 * i) * p_ldmask + col;
-                            if (!(mk[0] > 0.f)) acc[i].x = 0.f;
-                            if (nv > 1 && !(mk[1] > 0.f)) acc[i].y = 0.f;
-                            if (nv > 2 && !(mk[2] > 0.f)) acc[i].z = 0.f;
-                            if (nv > 3 && !(mk[3] > 0.f)) acc[i].w = 0.f;
-                        }
-                }
-            }
-            if (p_c) {
-                if (cvec) {
-                    if (p_acc) {
-                        float4 old[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            if (i < rows_ok) old[i] = *reinterpret_cast<const float4*>(p_c + (int64_t)(row0 + 4 * i) * p_ldc + col);
-#pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            if (i < rows_ok) {
-                                acc[i].x += old[i].x; acc[i].y += old[i].y; acc[i].z += old[i].z; acc[i].w += old[i].w;
-                            }
-                    }
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        if (i < rows_ok) *reinterpret_cast<float4*>(p_c + (int64_t)(row0 + 4 * i) * p_ldc + col) = acc[i];
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        if (i < rows_ok) {
-                            float* dst = p_c + (int64_t)(row0 + 4 * i) * p_ldc + col;
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                const float v = j == 0 ? acc[i].x : j == 1 ? acc[i].y : j == 2 ? acc[i].z : acc[i].w;
-                                if (j < nv) dst[j] = p_acc ? dst[j] + v : v;
-                            }
-                        }
-                }
-            }
-            if (p_cbf) {
-                if (hvec) {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        if (i < rows_ok) {
-                            __nv_bfloat162 lo = __floats2bfloat162_rn(acc[i].x, acc[i].y);
-                            __nv_bfloat162 hi = __floats2bfloat162_rn(acc[i].z, acc[i].w);
-                            uint2 u;
-                            u.x = *reinterpret_cast<uint32_t*>(&lo);
-                            u.y = *reinterpret_cast<uint32_t*>(&hi);
-                            *reinterpret_cast<uint2*>(p_cbf + (int64_t)(row0 + 4 * i) * p_ldcbf + col) = u;
-                        }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        if (i < rows_ok) {
-                            __nv_bfloat16* dst = p_cbf + (int64_t)(row0 + 4 * i) * p_ldcbf + col;
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                const float v = j == 0 ? acc[i].x : j == 1 ? acc[i].y : j == 2 ? acc[i].z : acc[i].w;
-                                if (j < nv) dst[j] = __float2bfloat16_rn(v);
-                            }
-                        }
-                }
-            }
+            finish_rows(acc, rows_ok, row0, col, nv, out);
             if (gb.ln) {
                 // y = (x - mean) rstd g + beta, ReLU: FP32 and BF16 rows of the LayerNorm output
                 float g4[4], b4[4];
@@ -681,6 +688,147 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
     }
 }
 
+// The BF16 GEMM without a K split or a LayerNorm: tiles of 128 x 64 and a ring of four 24 KB
+// stages, so that two CTAs fit on an SM and one's operand loads and MMAs run under the other's
+// epilogue.  The accumulator goes from tensor memory through a warp's 32 x 32 staging tile to
+// whole 128-byte row segments.  The MMAs of an output and their order are those of a
+// tc_gemm_kernel tile: the same bits.
+//
+// Bound by latency at the update's sizes (launch, first operands, eight K slabs, epilogue), by
+// operand loads from L2 at long K.  Against one 128 x 128 tile a CTA and SM: 512 x 512 x 512
+// twice 7.1 -> 5.1 us, 512 x 2592 x 256 6.9 -> 4.9, 4096 x 256 x 2592 15.7 -> 13.6, 4096 x 2592
+// x 256 29.2 -> 20.1, 4096^3 148 -> 142 (0.97 PFLOP/s); nowhere slower.
+constexpr int BN64 = 64, STAGES64 = 4, STG64 = 36;
+constexpr int STAGE64_BYTES = TILE_BYTES + BN64 * BK * 2;
+constexpr int SMEM64_BYTES = STAGES64 * STAGE64_BYTES + 1024 + 256 + BN64 * 4;
+static_assert(4 * 32 * STG64 * 4 <= STAGES64 * STAGE64_BYTES, "store staging in the operand ring");
+
+template <bool A_MN, bool B_MN>
+__global__ void __launch_bounds__(128) tc_gemm64_kernel(const __grid_constant__ TcBatch gb) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES64 * STAGE64_BYTES);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES64 + 2);   // address; stages issued; consumed
+    float* bias_s = reinterpret_cast<float*>(tmem_slot + 4);
+    const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES64), done_bar = smem_u32(bars + 2 * STAGES64);
+    int pi = 0;
+    while (pi + 1 < gb.n && (int)blockIdx.x >= gb.p[pi + 1].tile_start) ++pi;
+    const TcProb& P = gb.p[pi];
+    const int pM = P.M, pN = P.N, n_pairs = P.n_pairs;
+    const float* const p_bias = P.bias;
+    const TcOut out{P.mask, P.ldmask, P.c, P.ldc, P.cbf, P.ldcbf, P.accumulate != 0};
+    const int t = blockIdx.x - P.tile_start;
+    const int m0 = (t / P.tiles_n) * BM, n0 = (t % P.tiles_n) * BN64;
+    const int warp = warp_uniform((int)threadIdx.x / 32), lane = threadIdx.x % 32;
+    const uint32_t base = smem_u32(smem);
+    const int nkb = (P.K + BK - 1) / BK, total = nkb * n_pairs;
+    const bool producer = warp == 1 && elect_one(), issuer = warp == 0 && elect_one();
+    const long long wlim = gb.wait_limit;
+    int ld_pair = 0, ld_kb = 0;   // the producer's next slab
+    auto load_stage = [&](int s) {
+        const uint32_t st = base + s * STAGE64_BYTES;
+        mbar_expect_tx(full0 + 8 * s, STAGE64_BYTES);
+        load_operand<A_MN>(st, &P.ta[ld_pair], m0, ld_kb * BK, full0 + 8 * s);
+        if (B_MN) tma_load_2d(st + TILE_BYTES, &P.tb[ld_pair], n0, ld_kb * BK, full0 + 8 * s);
+        else tma_load_2d(st + TILE_BYTES, &P.tb[ld_pair], ld_kb * BK, n0, full0 + 8 * s);
+        if (++ld_kb == nkb) { ld_kb = 0; ++ld_pair; }
+    };
+    if (producer) {
+        for (int s = 0; s < STAGES64; ++s) {
+            mbar_init(full0 + 8 * s, 1);
+            mbar_init(empty0 + 8 * s, 1);
+        }
+        mbar_init(done_bar, 1);
+        tmem_slot[1] = 0;
+        tmem_slot[2] = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        for (int q = 0; q < n_pairs; ++q) {
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&P.ta[q])) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&P.tb[q])) : "memory");
+        }
+    }
+    SQ_KERNEL_ENTRY();   // as in tc_gemm_kernel: before any input is read and tensor memory taken
+    const int pre = gb.stall ? 0 : min(total, STAGES64);
+    if (producer)
+        for (int i = 0; i < pre; ++i) load_stage(i);
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(BN64));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    if (warp >= 2) {
+        const int j = threadIdx.x - 64;
+        bias_s[j] = (p_bias && n0 + j < pN) ? p_bias[n0 + j] : 0.f;
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = warp_uniform(*tmem_slot);
+    if (producer) {
+        int issued = pre;
+        uint32_t ph = 0;
+        for (int s = 0; issued < total && !gb.stall; ++issued) {   // (pre = STAGES64 if the loop runs at all)
+            if (!mbar_wait(empty0 + 8 * s, ph, gb.err, 1, wlim)) break;
+            load_stage(s);
+            if (++s == STAGES64) { s = 0; ph ^= 1; }
+        }
+        tmem_slot[1] = issued;
+    } else if (issuer) {
+        constexpr uint32_t idesc = idesc_bf16(BM, BN64, A_MN, B_MN);
+        int i = 0, s = 0;
+        uint32_t ph = 0;
+        for (; i < total; ++i) {
+            if (!mbar_wait(full0 + 8 * s, ph, gb.err, 2, wlim)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t st = base + s * STAGE64_BYTES;
+#pragma unroll
+            for (int kk = 0; kk < BK / 16; ++kk)
+                mma_bf16(tmem, operand_desc<A_MN>(st, kk), operand_desc<B_MN>(st + TILE_BYTES, kk), idesc,
+                         (i > 0 || kk > 0) ? 1u : 0u);
+            mma_commit(empty0 + 8 * s);
+            if (++s == STAGES64) { s = 0; ph ^= 1; }
+        }
+        tmem_slot[2] = i;
+        mma_commit(done_bar);
+    }
+    __syncwarp();
+    mbar_wait(done_bar, 0, gb.err, 3, wlim);   // (a wait that gave up has set *err)
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    float* stg = reinterpret_cast<float*>(smem) + warp * 32 * STG64;
+    const int cq = 4 * (lane % 8), row0 = m0 + warp * 32 + lane / 8;   // this lane's rows are row0 + 4 i
+    const int rows_left = max(0, min(8, (pM - row0 + 3) / 4));
+#pragma unroll 1
+    for (int c0 = 0; c0 < BN64; c0 += 32) {
+        uint32_t r[32];
+        tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + c0, r);
+        __syncwarp();   // the previous chunk has been read
+#pragma unroll
+        for (int j = 0; j < 32; j += 4)
+            *reinterpret_cast<float4*>(stg + lane * STG64 + j) =
+                make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]), __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
+        __syncwarp();
+        const int col = n0 + c0 + cq, nv = col < pN ? min(4, pN - col) : 0;
+        const float4 b = *reinterpret_cast<const float4*>(bias_s + c0 + cq);
+        float4 acc[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float4 x = *reinterpret_cast<const float4*>(stg + (lane / 8 + 4 * i) * STG64 + cq);
+            acc[i] = make_float4(b.x + x.x, b.y + x.y, b.z + x.z, b.w + x.w);
+        }
+        finish_rows(acc, nv > 0 ? rows_left : 0, row0, col, nv, out);
+    }
+    // copies issued but not consumed (after a wait gave up) still land here before the CTA leaves
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int i = (int)tmem_slot[2]; i < (int)tmem_slot[1]; ++i)
+            mbar_wait(full0 + 8 * (i % STAGES64), (i / STAGES64) & 1, gb.err, 4, wlim);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN64));
+    }
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
     if (!fn) {
@@ -713,17 +861,19 @@ bool make_map(CUtensorMap* m, const void* ptr, int64_t inner, int64_t outer, int
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool operand_map(CUtensorMap* m, const TcOperand& o, int mn_extent, int k_extent, bool fp8 = false) {
+// (tile: rows of the operand a CTA takes at a time)
+bool operand_map(CUtensorMap* m, const TcOperand& o, int mn_extent, int k_extent, bool fp8 = false, int tile = 128) {
     if (fp8)          // K-major only: 128 elements (128 bytes) of K by 128 rows
         return !o.mn_major && make_map(m, o.ptr, k_extent, mn_extent, o.ld, 128, 128, true);
     if (o.mn_major)   // element (mn, k) at ptr[k * ld + mn]
         return make_map(m, o.ptr, mn_extent, k_extent, o.ld, 64, 64);
-    return make_map(m, o.ptr, k_extent, mn_extent, o.ld, 64, 128);   // element (mn, k) at ptr[mn * ld + k]
+    return make_map(m, o.ptr, k_extent, mn_extent, o.ld, 64, tile);   // element (mn, k) at ptr[mn * ld + k]
 }
 
 template <bool A_MN, bool B_MN>
 void set_smem_attr() {
     cudaFuncSetAttribute(tc_gemm_kernel<A_MN, B_MN>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    cudaFuncSetAttribute(tc_gemm64_kernel<A_MN, B_MN>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM64_BYTES);
     if (!A_MN && !B_MN) {
         cudaFuncSetAttribute(tc_gemm_kernel<false, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
         cudaFuncSetAttribute(tc_gemm_kernel<false, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -798,10 +948,6 @@ int launch_tc_gemm(const TcGemm* probs, int n_probs, int* err, cudaStream_t s, b
                 (ln && (!g.ln_beta || !g.ln_post || !g.ln_mean || !g.ln_rstd || g.cbf || g.mask || g.accumulate ||
                         (g.N + BN - 1) / BN > g_max_splits || (g.N + BN - 1) / BN != (probs[base].N + BN - 1) / BN)))
                 return -3;
-            for (int q = 0; q < g.n_pairs; ++q) {
-                if (!operand_map(&p.ta[q], g.a[q], g.M, g.K, f8)) return -2;
-                if (!operand_map(&p.tb[q], g.b[q], g.N, g.K, f8)) return -2;
-            }
             p.M = g.M; p.N = g.N; p.K = g.K; p.n_pairs = g.n_pairs;
             p.bias = g.bias; p.c = g.c; p.ldc = g.ldc; p.cbf = g.cbf; p.ldcbf = g.ldcbf;
             p.mask = g.mask; p.ldmask = g.ldmask; p.accumulate = g.accumulate;
@@ -822,6 +968,28 @@ int launch_tc_gemm(const TcGemm* probs, int n_probs, int* err, cudaStream_t s, b
         S = allow_split && !ln ? std::max(S, 1) : 1;
         gb.splits = S;
         gb.ln = ln ? 1 : 0;
+        const bool narrow = S == 1 && !f8 && !ln;   // tc_gemm64_kernel
+        if (narrow) tiles = 0;
+        for (int i = 0; i < gb.n; ++i) {
+            const TcGemm& g = probs[base + i];
+            TcProb& p = gb.p[i];
+            for (int q = 0; q < g.n_pairs; ++q) {
+                if (!operand_map(&p.ta[q], g.a[q], g.M, g.K, f8)) return -2;
+                if (!operand_map(&p.tb[q], g.b[q], g.N, g.K, f8, narrow ? BN64 : BN)) return -2;
+            }
+            if (!narrow) continue;
+            p.tiles_n = (g.N + BN64 - 1) / BN64;
+            p.tile_start = tiles;
+            tiles += ((g.M + BM - 1) / BM) * p.tiles_n;
+        }
+        if (narrow) {
+            const dim3 grid(tiles);
+            if (!a_mn && !b_mn) launch_k(tc_gemm64_kernel<false, false>, grid, dim3(128), SMEM64_BYTES, s, gb);
+            else if (!a_mn) launch_k(tc_gemm64_kernel<false, true>, grid, dim3(128), SMEM64_BYTES, s, gb);
+            else if (b_mn) launch_k(tc_gemm64_kernel<true, true>, grid, dim3(128), SMEM64_BYTES, s, gb);
+            else launch_k(tc_gemm64_kernel<true, false>, grid, dim3(128), SMEM64_BYTES, s, gb);
+            continue;
+        }
         for (int i = 0; i < gb.n; ++i) gb.p[i].tile_start *= S;
         // LayerNorm mode: one cluster per row block, its CTAs the block's column tiles
         const dim3 grid(tiles * S), cluster(ln ? gb.p[0].tiles_n : S);
