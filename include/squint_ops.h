@@ -282,6 +282,63 @@ int squint_op_tanh_gaussian_fwd(int rows, int A, const float* out, const float* 
 int squint_op_tanh_gaussian_bwd(int rows, int A, const float* out, const float* eps, const float* da,
                                 const float* dlogp, float lo, float hi, float* dout, void* stream);
 
+/* ------------------------------------------------------------------ layers
+ * Whole layers, one call a direction: the operations above on the same operands (the
+ * same casts, products and reductions), without a host round trip, a fill or a pass
+ * between them.  All buffers are the caller's; contents need not be cleared.
+ *
+ * Linear layer on BF16 operands: y = bf16(x) bf16(w)^T + bias.  x [M, K], w [N, K] FP32
+ * (row strides ldx, ldw); xh, wh receive the BF16 operands (row strides multiples of 8,
+ * 16-byte aligned, pad columns zeroed) that the backward reads; y [M, N].
+ * Backward from dy [M, N] (contiguous): dyh receives bf16(dy) (row stride lddyh, a
+ * multiple of 8); dx = bf16(dy) wh [M, K], dw = bf16(dy)^T xh [N, K], db = the column
+ * sums of dy [N]; each may be NULL.  work: ..._bwd_workspace(M, N) bytes (with db).
+ */
+int squint_op_linear_bf16_fwd(int M, int N, int K, const float* x, int64_t ldx, const float* w, int64_t ldw,
+                              const float* bias, void* xh, int64_t ldxh, void* wh, int64_t ldwh, float* y, void* stream);
+size_t squint_op_linear_bf16_bwd_workspace(int M, int N);
+int squint_op_linear_bf16_bwd(int M, int N, int K, const float* dy, const void* xh, int64_t ldxh, const void* wh,
+                              int64_t ldwh, void* dyh, int64_t lddyh, float* dx, float* dw, float* db, void* work,
+                              size_t work_bytes, void* stream);
+/* Backward of the FP32 linear layer: dx = dy w [M, K], dw = dy^T x [N, K], db = column sums
+ * of dy; dy [M, N] contiguous, x and w with any strides; each output may be NULL. */
+int squint_op_linear_bwd(int M, int N, int K, const float* dy, const float* x, int64_t sx_m, int64_t sx_k, const float* w,
+                         int64_t sw_n, int64_t sw_k, float* dx, float* dw, float* db, void* stream);
+/*
+ * A LayerNorm MLP head (squint_op_mlp_bf16) from FP32 x and weights, which it rounds to
+ * BF16 into xh and wh[l] (row strides multiples of 8), and its whole backward from dout
+ * [M, nout] (contiguous): dx [M, kin] and, for every layer, dw[l], db[l] and (hidden layers)
+ * dg[l], dbeta[l].  pre, post, post_bf, mean, rstd: the forward's saves, every entry set.
+ * work: 256-byte aligned, squint_op_mlp_head_bwd_workspace() bytes.
+ */
+int squint_op_mlp_head_fwd(int M, int kin, int nh, int H, int nout, const float* x, int64_t ldx, const float* const* w,
+                           const int64_t* ldw, const float* const* bias, const float* const* g, const float* const* beta,
+                           float eps, void* xh, int64_t ldxh, void* const* wh, const int64_t* ldwh, float* out,
+                           float* const* pre, float* const* post, void* const* post_bf, float* const* mean,
+                           float* const* rstd, void* stream);
+size_t squint_op_mlp_head_bwd_workspace(int M, int nh, int H, int nout);
+int squint_op_mlp_head_bwd(int M, int kin, int nh, int H, int nout, const float* dout, const void* xh, int64_t ldxh,
+                           const void* const* wh, const int64_t* ldwh, const float* const* g, const float* const* pre,
+                           const float* const* post, const void* const* post_bf, const float* const* mean,
+                           const float* const* rstd, float* dx, float* const* dw, float* const* db, float* const* dg,
+                           float* const* dbeta, void* work, size_t work_bytes, void* stream);
+/*
+ * The 32 -> 32 channel, stride-1 convolution layer (squint_op_conv32) from NCHW FP32
+ * tensors: xp [nimg, (H+4)(W+4), 32] BF16 receives the padded input, w_fwd and w_bwd the
+ * filter layouts.  Backward from dy [nimg, 32, H-2, W-2]: dyp [nimg, (H+2)(W+2), 32] receives
+ * bf16(dy), zeroed where y (the ReLU output, NULL without ReLU) is not above zero; dx may be
+ * NULL; work: squint_op_wgrad32_workspace(nimg) bytes.
+ */
+int squint_op_conv32_layer_fwd(int nimg, int H, int W, const float* x, const float* w, const float* bias, int relu, void* xp,
+                               void* w_fwd, void* w_bwd, float* y, void* stream);
+int squint_op_conv32_layer_bwd(int nimg, int H, int W, const float* dy, const float* y, const void* xp, const void* w_bwd,
+                               void* dyp, float* dx, float* dw, float* db, void* work, size_t work_bytes, void* stream);
+/* The mean over rows of squint_op_categorical_ce's row_loss (row_loss [rows]: scratch, *loss on the
+ * device), and its gradient at the logits given the device scalar *dloss. */
+int squint_op_ce_mean_fwd(int rows, int K, const float* logits, const float* m, float* row_loss, float* loss, void* stream);
+int squint_op_ce_mean_bwd(int rows, int K, const float* logits, const float* m, const float* dloss, float* dlogits,
+                          void* stream);
+
 #ifdef __cplusplus
 }
 #endif

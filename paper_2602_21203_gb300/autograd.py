@@ -49,6 +49,8 @@ class Linear(torch.autograd.Function):
     def backward(ctx, dy):
         x, w = ctx.saved_tensors
         dy = dy.contiguous()
+        if dy.dtype == torch.float32:
+            return ops.linear_bwd(dy, x, w, ctx.needs_input_grad)
         rows, n_out = dy.shape
         n_in = x.shape[1]
         dx = ops.gemm(dy, w.t(), M=rows, N=n_in, K=n_out) if ctx.needs_input_grad[0] else None
@@ -98,19 +100,13 @@ class CategoricalCE(torch.autograd.Function):
     @staticmethod
     def forward(ctx, logits, m, v_min, v_max):
         logits, m = logits.contiguous(), m.contiguous()
-        rows = logits.shape[0]
-        loss_rows, _, _ = ops.categorical_ce(logits, m, v_min, v_max, 1.0 / rows)
-        ctx.v = (v_min, v_max)
         ctx.save_for_backward(logits, m)
-        inv = torch.full((1, rows), 1.0 / rows, dtype=loss_rows.dtype, device=loss_rows.device)
-        return ops.gemm(inv, loss_rows.reshape(1, rows), M=1, N=1, K=rows).reshape(())
+        return ops.ce_mean(logits, m)
 
     @staticmethod
     def backward(ctx, dloss):
         logits, m = ctx.saved_tensors
-        scale = float(dloss) / logits.shape[0]
-        _, dlogits, _ = ops.categorical_ce(logits, m, ctx.v[0], ctx.v[1], scale)
-        return dlogits, None, None, None
+        return ops.ce_mean_bwd(logits, m, dloss.contiguous()), None, None, None
 
 
 class TanhGaussian(torch.autograd.Function):
@@ -141,21 +137,14 @@ class LinearBF16(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, x, w, b):
-        xh, wh = ops.cast_bf16(x), ops.cast_bf16(w)
+        y, xh, wh = ops.linear_bf16_fwd(x, w, b)
         ctx.save_for_backward(xh, wh)
-        return ops.gemm(xh, wh, bias=b)
+        return y
 
     @staticmethod
     def backward(ctx, dy):
         xh, wh = ctx.saved_tensors
-        dy = dy.contiguous()
-        dyh = ops.cast_bf16(dy)
-        rows, n_out = dy.shape
-        n_in = xh.shape[1]
-        dx = ops.gemm(dyh, wh.t(), M=rows, N=n_in, K=n_out) if ctx.needs_input_grad[0] else None
-        dw = ops.gemm(dyh.t(), xh.t(), M=n_out, N=n_in, K=rows) if ctx.needs_input_grad[1] else None
-        db = _col_sum(dy) if ctx.needs_input_grad[2] else None
-        return dx, dw, db
+        return ops.linear_bf16_bwd(dy.contiguous(), xh, wh, ctx.needs_input_grad)
 
 
 class Conv32BF16(torch.autograd.Function):
@@ -165,24 +154,15 @@ class Conv32BF16(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, x, w, b, relu=True):
-        n, c, H, W = x.shape
-        xp = ops.to_phwc(x.contiguous())
-        wf, wb = ops.conv32_layouts(w)
-        _, y = ops.conv32_fwd(xp, H, W, wf, b, relu)
-        ctx.relu, ctx.hw = relu, (H, W)
+        y, xp, wb = ops.conv32_layer_fwd(x.contiguous(), w, b, relu)
+        ctx.relu = relu
         ctx.save_for_backward(xp, wb, y)
         return y
 
     @staticmethod
     def backward(ctx, dy):
         xp, wb, y = ctx.saved_tensors
-        H, W = ctx.hw
-        dy = dy.contiguous()
-        if ctx.relu:
-            dy = ops.relu_bwd(dy, y)
-        dyp = ops.to_phwc(dy)
-        dx = ops.conv32_dgrad(dyp, H - 2, W - 2, wb)[1] if ctx.needs_input_grad[0] else None
-        dw, db = ops.wgrad32(xp, dyp, H, W)
+        dx, dw, db = ops.conv32_layer_bwd(dy.contiguous(), y if ctx.relu else None, xp, wb, ctx.needs_input_grad[0])
         return dx, dw, db, None
 
 
@@ -197,41 +177,21 @@ class MlpHeadBF16(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x, eps, *params):
         nh = (len(params) - 2) // 4
-        ws = [ops.cast_bf16(params[4 * l]) for l in range(nh)] + [ops.cast_bf16(params[4 * nh])]
-        bs = [params[4 * l + 1] for l in range(nh)] + [params[4 * nh + 1]]
         gs = [params[4 * l + 2] for l in range(nh)]
-        betas = [params[4 * l + 3] for l in range(nh)]
-        xh = ops.cast_bf16(x)
-        out, saved = ops.mlp_bf16(xh, ws, bs, gs, betas, eps=eps)
-        ctx.nh = nh
-        flat = [t for sv in saved for t in sv]
-        ctx.save_for_backward(xh, *ws, *gs, *flat)
+        out, saved = ops.mlp_head_fwd(x, params[0::4], params[1::4], gs, [params[4 * l + 3] for l in range(nh)], eps)
+        ctx.kin = x.shape[1]
+        ctx.save_for_backward(*gs, *saved)
         return out
 
     @staticmethod
     def backward(ctx, dout):
-        nh = ctx.nh
         st = ctx.saved_tensors
-        xh, ws, gs = st[0], st[1:nh + 2], st[nh + 2:2 * nh + 2]
-        saved = [st[2 * nh + 2 + 5 * l: 2 * nh + 7 + 5 * l] for l in range(nh)]   # pre, post, post_bf, mean, rstd
-        grads = [None] * (4 * nh + 2)
-        dy = dout.contiguous()
-        for l in range(nh, -1, -1):
-            h = xh if l == 0 else saved[l - 1][2]                       # the layer's BF16 input
-            dyh = ops.cast_bf16(dy)
-            rows, n_out = dy.shape
-            n_in = h.shape[1]
-            gi = 4 * l
-            grads[gi] = ops.gemm(dyh.t(), h.t(), M=n_out, N=n_in, K=rows)
-            grads[gi + 1] = _col_sum(dy)
-            dh = ops.gemm(dyh, ws[l].t(), M=rows, N=n_in, K=n_out)
-            if l == 0:
-                dx = dh
-                break
-            pre, post, _, mean, rstd = saved[l - 1]
-            dy, dg, dbeta = ops.layernorm_bwd(dh, post, pre, mean, rstd, gs[l - 1], relu=True)
-            grads[4 * (l - 1) + 2], grads[4 * (l - 1) + 3] = dg, dbeta
-        return (dx, None, *grads)
+        gs, saved = st[:-6], st[-6:]
+        dx, dws, dbs, dgs, dbetas = ops.mlp_head_bwd(dout.contiguous(), gs, saved, ctx.kin)
+        grads = []
+        for l in range(len(gs)):
+            grads += [dws[l], dbs[l], dgs[l], dbetas[l]]
+        return (dx, None, *grads, dws[-1], dbs[-1])
 
 
 linear = Linear.apply

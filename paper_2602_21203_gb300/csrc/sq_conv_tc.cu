@@ -1026,6 +1026,40 @@ __global__ void to_phwc_kernel(const float* __restrict__ src, int64_t img_stride
     for (int c = 0; c < 4; ++c) reinterpret_cast<uint4*>(d)[c] = reinterpret_cast<const uint4*>(hb)[c];
 }
 
+// The same with the zero border and an optional ReLU mask, a thread a padded pixel: one pass
+// where filling the buffer, masking and converting were three.
+template <bool MASK>
+__global__ void __launch_bounds__(128) to_phwc_whole_kernel(const float* __restrict__ src, const float* __restrict__ mask, int nimg,
+                                                            int H, int W, __nv_bfloat16* __restrict__ dst) {
+    SQ_KERNEL_ENTRY();
+    const int wp = W + 4, pix = (H + 4) * wp;
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= (int64_t)nimg * pix) return;
+    const int img = (int)(p / pix), rem = (int)(p - (int64_t)img * pix);
+    const int y = rem / wp - 2, x = rem - (rem / wp) * wp - 2;
+    uint4* d = reinterpret_cast<uint4*>(dst + p * kCh);
+    if (y < 0 || y >= H || x < 0 || x >= W) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) d[c] = make_uint4(0u, 0u, 0u, 0u);
+        return;
+    }
+    const int64_t at = (int64_t)img * kCh * H * W + y * W + x;
+    float v[kCh];
+#pragma unroll
+    for (int c = 0; c < kCh; ++c) v[c] = src[at + (int64_t)c * H * W];
+    if (MASK) {
+        float m[kCh];
+#pragma unroll
+        for (int c = 0; c < kCh; ++c) m[c] = mask[at + (int64_t)c * H * W];
+#pragma unroll
+        for (int c = 0; c < kCh; ++c) v[c] = m[c] > 0.f ? v[c] : 0.f;
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        d[c] = make_uint4(pack2_bf16(v[8 * c], v[8 * c + 1]), pack2_bf16(v[8 * c + 2], v[8 * c + 3]),
+                          pack2_bf16(v[8 * c + 4], v[8 * c + 5]), pack2_bf16(v[8 * c + 6], v[8 * c + 7]));
+}
+
 // Padded HWC BF16 interior -> NCHW FP32.
 __global__ void from_phwc_kernel(const __nv_bfloat16* __restrict__ src, int nimg, int H, int W, float* __restrict__ dst) {
     SQ_KERNEL_ENTRY();
@@ -1280,6 +1314,13 @@ int launch_encoder_tc(const EncoderTc& c, int* err, cudaStream_t s) {
 void launch_to_phwc(const float* src, int64_t img_stride, int nimg, int H, int W, __nv_bfloat16* dst, cudaStream_t s) {
     const int64_t n = (int64_t)nimg * H * W;
     if (n) launch_k(to_phwc_kernel, dim3((unsigned)((n + 127) / 128)), dim3(128), 0, s, src, img_stride, nimg, H, W, dst);
+}
+void launch_to_phwc_whole(const float* src, const float* mask, int nimg, int H, int W, __nv_bfloat16* dst, cudaStream_t s) {
+    const int64_t n = (int64_t)nimg * (H + 4) * (W + 4);
+    if (n <= 0) return;
+    const dim3 grid((unsigned)((n + 127) / 128));
+    if (mask) launch_k(to_phwc_whole_kernel<true>, grid, dim3(128), 0, s, src, mask, nimg, H, W, dst);
+    else launch_k(to_phwc_whole_kernel<false>, grid, dim3(128), 0, s, src, mask, nimg, H, W, dst);
 }
 void launch_from_phwc(const __nv_bfloat16* src, int nimg, int H, int W, float* dst, cudaStream_t s) {
     const int64_t n = (int64_t)nimg * kCh * H * W;

@@ -219,13 +219,16 @@ struct CeArgs {
     const float* m;            // [B, K]
     float v_min, v_max;
     float scale;               // dlogits = (softmax - m) * scale
-    float* dlogits;            // [E, B, K]
+    const float* upstream;     // optional device scalar: scale = *upstream / (E B) instead
+    float* dlogits;            // [E, B, K] (null: losses only)
     __nv_bfloat16* dlogits_bf; int64_t ld_bf;   // optional BF16 copy [E, B, ld_bf]
-    float* row_loss;           // [E*B]
-    float* row_q;              // [E*B]
+    float* row_loss;           // [E*B] (null: gradients only)
+    float* row_q;              // [E*B] (may be null)
     int mse;                   // scalar critics (Eq. 2): loss (Q - y)^2, dQ = 2 (Q - y) scale
 };
 void launch_ce(const CeArgs& a, cudaStream_t s);
+// *out = the mean of v[0 .. n) (one block, fixed order).
+void launch_mean(const float* v, int n, float* out, cudaStream_t s);
 
 struct ActorQArgs {
     int B, K, E;

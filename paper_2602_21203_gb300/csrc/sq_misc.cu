@@ -408,6 +408,7 @@ __global__ void __launch_bounds__(32 * kHeadRows) ce_kernel(CeArgs a) {
         }
         return;
     }
+    const float scale = a.upstream ? __fdiv_rn(*a.upstream, (float)(a.E * a.B)) : a.scale;
     const float dz = (a.v_max - a.v_min) / (float)(K - 1);
     float l[V], mv[V], mx = -INFINITY;
 #pragma unroll
@@ -433,13 +434,35 @@ __global__ void __launch_bounds__(32 * kHeadRows) ce_kernel(CeArgs a) {
         const float p = expf(ls);
         loss -= mv[k] * ls;
         q += p * (a.v_min + (float)j * dz);
-        const float g = (p - mv[k]) * a.scale;
-        a.dlogits[(int64_t)er * K + j] = g;
+        const float g = (p - mv[k]) * scale;
+        if (a.dlogits) a.dlogits[(int64_t)er * K + j] = g;
         if (a.dlogits_bf) a.dlogits_bf[(int64_t)er * a.ld_bf + j] = __float2bfloat16_rn(g);
     }
     loss = warp_sum(loss);
     q = warp_sum(q);
-    if (lane == 0) { a.row_loss[er] = loss; a.row_q[er] = q; }
+    if (lane == 0) {
+        if (a.row_loss) a.row_loss[er] = loss;
+        if (a.row_q) a.row_q[er] = q;
+    }
+}
+
+__global__ void __launch_bounds__(512) mean_kernel(const float* __restrict__ v, int n, float* __restrict__ out) {
+    SQ_KERNEL_ENTRY();
+    __shared__ float part[16];
+    float s = 0.f;
+    for (int i0 = threadIdx.x; i0 < n; i0 += 4 * 512) {   // four loads in flight, added in order
+        float x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = i0 + 512 * u < n ? v[i0 + 512 * u] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) s += x[u];
+    }
+    s = warp_sum(s);
+    if (threadIdx.x % 32 == 0) part[threadIdx.x / 32] = s;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    s = warp_sum(threadIdx.x < 16 ? part[threadIdx.x] : 0.f);
+    if (threadIdx.x == 0) *out = s / (float)n;
 }
 
 // Actor objective through the critics, one warp per sample over all critics:
@@ -991,6 +1014,9 @@ void launch_ce(const CeArgs& a, cudaStream_t s) {
     const dim3 g((a.E * a.B + kHeadRows - 1) / kHeadRows), t(32 * kHeadRows);
     if (a.K <= 128) launch_k(ce_kernel<4>, g, t, 0, s, a);
     else launch_k(ce_kernel<8>, g, t, 0, s, a);
+}
+void launch_mean(const float* v, int n, float* out, cudaStream_t s) {
+    launch_k(mean_kernel, dim3(1), dim3(512), 0, s, v, n, out);
 }
 void launch_actor_q(const ActorQArgs& a, cudaStream_t s) {
     const dim3 g((a.B + kHeadRows - 1) / kHeadRows), t(32 * kHeadRows);

@@ -455,6 +455,196 @@ int squint_op_c51_project(int rows, int K, int E, const float* logits, const flo
     return launch_status();
 }
 
+// ---------------------------------------------------------------- layers, one call a direction
+int squint_op_linear_bf16_fwd(int M, int N, int K, const float* x, int64_t ldx, const float* w, int64_t ldw,
+                              const float* bias, void* xh, int64_t ldxh, void* wh, int64_t ldwh, float* y, void* stream) {
+    if (M < 0 || N < 1 || K < 1 || !x || !w || !xh || !wh || !y || ldx < K || ldw < K || ldxh < K || ldwh < K)
+        return SQUINT_EINVAL;
+    cudaStream_t s = (cudaStream_t)stream;
+    const CastItem it[2] = {{x, ldx, M, K, (__nv_bfloat16*)xh, ldxh}, {w, ldw, N, K, (__nv_bfloat16*)wh, ldwh}};
+    launch_cast_rows(it, 2, s);
+    if (M == 0) return launch_status();
+    TcGemm g{};
+    bf16_problem(M, N, K, xh, ldxh, 1, wh, ldwh, 1, y, N, bias, 0, &g);
+    int* err = tc_error_flag();
+    if (!err) return SQUINT_ECUDA;
+    if (launch_tc_gemm(&g, 1, err, s) != 0) return SQUINT_EINVAL;
+    return launch_status();
+}
+
+size_t squint_op_linear_bf16_bwd_workspace(int M, int N) {
+    return M < 1 || N < 1 ? 0 : sizeof(float) * (size_t)cast_colsum_workspace(M, N);
+}
+
+int squint_op_linear_bf16_bwd(int M, int N, int K, const float* dy, const void* xh, int64_t ldxh, const void* wh,
+                              int64_t ldwh, void* dyh, int64_t lddyh, float* dx, float* dw, float* db, void* work,
+                              size_t work_bytes, void* stream) {
+    if (M < 1 || N < 1 || K < 1 || !dy || !xh || !wh || !dyh || lddyh < N || ldxh < K || ldwh < K ||
+        (db && (!work || work_bytes < squint_op_linear_bf16_bwd_workspace(M, N))))
+        return SQUINT_EINVAL;
+    cudaStream_t s = (cudaStream_t)stream;
+    int* err = tc_error_flag();
+    if (!err) return SQUINT_ECUDA;
+    const CastItem it{dy, N, M, N, (__nv_bfloat16*)dyh, lddyh};
+    if (db) launch_cast_colsum(it, db, (float*)work, s);
+    else launch_cast_rows(&it, 1, s);
+    TcGemm g{};
+    if (dx) {
+        bf16_problem(M, K, N, dyh, lddyh, 1, wh, 1, ldwh, dx, K, nullptr, 0, &g);
+        if (launch_tc_gemm(&g, 1, err, s) != 0) return SQUINT_EINVAL;
+    }
+    if (dw) {
+        g = TcGemm{};
+        bf16_problem(N, K, M, dyh, 1, lddyh, xh, 1, ldxh, dw, K, nullptr, 0, &g);
+        if (launch_tc_gemm(&g, 1, err, s) != 0) return SQUINT_EINVAL;
+    }
+    return launch_status();
+}
+
+int squint_op_linear_bwd(int M, int N, int K, const float* dy, const float* x, int64_t sx_m, int64_t sx_k, const float* w,
+                         int64_t sw_n, int64_t sw_k, float* dx, float* dw, float* db, void* stream) {
+    if (M < 1 || N < 1 || K < 1 || !dy || !x || !w) return SQUINT_EINVAL;
+    int rc = SQUINT_OK;
+    if (dx) rc = squint_op_gemm(SQUINT_DT_F32, M, K, N, dy, N, 1, w, sw_k, sw_n, dx, K, nullptr, 0, stream);
+    if (dw && rc == SQUINT_OK) rc = squint_op_gemm(SQUINT_DT_F32, N, K, M, dy, 1, N, x, sx_k, sx_m, dw, K, nullptr, 0, stream);
+    if (rc != SQUINT_OK) return rc;
+    if (db) {
+        const ColSumProblem p{M, N, dy, N, db};
+        launch_colsum(&p, 1, (cudaStream_t)stream);
+    }
+    return launch_status();
+}
+
+int squint_op_mlp_head_fwd(int M, int kin, int nh, int H, int nout, const float* x, int64_t ldx, const float* const* w,
+                           const int64_t* ldw, const float* const* bias, const float* const* g, const float* const* beta,
+                           float eps, void* xh, int64_t ldxh, void* const* wh, const int64_t* ldwh, float* out,
+                           float* const* pre, float* const* post, void* const* post_bf, float* const* mean,
+                           float* const* rstd, void* stream) {
+    if (M < 0 || kin < 1 || nh < 1 || nh > kMlpMaxHidden || H < 1 || nout < 1 || !x || !w || !ldw || !xh || !wh || !ldwh)
+        return SQUINT_EINVAL;
+    CastItem it[kMlpMaxHidden + 2];
+    it[0] = CastItem{x, ldx, M, kin, (__nv_bfloat16*)xh, ldxh};
+    const void* whc[kMlpMaxHidden + 1];
+    for (int l = 0; l <= nh; ++l) {
+        const int rows = l == nh ? nout : H, cols = l == 0 ? kin : H;
+        if (!w[l] || !wh[l] || ldw[l] < cols || ldwh[l] < cols) return SQUINT_EINVAL;
+        it[l + 1] = CastItem{w[l], ldw[l], rows, cols, (__nv_bfloat16*)wh[l], ldwh[l]};
+        whc[l] = wh[l];
+    }
+    launch_cast_rows(it, nh + 2, (cudaStream_t)stream);
+    return squint_op_mlp_bf16(M, kin, nh, H, nout, xh, ldxh, whc, ldwh, bias, g, beta, eps, out, nout, pre, post, post_bf,
+                              mean, rstd, 0, stream);
+}
+
+// Workspace of the backward: per product a BF16 gradient, per hidden layer the gradient at its
+// output (FP32, reused), the gradient at its pre-activation and the LayerNorm's per-element terms.
+namespace {
+struct HeadBwdPlan { size_t dyh[kMlpMaxHidden + 1], dpre[kMlpMaxHidden], terms[kMlpMaxHidden], dh, part, bytes; };
+HeadBwdPlan head_bwd_plan(int M, int nh, int H, int nout) {
+    HeadBwdPlan p{};
+    size_t at = 0;
+    auto take = [&](size_t bytes) { const size_t o = at; at += (bytes + 255) / 256 * 256; return o; };
+    for (int l = 0; l <= nh; ++l) p.dyh[l] = take(2 * (size_t)M * (((l == nh ? nout : H) + 7) / 8 * 8));
+    for (int l = 0; l < nh; ++l) {
+        p.dpre[l] = take(4 * (size_t)M * H);
+        p.terms[l] = take(8 * (size_t)M * H);
+    }
+    p.dh = take(4 * (size_t)M * H);
+    p.part = take(4 * (size_t)cast_colsum_workspace(M, nout));
+    p.bytes = at;
+    return p;
+}
+}  // namespace
+
+size_t squint_op_mlp_head_bwd_workspace(int M, int nh, int H, int nout) {
+    if (M < 1 || nh < 1 || nh > kMlpMaxHidden || H < 1 || nout < 1) return 0;
+    return head_bwd_plan(M, nh, H, nout).bytes;
+}
+
+int squint_op_mlp_head_bwd(int M, int kin, int nh, int H, int nout, const float* dout, const void* xh, int64_t ldxh,
+                           const void* const* wh, const int64_t* ldwh, const float* const* g, const float* const* pre,
+                           const float* const* post, const void* const* post_bf, const float* const* mean,
+                           const float* const* rstd, float* dx, float* const* dw, float* const* db, float* const* dg,
+                           float* const* dbeta, void* work, size_t work_bytes, void* stream) {
+    if (M < 1 || kin < 1 || nh < 1 || nh > kMlpMaxHidden || H < 1 || nout < 1 || !dout || !xh || !wh || !ldwh || !g || !pre ||
+        !post || !post_bf || !mean || !rstd || !dx || !dw || !db || !dg || !dbeta || !work ||
+        (reinterpret_cast<uintptr_t>(work) & 255) || work_bytes < squint_op_mlp_head_bwd_workspace(M, nh, H, nout))
+        return SQUINT_EINVAL;
+    cudaStream_t s = (cudaStream_t)stream;
+    int* err = tc_error_flag();
+    if (!err) return SQUINT_ECUDA;
+    const HeadBwdPlan p = head_bwd_plan(M, nh, H, nout);
+    char* base = static_cast<char*>(work);
+    auto f32 = [&](size_t off) { return reinterpret_cast<float*>(base + off); };
+    auto width = [&](int l) { return l == nh ? nout : H; };
+    auto ldh = [&](int l) { return (int64_t)(width(l) + 7) / 8 * 8; };
+    const CastItem top{dout, nout, M, nout, (__nv_bfloat16*)(base + p.dyh[nh]), ldh(nh)};
+    launch_cast_colsum(top, db[nh], f32(p.part), s);
+    ln_prepare();
+    TcGemm wg[kMlpMaxHidden + 1] = {};
+    LnBwdProblem ln[kMlpMaxHidden] = {};
+    for (int l = nh; l >= 0; --l) {
+        const void* dyh = base + p.dyh[l];
+        const int n_in = l == 0 ? kin : H;
+        const void* h = l == 0 ? xh : post_bf[l - 1];
+        bf16_problem(width(l), n_in, M, dyh, 1, ldh(l), h, 1, l == 0 ? ldxh : H, dw[l], n_in, nullptr, 0, &wg[l]);
+        TcGemm gx{};
+        bf16_problem(M, n_in, width(l), dyh, ldh(l), 1, wh[l], 1, ldwh[l], l == 0 ? dx : f32(p.dh), n_in, nullptr, 0, &gx);
+        if (launch_tc_gemm(&gx, 1, err, s) != 0) return SQUINT_EINVAL;
+        if (l == 0) break;
+        LnBwdProblem& q = ln[l - 1];
+        q.rows = M; q.n = H;
+        q.dout = f32(p.dh); q.ld_dout = H; q.out = post[l - 1]; q.ld_out = H; q.pre = pre[l - 1]; q.ld_pre = H;
+        q.mean = mean[l - 1]; q.rstd = rstd[l - 1]; q.g = g[l - 1];
+        q.dpre = f32(p.dpre[l - 1]); q.ld_dpre = H;
+        q.dpre_bf = (__nv_bfloat16*)(base + p.dyh[l - 1]); q.ld_dpre_bf = ldh(l - 1);
+        q.dg = dg[l - 1]; q.dbeta = dbeta[l - 1]; q.dbias = db[l - 1];
+        q.terms = f32(p.terms[l - 1]);
+        launch_ln_bwd(&q, 1, nullptr, s);
+    }
+    if (launch_tc_gemm(wg, nh + 1, err, s) != 0) return SQUINT_EINVAL;
+    launch_ln_bwd_cols(ln, nh, s);
+    return launch_status();
+}
+
+int squint_op_conv32_layer_fwd(int nimg, int H, int W, const float* x, const float* w, const float* bias, int relu, void* xp,
+                               void* w_fwd, void* w_bwd, float* y, void* stream) {
+    if (nimg < 0 || H < 3 || W < 3 || !x || !w || !bias || !xp || !w_fwd || !w_bwd || !y) return SQUINT_EINVAL;
+    launch_to_phwc_whole(x, nullptr, nimg, H, W, (__nv_bfloat16*)xp, (cudaStream_t)stream);
+    launch_conv_weight_cast(w, (__nv_bfloat16*)w_fwd, (__nv_bfloat16*)w_bwd, (cudaStream_t)stream);
+    return squint_op_conv32(0, nimg, H, W, xp, w_fwd, bias, relu, nullptr, nullptr, y, stream);
+}
+
+int squint_op_conv32_layer_bwd(int nimg, int H, int W, const float* dy, const float* y, const void* xp, const void* w_bwd,
+                               void* dyp, float* dx, float* dw, float* db, void* work, size_t work_bytes, void* stream) {
+    if (nimg < 1 || H < 3 || W < 3 || !dy || !xp || !w_bwd || !dyp || !dw || !db) return SQUINT_EINVAL;
+    launch_to_phwc_whole(dy, y, nimg, H - 2, W - 2, (__nv_bfloat16*)dyp, (cudaStream_t)stream);
+    if (dx) {
+        const int rc = squint_op_conv32(1, nimg, H - 2, W - 2, dyp, w_bwd, nullptr, 0, nullptr, nullptr, dx, stream);
+        if (rc != SQUINT_OK) return rc;
+    }
+    return squint_op_wgrad32(nimg, H, W, xp, dyp, dw, db, work, work_bytes, stream);
+}
+
+int squint_op_ce_mean_fwd(int rows, int K, const float* logits, const float* m, float* row_loss, float* loss, void* stream) {
+    if (rows < 1 || K < 2 || K > 256 || !logits || !m || !row_loss || !loss) return SQUINT_EINVAL;
+    CeArgs a{};
+    a.B = rows; a.K = K; a.E = 1; a.logits = logits; a.m = m; a.v_min = 0.f; a.v_max = 1.f; a.row_loss = row_loss;
+    launch_ce(a, (cudaStream_t)stream);
+    launch_mean(row_loss, rows, loss, (cudaStream_t)stream);
+    return launch_status();
+}
+
+int squint_op_ce_mean_bwd(int rows, int K, const float* logits, const float* m, const float* dloss, float* dlogits,
+                          void* stream) {
+    if (rows < 1 || K < 2 || K > 256 || !logits || !m || !dloss || !dlogits) return SQUINT_EINVAL;
+    CeArgs a{};
+    a.B = rows; a.K = K; a.E = 1; a.logits = logits; a.m = m; a.v_min = 0.f; a.v_max = 1.f;
+    a.upstream = dloss; a.dlogits = dlogits;
+    launch_ce(a, (cudaStream_t)stream);
+    return launch_status();
+}
+
 int squint_op_tanh_gaussian_fwd(int rows, int A, const float* out, const float* eps, float lo, float hi, float* a,
                                 float* logp, void* stream) {
     if (rows < 0 || A < 1 || !out || !eps || !a || !logp) return SQUINT_EINVAL;

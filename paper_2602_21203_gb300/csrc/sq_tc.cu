@@ -1180,34 +1180,132 @@ void launch_quantize_mx(const QuantItem* items, int n, cudaStream_t s) {
 // ---------------------------------------------------------------- casts
 namespace {
 constexpr int kMaxCast = 48;
-struct CastBatch { CastItem it[kMaxCast]; int row_start[kMaxCast + 1]; int n; };
+struct CastBatch { CastItem it[kMaxCast]; int block_start[kMaxCast + 1]; int n; };
+constexpr int kCastRows = 8;   // rows a CTA, one a warp
 
-// One CTA per (matrix, row): FP32 row -> BF16 row of a padded matrix (pad columns zero).
-__global__ void cast_rows_kernel(CastBatch cb) {
+// FP32 rows -> BF16 rows of a padded matrix (pad columns zero), a warp a row, four elements a
+// lane where both rows are aligned for it.  4096 x 2592 and 256 x 2592 (68 MB, 10 us at the
+// measured copy rate): 12.6 us; 38 us in two launches with a 128-thread CTA a row and one element
+// a thread.
+__global__ void __launch_bounds__(32 * kCastRows) cast_rows_kernel(CastBatch cb) {
     SQ_KERNEL_ENTRY();
     int i = 0;
-    while (i + 1 < cb.n && (int)blockIdx.x >= cb.row_start[i + 1]) ++i;
+    while (i + 1 < cb.n && (int)blockIdx.x >= cb.block_start[i + 1]) ++i;
     const CastItem& c = cb.it[i];
-    const int r = blockIdx.x - cb.row_start[i];
+    const int r = (blockIdx.x - cb.block_start[i]) * kCastRows + threadIdx.x / 32, lane = threadIdx.x % 32;
+    if (r >= c.rows) return;
     const float* src = c.src + (int64_t)r * c.src_ld;
     __nv_bfloat16* dst = c.dst + (int64_t)r * c.dst_ld;
-    for (int j = threadIdx.x; j < c.dst_ld; j += blockDim.x)
-        dst[j] = __float2bfloat16_rn(j < c.cols ? src[j] : 0.f);
+    const int cols = c.cols, ld = (int)c.dst_ld;
+    if (((reinterpret_cast<uintptr_t>(src) & 15) | (reinterpret_cast<uintptr_t>(dst) & 7) | (ld & 3)) == 0) {
+        for (int j0 = 4 * lane; j0 < ld; j0 += 4 * 128) {
+            float4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int j = j0 + 128 * u;
+                if (j + 3 < cols) v[u] = *reinterpret_cast<const float4*>(src + j);
+                else v[u] = make_float4(j < cols ? src[j] : 0.f, j + 1 < cols ? src[j + 1] : 0.f,
+                                        j + 2 < cols ? src[j + 2] : 0.f, 0.f);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int j = j0 + 128 * u;
+                if (j >= ld) break;
+                const __nv_bfloat162 lo = __floats2bfloat162_rn(v[u].x, v[u].y), hi = __floats2bfloat162_rn(v[u].z, v[u].w);
+                *reinterpret_cast<uint2*>(dst + j) =
+                    make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+            }
+        }
+    } else {
+        for (int j0 = lane; j0 < ld; j0 += 4 * 32) {
+            float v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = j0 + 32 * u < cols ? src[j0 + 32 * u] : 0.f;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (j0 + 32 * u < ld) dst[j0 + 32 * u] = __float2bfloat16_rn(v[u]);
+        }
+    }
+}
+
+// The same for one matrix, with the column sums of 32 rows at a time: a warp takes rows w, w + 8,
+// ... of a block's 32 in order, four columns a lane, and the block adds its warps in order into
+// part[block][cols].
+__global__ void __launch_bounds__(256) cast_colsum_kernel(CastItem c, float* __restrict__ part) {
+    SQ_KERNEL_ENTRY();
+    __shared__ float4 sums[8][32];
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+    const int col = blockIdx.x * 128 + 4 * lane;
+    const int cols = c.cols, ld = (int)c.dst_ld;
+    const bool vec = ((reinterpret_cast<uintptr_t>(c.src) & 15) | (c.src_ld & 3)) == 0 && col + 3 < cols;
+    float4 v[4], s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int r = blockIdx.y * 32 + warp + 8 * u;
+        const float* p = c.src + (int64_t)r * c.src_ld + col;
+        v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r >= c.rows) continue;
+        if (vec) v[u] = *reinterpret_cast<const float4*>(p);
+        else v[u] = make_float4(col < cols ? p[0] : 0.f, col + 1 < cols ? p[1] : 0.f, col + 2 < cols ? p[2] : 0.f,
+                                col + 3 < cols ? p[3] : 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int r = blockIdx.y * 32 + warp + 8 * u;
+        s.x += v[u].x; s.y += v[u].y; s.z += v[u].z; s.w += v[u].w;
+        if (r >= c.rows) continue;
+        __nv_bfloat16* d = c.dst + (int64_t)r * c.dst_ld + col;
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(v[u].x, v[u].y), hi = __floats2bfloat162_rn(v[u].z, v[u].w);
+        if (((reinterpret_cast<uintptr_t>(c.dst) & 7) | (ld & 3)) == 0) {
+            if (col < ld)
+                *reinterpret_cast<uint2*>(d) =
+                    make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+            continue;
+        }
+        const __nv_bfloat16 h[4] = {lo.x, lo.y, hi.x, hi.y};
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (col + k < ld) d[k] = h[k];
+    }
+    sums[warp][lane] = s;
+    __syncthreads();
+    if (warp > 0) return;
+    s = sums[0][lane];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) {
+        const float4 t = sums[w][lane];
+        s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
+    }
+    float* out = part + (int64_t)blockIdx.y * cols + col;
+    const float f[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (col + k < cols) out[k] = f[k];
 }
 }  // namespace
+
+int64_t cast_colsum_workspace(int rows, int cols) { return (int64_t)((rows + 31) / 32) * cols; }
+
+void launch_cast_colsum(const CastItem& c, float* out, float* work, cudaStream_t s) {
+    const int blocks = (c.rows + 31) / 32;
+    if (!blocks || !c.cols) return;
+    launch_k(cast_colsum_kernel, dim3((unsigned)((c.dst_ld + 127) / 128), blocks), dim3(256), 0, s, c, work);
+    const ColSumProblem p{blocks, c.cols, work, c.cols, out};
+    launch_colsum(&p, 1, s);
+}
 
 void launch_cast_rows(const CastItem* items, int n, cudaStream_t s) {
     for (int base = 0; base < n; base += kMaxCast) {
         CastBatch cb;
         cb.n = std::min(kMaxCast, n - base);
-        int rows = 0;
+        int blocks = 0;
         for (int i = 0; i < cb.n; ++i) {
             cb.it[i] = items[base + i];
-            cb.row_start[i] = rows;
-            rows += items[base + i].rows;
+            cb.block_start[i] = blocks;
+            blocks += (items[base + i].rows + kCastRows - 1) / kCastRows;
         }
-        cb.row_start[cb.n] = rows;
-        if (rows) launch_k(cast_rows_kernel, dim3(rows), dim3(128), 0, s, cb);
+        cb.block_start[cb.n] = blocks;
+        if (blocks) launch_k(cast_rows_kernel, dim3(blocks), dim3(32 * kCastRows), 0, s, cb);
     }
 }
 

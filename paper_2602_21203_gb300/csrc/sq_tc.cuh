@@ -148,6 +148,9 @@ int launch_wgrad32_tc_partials(const WgradTc& c, int per_cta, float* work, int* 
 void launch_wgrad32_reduce(const float* work, int ctas, float* dw, float* db, cudaStream_t s);
 void conv_tc_prepare();
 void launch_to_phwc(const float* src, int64_t img_stride, int nimg, int H, int W, __nv_bfloat16* dst, cudaStream_t s);
+// The same from contiguous planes into a buffer of any contents: the zero border is written too.
+// With `mask` (planes like src), values whose mask is not above zero become zero.
+void launch_to_phwc_whole(const float* src, const float* mask, int nimg, int H, int W, __nv_bfloat16* dst, cudaStream_t s);
 void launch_from_phwc(const __nv_bfloat16* src, int nimg, int H, int W, float* dst, cudaStream_t s);
 // FP32 filter [32, 32, 3, 3] -> BF16 forward and data-gradient layouts (18432 B each).
 void launch_conv_weight_cast(const float* w, __nv_bfloat16* fwd, __nv_bfloat16* bwd, cudaStream_t s);
@@ -155,5 +158,9 @@ void launch_conv_weight_cast(const float* w, __nv_bfloat16* fwd, __nv_bfloat16* 
 // FP32 rows -> BF16 rows of a padded matrix (columns cols..dst_ld-1 set to zero).
 struct CastItem { const float* src; int64_t src_ld; int rows, cols; __nv_bfloat16* dst; int64_t dst_ld; };
 void launch_cast_rows(const CastItem* items, int n, cudaStream_t s);
+// The same for one matrix together with its column sums, out[j] = sum_r src[r, j] (deterministic
+// order), in two launches; `work` holds cast_colsum_workspace(rows, cols) floats.
+int64_t cast_colsum_workspace(int rows, int cols);
+void launch_cast_colsum(const CastItem& item, float* out, float* work, cudaStream_t s);
 
 }  // namespace sq

@@ -151,6 +151,18 @@ def load():
                                       ctypes.c_float, P, P]),
         "squint_op_tanh_gaussian_fwd": (I, [I, I, P, P, ctypes.c_float, ctypes.c_float, P, P, P]),
         "squint_op_tanh_gaussian_bwd": (I, [I, I, P, P, P, P, ctypes.c_float, ctypes.c_float, P, P]),
+        "squint_op_linear_bf16_fwd": (I, [I, I, I, P, I64, P, I64, P, P, I64, P, I64, P, P]),
+        "squint_op_linear_bf16_bwd_workspace": (SZ, [I, I]),
+        "squint_op_linear_bf16_bwd": (I, [I, I, I, P, P, I64, P, I64, P, I64, P, P, P, P, SZ, P]),
+        "squint_op_linear_bwd": (I, [I, I, I, P, P, I64, I64, P, I64, I64, P, P, P, P]),
+        "squint_op_mlp_head_fwd": (I, [I, I, I, I, I, P, I64, P, P, P, P, P, ctypes.c_float, P, I64, P, P, P, P, P, P, P,
+                                       P, P]),
+        "squint_op_mlp_head_bwd_workspace": (SZ, [I, I, I, I]),
+        "squint_op_mlp_head_bwd": (I, [I, I, I, I, I, P, P, I64, P, P, P, P, P, P, P, P, P, P, P, P, P, P, SZ, P]),
+        "squint_op_conv32_layer_fwd": (I, [I, I, I, P, P, P, I, P, P, P, P, P]),
+        "squint_op_conv32_layer_bwd": (I, [I, I, I, P, P, P, P, P, P, P, P, P, SZ, P]),
+        "squint_op_ce_mean_fwd": (I, [I, I, P, P, P, P, P]),
+        "squint_op_ce_mean_bwd": (I, [I, I, P, P, P, P, P]),
         "squint_op_to_phwc": (I, [I, I, I, P, P, P]),
         "squint_op_from_phwc": (I, [I, I, I, P, P, P]),
         "squint_op_conv32_layouts": (I, [P, P, P, P]),

@@ -14,11 +14,12 @@ _DT = {torch.float32: DT_F32, torch.float64: DT_F64, torch.bfloat16: DT_BF16}
 
 
 def _p(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _s():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """The current stream of the current device as an integer (cudaStream_t)."""
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _chk(rc, what):
@@ -41,8 +42,8 @@ def gemm(A, B, bias=None, out=None, accumulate=False, M=None, N=None, K=None):
     N = B.shape[0] if N is None else N
     dt = _DT[A.dtype]
     odt = torch.float32 if dt == DT_BF16 else A.dtype
-    if out is None:
-        out = torch.zeros(M, N, device=A.device, dtype=odt)
+    if out is None:   # (every element is written unless it is added to)
+        out = (torch.zeros if accumulate else torch.empty)(M, N, device=A.device, dtype=odt)
     _need(out, odt, "out")
     if bias is not None:
         _need(bias, odt, "bias")
@@ -291,6 +292,192 @@ def tanh_gaussian_bwd(out, eps, da, dlogp, lo=-5.0, hi=2.0):
     _chk(_lib.load().squint_op_tanh_gaussian_bwd(rows, A, _p(out), _p(eps), _p(da), _p(dlogp), float(lo), float(hi),
                                                  _p(dout), _s()), "squint_op_tanh_gaussian_bwd")
     return dout
+
+
+# ---------------------------------------------------------------- layers, one call a direction
+def _ptrs(tensors):
+    return (ctypes.c_void_p * len(tensors))(*[t.data_ptr() for t in tensors])
+
+
+def _addrs(base, step, n):
+    return (ctypes.c_void_p * n)(*[base + i * step for i in range(n)])
+
+
+def _pad8(n):
+    return (n + 7) // 8 * 8
+
+
+def linear_bf16_fwd(x, w, b):
+    """bf16(x) bf16(w)^T + b for FP32 x [rows, n_in], w [n_out, n_in].  Returns (y, xh, wh): the BF16
+    operands for the backward, row strides rounded up to 8."""
+    _need(x, torch.float32, "x")
+    _need(w, torch.float32, "w")
+    if b is not None:
+        _need(b, torch.float32, "bias")
+    M, K = x.shape
+    N = w.shape[0]
+    if x.stride(1) != 1:
+        x = x.contiguous()
+    if w.stride(1) != 1:
+        w = w.contiguous()
+    ld = _pad8(K)
+    xh, wh = x.new_empty((M, ld), dtype=torch.bfloat16), x.new_empty((N, ld), dtype=torch.bfloat16)
+    y = x.new_empty((M, N))
+    _chk(_lib.load().squint_op_linear_bf16_fwd(M, N, K, x.data_ptr(), x.stride(0), w.data_ptr(), w.stride(0), _p(b),
+                                               xh.data_ptr(), ld, wh.data_ptr(), ld, y.data_ptr(), _s()),
+         "squint_op_linear_bf16_fwd")
+    return y, xh[:, :K], wh[:, :K]
+
+
+def linear_bf16_bwd(dy, xh, wh, need=(True, True, True)):
+    """(dx, dw, db) of linear_bf16_fwd from dy [rows, n_out] FP32 (contiguous); None where not needed."""
+    _need(dy, torch.float32, "dy")
+    L = _lib.load()
+    M, N = dy.shape
+    K = xh.shape[1]
+    dx = dy.new_empty((M, K)) if need[0] else None
+    dw = dy.new_empty((N, K)) if need[1] else None
+    db = dy.new_empty(N) if need[2] else None
+    ld = _pad8(N)
+    wb = L.squint_op_linear_bf16_bwd_workspace(M, N) if need[2] else 0
+    buf = dy.new_empty(M * ld * 2 + wb, dtype=torch.uint8)      # bf16(dy), then the workspace
+    _chk(L.squint_op_linear_bf16_bwd(M, N, K, dy.data_ptr(), xh.data_ptr(), xh.stride(0), wh.data_ptr(), wh.stride(0),
+                                     buf.data_ptr(), ld, _p(dx), _p(dw), _p(db), buf.data_ptr() + M * ld * 2, wb, _s()),
+         "squint_op_linear_bf16_bwd")
+    return dx, dw, db
+
+
+def linear_bwd(dy, x, w, need=(True, True, True)):
+    """(dx, dw, db) of the FP32 y = x w^T + b from dy [rows, n_out] (contiguous); None where not needed."""
+    _need(dy, torch.float32, "dy")
+    M, N = dy.shape
+    K = x.shape[1]
+    dx = dy.new_empty((M, K)) if need[0] else None
+    dw = dy.new_empty((N, K)) if need[1] else None
+    db = dy.new_empty(N) if need[2] else None
+    _chk(_lib.load().squint_op_linear_bwd(M, N, K, dy.data_ptr(), x.data_ptr(), x.stride(0), x.stride(1), w.data_ptr(),
+                                          w.stride(0), w.stride(1), _p(dx), _p(dw), _p(db), _s()), "squint_op_linear_bwd")
+    return dx, dw, db
+
+
+def mlp_head_fwd(x, ws, biases, gs, betas, eps=1e-5):
+    """A LayerNorm MLP head from FP32 x [M, kin] and FP32 weights.  Returns (out, saved): saved =
+    (xh, wh, pre, post, post_bf, stats) with the BF16 weights in one buffer, the hidden layers'
+    pre-activations and outputs as [layers, M, H] and their (mean, rstd) as [2, layers, M]."""
+    _need(x, torch.float32, "x")
+    nh = len(ws) - 1
+    if x.stride(1) != 1:
+        x = x.contiguous()
+    ws = [w if w.stride(1) == 1 else w.contiguous() for w in ws]
+    for w in ws:
+        _need(w, torch.float32, "w")
+    M, kin = x.shape
+    H, nout = ws[0].shape[0], ws[-1].shape[0]
+    lds = [_pad8(w.shape[1]) for w in ws]
+    xh = x.new_empty((M, _pad8(kin)), dtype=torch.bfloat16)
+    sizes = [w.shape[0] * ld for w, ld in zip(ws, lds)]
+    wh = x.new_empty(sum(sizes), dtype=torch.bfloat16)
+    out = x.new_empty((M, nout))
+    pre, post = x.new_empty((nh, M, H)), x.new_empty((nh, M, H))
+    post_bf = x.new_empty((nh, M, H), dtype=torch.bfloat16)
+    stats = x.new_empty((2, nh, M))
+    at, wp = wh.data_ptr(), []
+    for n in sizes:
+        wp.append(at)
+        at += 2 * n
+    P, I64 = ctypes.c_void_p, ctypes.c_int64
+    _chk(_lib.load().squint_op_mlp_head_fwd(
+        M, kin, nh, H, nout, x.data_ptr(), x.stride(0), _ptrs(ws), (I64 * (nh + 1))(*[w.stride(0) for w in ws]),
+        _ptrs(biases), _ptrs(gs), _ptrs(betas), float(eps), xh.data_ptr(), xh.stride(0), (P * (nh + 1))(*wp),
+        (I64 * (nh + 1))(*lds), out.data_ptr(), _addrs(pre.data_ptr(), 4 * M * H, nh), _addrs(post.data_ptr(), 4 * M * H, nh),
+        _addrs(post_bf.data_ptr(), 2 * M * H, nh), _addrs(stats.data_ptr(), 4 * M, nh),
+        _addrs(stats.data_ptr() + 4 * nh * M, 4 * M, nh), _s()), "squint_op_mlp_head_fwd")
+    return out, (xh, wh, pre, post, post_bf, stats)
+
+
+def mlp_head_bwd(dout, gs, saved, kin):
+    """Gradients of mlp_head_fwd from dout [M, nout] (contiguous): (dx, dws, dbs, dgs, dbetas)."""
+    _need(dout, torch.float32, "dout")
+    xh, wh, pre, post, post_bf, stats = saved
+    L = _lib.load()
+    nh, M, H = pre.shape
+    nout = dout.shape[1]
+    ins = [kin] + [H] * nh
+    outs = [H] * nh + [nout]
+    lds = [_pad8(k) for k in ins]
+    at, wp = wh.data_ptr(), []
+    for n, ld in zip(outs, lds):
+        wp.append(at)
+        at += 2 * n * ld
+    dx = dout.new_empty((M, kin))
+    dws = [dout.new_empty((n, k)) for n, k in zip(outs, ins)]
+    dbs = [dout.new_empty(n) for n in outs]
+    dgs = [dout.new_empty(H) for _ in range(nh)]
+    dbetas = [dout.new_empty(H) for _ in range(nh)]
+    wb = L.squint_op_mlp_head_bwd_workspace(M, nh, H, nout)
+    work = dout.new_empty(max(wb, 1), dtype=torch.uint8)
+    P, I64 = ctypes.c_void_p, ctypes.c_int64
+    _chk(L.squint_op_mlp_head_bwd(
+        M, kin, nh, H, nout, dout.data_ptr(), xh.data_ptr(), xh.stride(0), (P * (nh + 1))(*wp), (I64 * (nh + 1))(*lds),
+        _ptrs(gs), _addrs(pre.data_ptr(), 4 * M * H, nh), _addrs(post.data_ptr(), 4 * M * H, nh),
+        _addrs(post_bf.data_ptr(), 2 * M * H, nh), _addrs(stats.data_ptr(), 4 * M, nh),
+        _addrs(stats.data_ptr() + 4 * nh * M, 4 * M, nh), dx.data_ptr(), _ptrs(dws), _ptrs(dbs), _ptrs(dgs), _ptrs(dbetas),
+        work.data_ptr(), wb, _s()), "squint_op_mlp_head_bwd")
+    return dx, dws, dbs, dgs, dbetas
+
+
+def conv32_layer_fwd(x, w, b, relu=True):
+    """The 32 -> 32 channel convolution layer from NCHW FP32 x.  Returns (y, xp, w_bwd): the padded-HWC
+    BF16 input and the data gradient's filter layout for the backward."""
+    n, c, H, W = x.shape
+    assert c == 32 and x.dtype == torch.float32
+    _need(x, torch.float32, "x")
+    xp = x.new_empty((n, (H + 4) * (W + 4), 32), dtype=torch.bfloat16)
+    wl = x.new_empty((2, 9 * 32 * 32), dtype=torch.bfloat16)
+    y = x.new_empty((n, 32, H - 2, W - 2))
+    w = w.contiguous()
+    _chk(_lib.load().squint_op_conv32_layer_fwd(n, H, W, x.data_ptr(), w.data_ptr(), b.data_ptr(), int(relu), xp.data_ptr(),
+                                                wl.data_ptr(), wl.data_ptr() + 9 * 32 * 32 * 2, y.data_ptr(), _s()),
+         "squint_op_conv32_layer_fwd")
+    return y, xp, wl[1]
+
+
+def conv32_layer_bwd(dy, y, xp, w_bwd, need_dx=True):
+    """(dx, dw, db) of conv32_layer_fwd from dy [n, 32, H-2, W-2] (contiguous); y: the ReLU's output, or None."""
+    n, _, oh, ow = dy.shape
+    H, W = oh + 2, ow + 2
+    L = _lib.load()
+    dx = dy.new_empty((n, 32, H, W)) if need_dx else None
+    dw, db = dy.new_empty((32, 32, 3, 3)), dy.new_empty(32)
+    pb = n * (oh + 4) * (ow + 4) * 64
+    wb = max(L.squint_op_wgrad32_workspace(n), 16)
+    buf = dy.new_empty(pb + wb, dtype=torch.uint8)      # bf16(dy) padded HWC, then the workspace
+    _chk(L.squint_op_conv32_layer_bwd(n, H, W, dy.data_ptr(), _p(y), xp.data_ptr(), w_bwd.data_ptr(), buf.data_ptr(), _p(dx),
+                                      dw.data_ptr(), db.data_ptr(), buf.data_ptr() + pb, wb, _s()),
+         "squint_op_conv32_layer_bwd")
+    return dx, dw, db
+
+
+def ce_mean(logits, m):
+    """Mean over rows of -sum_j m[r, j] log softmax(logits[r])_j, a 0-d tensor (nothing waits for it)."""
+    _need(logits, torch.float32, "logits")
+    _need(m, torch.float32, "m")
+    rows, K = logits.shape
+    buf = logits.new_empty(rows)
+    loss = logits.new_empty(())
+    _chk(_lib.load().squint_op_ce_mean_fwd(rows, K, logits.data_ptr(), m.data_ptr(), buf.data_ptr(), loss.data_ptr(), _s()),
+         "squint_op_ce_mean_fwd")
+    return loss
+
+
+def ce_mean_bwd(logits, m, dloss):
+    """Gradient of ce_mean at the logits, times the device scalar dloss."""
+    _need(dloss, torch.float32, "dloss")
+    rows, K = logits.shape
+    d = torch.empty_like(logits)
+    _chk(_lib.load().squint_op_ce_mean_bwd(rows, K, logits.data_ptr(), m.data_ptr(), dloss.data_ptr(), d.data_ptr(), _s()),
+         "squint_op_ce_mean_bwd")
+    return d
 
 
 # ---------------------------------------------------------------- tensor-core convolutions (32 -> 32, stride 1)
