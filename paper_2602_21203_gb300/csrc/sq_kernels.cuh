@@ -48,6 +48,7 @@ struct ActFrontArgs {
     int rows, C, H, W, f, P;
     float* x;                    // [rows, C, Hs, Ws]
     float* xin; int64_t ld_xin; int col;   // proprio goes to xin[row, col:col+P]
+    int aligned;                 // every frame of every request starts on 16 bytes
 };
 void launch_act_frontend(const ActFrontArgs& a, cudaStream_t s);
 // Opt the front-end kernels in to `frame_bytes` of dynamic shared memory (call once, outside capture).

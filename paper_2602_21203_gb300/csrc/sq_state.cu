@@ -244,7 +244,9 @@ int squint_handle::act(sq::ActArena& a, const squint_act_request* reqs, int n_re
     uint64_t* p64 = reinterpret_cast<uint64_t*>(hb + (size_t)act_cap * 8);
     int32_t* modes = reinterpret_cast<int32_t*>(p64 + 4 * (size_t)req_cap);
     int r = 0;
+    uintptr_t low = (uintptr_t)c.obs_c * c.obs_h * c.obs_w;   // low bits of every frame's address
     for (int q = 0; q < n_reqs; ++q) {
+        low |= reinterpret_cast<uintptr_t>(reqs[q].obs);
         for (int i = 0; i < reqs[q].n; ++i, ++r) { row_req[r] = q; row_in[r] = i; }
         p64[q] = (uint64_t)(uintptr_t)reqs[q].obs;
         p64[req_cap + q] = (uint64_t)(uintptr_t)reqs[q].proprio;
@@ -274,6 +276,7 @@ int squint_handle::act(sq::ActArena& a, const squint_act_request* reqs, int n_re
     af.rows = rows; af.C = c.obs_c; af.H = c.obs_h; af.W = c.obs_w; af.f = c.squint_f; af.P = c.proprio_dim;
     if (L.conv.empty()) { af.C = 0; af.H = af.W = af.f = 1; }   // state-based: no image
     af.x = ax; af.xin = axin; af.ld_xin = Da; af.col = L.zdim;
+    af.aligned = (low & 15) == 0;
     launch_act_frontend(af, s);
     // BF16 policy: layer-0 conv on CUDA cores, the 32-channel convs and every linear
     // layer on tcgen05 with the snapshot's BF16 copies, no K split (each row's result
