@@ -216,6 +216,13 @@ void launch_frontend(const FrontendArgs& a, cudaStream_t s) {
     launch_k(frontend_kernel, dim3(dim3(a.B, 2)), dim3(256), smem, s, a);
 }
 
+__device__ __forceinline__ void put_proprio(const ActFrontArgs& a, int r, const float* p, int threads) {
+    for (int k = threadIdx.x; k < a.P; k += threads) {
+        a.xin[(int64_t)r * a.ld_xin + a.col + k] = p[k];
+        if (a.xin_h) a.xin_h[(int64_t)r * a.ld_xin_h + a.col + k] = __float2bfloat16_rn(p[k]);
+    }
+}
+
 // Inference: one CTA per row; no shift (crop at the centre offset p = pad means
 // the identity, so it is left out entirely).
 __global__ void __launch_bounds__(256) act_frontend_kernel(ActFrontArgs a) {
@@ -257,7 +264,7 @@ __global__ void __launch_bounds__(256) act_frontend_kernel(ActFrontArgs a) {
         a.x[(int64_t)r * n_out + o] = (float)sum / denom - 0.5f;
     }
     const float* p = a.prop[q] + (int64_t)a.row_in_req[r] * a.P;
-    for (int k = threadIdx.x; k < a.P; k += blockDim.x) a.xin[(int64_t)r * a.ld_xin + a.col + k] = p[k];
+    put_proprio(a, r, p, (int)blockDim.x);
 }
 
 // The same where every frame starts on 16 bytes and its rows are whole 16-byte chunks (f = 4, 2
@@ -299,7 +306,7 @@ __global__ void __launch_bounds__(256) act_frontend_direct_kernel(ActFrontArgs a
     }
     if (blockIdx.y == 0) {
         const float* p = a.prop[q] + (int64_t)in_req * a.P;
-        for (int k = threadIdx.x; k < a.P; k += 256) a.xin[(int64_t)r * a.ld_xin + a.col + k] = p[k];
+        put_proprio(a, r, p, 256);
     }
 }
 

@@ -48,6 +48,7 @@ struct ActFrontArgs {
     int rows, C, H, W, f, P;
     float* x;                    // [rows, C, Hs, Ws]
     float* xin; int64_t ld_xin; int col;   // proprio goes to xin[row, col:col+P]
+    __nv_bfloat16* xin_h; int64_t ld_xin_h;   // optional BF16 copy of the same columns
     int aligned;                 // every frame of every request starts on 16 bytes
 };
 void launch_act_frontend(const ActFrontArgs& a, cudaStream_t s);

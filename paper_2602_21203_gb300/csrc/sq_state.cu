@@ -277,6 +277,8 @@ int squint_handle::act(sq::ActArena& a, const squint_act_request* reqs, int n_re
     if (L.conv.empty()) { af.C = 0; af.H = af.W = af.f = 1; }   // state-based: no image
     af.x = ax; af.xin = axin; af.ld_xin = Da; af.col = L.zdim;
     af.aligned = (low & 15) == 0;
+    const int64_t Da8 = (Da + 7) / 8 * 8;
+    if (bf16) { af.xin_h = axin_h; af.ld_xin_h = Da8; }
     launch_act_frontend(af, s);
     // BF16 policy: layer-0 conv on CUDA cores, the 32-channel convs and every linear
     // layer on tcgen05 with the snapshot's BF16 copies, no K split (each row's result
@@ -353,14 +355,14 @@ int squint_handle::act(sq::ActArena& a, const squint_act_request* reqs, int n_re
         p.rows = rows; p.n = Dd; p.pre = apre; p.ld_pre = Dd;
         p.g = Wp + L.aproj.g; p.beta = Wp + L.aproj.beta;
         p.out = axin; p.ld_out = Da; p.mean = amean; p.rstd = arstd;
+        if (bf16) { p.out_bf = axin_h; p.ld_out_bf = Da8; }
         launch_ln_fwd(&p, 1, false, (float)c.ln_eps, s);
     } else if (F > 0) {
         SQ_CK(this, cudaMemcpy2DAsync(axin, Da * sizeof(float), in, F * sizeof(float), F * sizeof(float), rows,
                                       cudaMemcpyDeviceToDevice, s));
     }
-    const int64_t Da8 = (Da + 7) / 8 * 8;
-    if (bf16) {
-        CastItem ci{axin, Da, rows, Da, axin_h, Da8};   // projected features and proprio, BF16
+    if (bf16 && Dd == 0 && F > 0) {   // features without a projection (else BF16 is written where the values arise)
+        CastItem ci{axin, Da, rows, Da, axin_h, Da8};
         launch_cast_rows(&ci, 1, s);
     }
     MlpRef actor_ref;
