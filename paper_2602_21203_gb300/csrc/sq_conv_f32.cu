@@ -91,7 +91,7 @@ struct ConvF32Args {
 // 46 % busy, the issue slots 77 %.
 template <int P, bool DGRAD>
 __global__ void __launch_bounds__(128) conv_f32_kernel(const __grid_constant__ ConvF32Args a) {
-    SQ_KERNEL_ENTRY();
+    SQ_KERNEL_WAIT();
     extern __shared__ __align__(16) float smem[];
     const int nt = blockDim.x, tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
     const int m0 = blockIdx.x * 32 * P, m1 = min(a.M, m0 + 32 * P), n0 = blockIdx.y * 32;
@@ -189,6 +189,7 @@ __global__ void __launch_bounds__(128) conv_f32_kernel(const __grid_constant__ C
             }
         }
     }
+    SQ_KERNEL_TRIGGER();
 #pragma unroll
     for (int i = 0; i < P; ++i) {
         const int m = m0 + lane + 32 * i;
@@ -302,7 +303,7 @@ template <int CI, int CO, bool SLIDE>
 __global__ void __launch_bounds__(CI * 32 / CO) wgrad_f32_kernel(const __grid_constant__ WgradF32Args a) {
     static_assert(CI * 32 / CO % kWTile == 0, "whole pixels a pass");
     constexpr int NT = CI * 32 / CO, DROW = CO == 4 ? 36 : 34;
-    SQ_KERNEL_ENTRY();
+    SQ_KERNEL_WAIT();
     extern __shared__ __align__(16) float smem[];
     const int tid = threadIdx.x, cg = tid % (32 / CO), ci_l = tid / (32 / CO);
     const int c0 = blockIdx.x * CI, co0 = blockIdx.y * 32, nci = min(CI, a.Cin - c0);
@@ -374,6 +375,7 @@ __global__ void __launch_bounds__(CI * 32 / CO) wgrad_f32_kernel(const __grid_co
             if (++oy == a.g.oh) { oy = 0; ++img; }
         }
     }
+    SQ_KERNEL_TRIGGER();
     const int N = a.Cin * 9 + 1;
     float* out = a.work + (int64_t)blockIdx.z * a.Cout * N;
 #pragma unroll
@@ -395,7 +397,7 @@ bool launch_wgrad(WgradF32Args a, int splits, cudaStream_t s) {
     const int64_t bytes = 8 * (kWTile * DROW + (CI * words + 3) / 4 * 4);
     if (bytes > kSmemBytes) return false;
     a.words = (int)words;
-    launch_k(wgrad_f32_kernel<CI, CO, SLIDE>, dim3((a.Cin + CI - 1) / CI, (a.Cout + 31) / 32, splits), dim3(CI * 32 / CO),
+    launch_with(false, wgrad_f32_kernel<CI, CO, SLIDE>, dim3((a.Cin + CI - 1) / CI, (a.Cout + 31) / 32, splits), dim3(CI * 32 / CO),
              (size_t)bytes, s, a);
     return true;
 }

@@ -139,7 +139,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 }
 
 __global__ void __launch_bounds__(kConvThreads) conv32_tc_kernel(const __grid_constant__ ConvArgs a) {
-    SQ_KERNEL_ENTRY();
+    SQ_KERNEL_WAIT();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t plane = (uint32_t)a.load_rows * 16;
@@ -297,6 +297,7 @@ __global__ void __launch_bounds__(kConvThreads) conv32_tc_kernel(const __grid_co
             if (!have) break;
         }
     }
+    SQ_KERNEL_TRIGGER();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 1) {
@@ -335,7 +336,7 @@ __host__ __device__ inline uint32_t wgrad_operand_bytes(uint32_t xbytes, uint32_
 }
 
 __global__ void __launch_bounds__(128) wgrad32_tc_kernel(const __grid_constant__ WgradArgs a) {
-    SQ_KERNEL_ENTRY();
+    SQ_KERNEL_WAIT();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t slot = (uint32_t)a.slot_rows * 16;
@@ -435,6 +436,7 @@ __global__ void __launch_bounds__(128) wgrad32_tc_kernel(const __grid_constant__
     }
     if (warp == 1 && elect_one()) mma_commit(done_bar);
     __syncwarp();
+    SQ_KERNEL_TRIGGER();
     const bool have = mbar_wait(done_bar, 0, a.err, 23) && ok && i1 > i0;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     // bias partials: reduce the 32 threads of each chunk in a fixed order.  The partial
@@ -818,7 +820,7 @@ __device__ __forceinline__ void gather_conv0(const EncArgs& a, const float* in, 
 }
 
 __global__ void __launch_bounds__(128 * kEncGroups, 1) encoder_tc_kernel(const __grid_constant__ EncArgs a) {
-    SQ_KERNEL_ENTRY();
+    SQ_KERNEL_WAIT();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
     const uint32_t group_bytes = a.xbytes + a.ybytes + a.ibytes;
@@ -993,6 +995,7 @@ __global__ void __launch_bounds__(128 * kEncGroups, 1) encoder_tc_kernel(const _
             if (last && l % 2 == 0 && img + step < a.nimg) gather();
         }
     }
+    SQ_KERNEL_TRIGGER();
     if (quarter == 0 && elect_one()) {   // every MMA this group issued has completed before the tensor memory is freed
         mma_commit(bar);
         mbar_wait(bar, phase & 1, a.err, 43);

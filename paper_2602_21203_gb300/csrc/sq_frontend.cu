@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(256, 4) frontend_kernel(FrontendArgs a) {
 
 void launch_frontend(const FrontendArgs& a, cudaStream_t s) {
     const size_t smem = squint4_direct(a) ? 0 : (size_t)a.C * a.H * a.W;   // the direct squint stages nothing
-    launch_k(frontend_kernel, dim3(dim3(a.B, 2)), dim3(256), smem, s, a);
+    launch_with(false, frontend_kernel, dim3(dim3(a.B, 2)), dim3(256), smem, s, a);
 }
 
 __device__ __forceinline__ void put_proprio(const ActFrontArgs& a, int r, const float* p, int threads) {

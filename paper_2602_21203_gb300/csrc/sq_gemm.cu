@@ -395,7 +395,7 @@ template <bool PHWC>
 __global__ void __launch_bounds__(128) conv_wgrad_c32_kernel(ConvShape sh, const void* __restrict__ dy_v,
                                                              const float* __restrict__ x, float* __restrict__ work,
                                                              int chunk) {
-    SQ_KERNEL_ENTRY();
+    SQ_KERNEL_WAIT();
     __shared__ float dys[32][kW0Tile + 1];   // [co][pixel]
     __shared__ float xs[32][kW0Tile + 1];    // [column][pixel]; column N - 1 is the bias (1)
     const int t = threadIdx.x;
@@ -485,6 +485,7 @@ __global__ void __launch_bounds__(128) conv_wgrad_c32_kernel(ConvShape sh, const
             }
         }
     }
+    SQ_KERNEL_TRIGGER();
     float* out = work + (int64_t)blockIdx.x * 32 * N;
 #pragma unroll
     for (int i = 0; i < 2; ++i)

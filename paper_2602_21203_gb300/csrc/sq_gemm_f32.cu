@@ -137,7 +137,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) gemm_f32_kernel(const _
     constexpr int FIT = kSmemBytes / (4 * (A_FLOATS + B_FLOATS)), kStages = FIT < 8 ? FIT : 8;
     static_assert(kStages >= 3, "operand ring");
     __shared__ __align__(16) float smem[kStages * (A_FLOATS + B_FLOATS)];
-    SQ_KERNEL_ENTRY();
+    SQ_KERNEL_WAIT();
     int pi = 0;
     while (pi + 1 < gb.n && (int)blockIdx.x >= gb.p[pi + 1].tile_start) ++pi;
     const GemmF32Problem& Q = gb.p[pi];
@@ -223,6 +223,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) gemm_f32_kernel(const _
         slot = next_slot;
     }
 
+    SQ_KERNEL_TRIGGER();
     float* C = static_cast<float*>(P.C);
     const float* bias = static_cast<const float*>(P.bias);
     const float* mask = static_cast<const float*>(P.mask);
@@ -260,7 +261,8 @@ void launch_tiles(GemmF32Batch& gb, cudaStream_t s) {
         tiles += ((gb.p[i].g.M + BM - 1) / BM) * gb.p[i].tiles_n;
     }
     if (tiles == 0) return;
-    launch_k(gemm_f32_kernel<BM, BN, TM, TN, BK, A_K, B_K>, dim3(tiles), dim3((BM / TM) * (BN / TN)), 0, s, gb);
+    // (a full grid of the large tile is not let in early: launch_with)
+    launch_with(BN < 64, gemm_f32_kernel<BM, BN, TM, TN, BK, A_K, B_K>, dim3(tiles), dim3((BM / TM) * (BN / TN)), 0, s, gb);
 }
 
 int count_tiles(const GemmF32Batch& gb, int bm, int bn) {

@@ -1029,7 +1029,7 @@ int launch_adam(const AdamArgs& a, cudaStream_t s) {
     if (a.n <= 0) return 0;
     RowPlan plan;
     if (!row_plan(a.n, a.seg, a.n_seg, a.tseg, a.target ? a.n_tseg : 0, &plan) || plan.rows < 1) return -1;
-    launch_k(adam_rows_kernel, dim3(plan.rows), dim3(kRowThreads), 0, s, a, plan);
+    launch_with(false, adam_rows_kernel, dim3(plan.rows), dim3(kRowThreads), 0, s, a, plan);
     return 0;
 }
 template <typename T>

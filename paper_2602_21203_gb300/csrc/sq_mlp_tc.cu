@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
     // every CTA of the cluster has started and initialised its barriers before any remote access
     if (CL > 1) cluster_sync_all();
     // inputs are read, and tensor memory taken, only once the previous kernel has finished
-    SQ_KERNEL_ENTRY();
+    SQ_KERNEL_WAIT();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
                      "r"(a.tmem_cols));
@@ -521,6 +521,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
                 // ------------------------------------------------------------ output layer epilogue
                 const int nout = a.nout;
                 const float* pob = par + nh * 3 * NS;
+                SQ_KERNEL_TRIGGER();
                 // this row's output (or partial output) into the idle weight ring, then coalesced
                 for (int c = 0; c < nop; c += 16) {
                     float v[16];
@@ -781,7 +782,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
     }
     __syncthreads();
     if (CL > 1) cluster_sync_all();
-    SQ_KERNEL_ENTRY();
+    SQ_KERNEL_WAIT();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
                      "r"(a.tmem_cols));
@@ -874,6 +875,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
             mbar_wait(acc_full, st & 1, err, 44, wlim);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (st == 0) epi_bar();   // the staged g slices
+            if (st + 1 == nsteps) SQ_KERNEL_TRIGGER();
             if (!fin) {
                 // ------------------------------------------------------------ LayerNorm (+ReLU) backward
                 const int c0 = rank * NS;

@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
     }
     // inputs are read, and tensor memory taken, only once the previous kernel has finished:
     // a kernel that holds tensor memory never waits on a later one
-    SQ_KERNEL_ENTRY();
+    SQ_KERNEL_WAIT();
     const int pre = gb.stall ? 0 : (total < STAGES ? total : STAGES);
     if (producer)
         for (int i = 0; i < pre; ++i) load_stage(i, i);   // first stages: no slot to wait for
@@ -493,6 +493,7 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
     // shared memory (the operand stages are idle once the final commit has arrived)
     const bool have = mbar_wait(done_bar, 0, gb.err, 3, wlim);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    SQ_KERNEL_TRIGGER();
     float* red = reinterpret_cast<float*>(smem);   // [BM][RED_LD]
     const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
     {
@@ -747,7 +748,7 @@ __global__ void __launch_bounds__(128) tc_gemm64_kernel(const __grid_constant__ 
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&P.tb[q])) : "memory");
         }
     }
-    SQ_KERNEL_ENTRY();   // as in tc_gemm_kernel: before any input is read and tensor memory taken
+    SQ_KERNEL_WAIT();   // as in tc_gemm_kernel: before any input is read and tensor memory taken
     const int pre = gb.stall ? 0 : min(total, STAGES64);
     if (producer)
         for (int i = 0; i < pre; ++i) load_stage(i);
@@ -793,6 +794,7 @@ __global__ void __launch_bounds__(128) tc_gemm64_kernel(const __grid_constant__ 
     __syncwarp();
     mbar_wait(done_bar, 0, gb.err, 3, wlim);   // (a wait that gave up has set *err)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    SQ_KERNEL_TRIGGER();
     float* stg = reinterpret_cast<float*>(smem) + warp * 32 * STG64;
     const int cq = 4 * (lane % 8), row0 = m0 + warp * 32 + lane / 8;   // this lane's rows are row0 + 4 i
     const int rows_left = max(0, min(8, (pM - row0 + 3) / 4));
