@@ -8,8 +8,8 @@
 // it needs.  Every output is one chain of fused multiply-adds in the order of conv_fwd_kernel,
 // conv_dgrad_kernel and conv_wgrad_kernel (sq_gemm.cu), so the results are the same bits.
 // 512 images of 32 x 15 x 15 to 32 channels, stride 1 (floor 19.8 us at one FMA per lane and
-// cycle; before, there, and now): forward 98 and 53 us, data gradient 190 and 77 us, weight
-// gradient 375 and 105 us.
+// cycle; before, there, and now): forward 98 and 53 us, data gradient 190 and 72 us, weight
+// gradient 375 and 82 us.
 #include "sq_kernels.cuh"
 
 #include <algorithm>
@@ -26,6 +26,21 @@ __device__ __forceinline__ void copy4(float* dst, const float* src, bool valid) 
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(valid ? 4 : 0) : "memory");
 }
 __device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+
+// c += a x of two chains at once, each half rounded as fmaf rounds: one issue slot for two
+// products.
+__device__ __forceinline__ void fma_pair(uint64_t& c, uint64_t a, uint64_t x) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(x));
+}
+__device__ __forceinline__ uint64_t both(float x) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(v) : "f"(x));
+    return v;
+}
+template <int N>
+__device__ __forceinline__ float half_of(const uint64_t (&v)[N], int i) {
+    return __uint_as_float((uint32_t)(v[i / 2] >> (32 * (i % 2))));
+}
 
 // Output grid of oh x ow pixels an image; output row r reads staged rows r rs .. r rs + 2 of
 // a plane pw wide.
@@ -87,8 +102,8 @@ struct ConvF32Args {
 };
 
 // 32 P pixels x 32 output channels a CTA, P pixels (32 apart) x 8 channels a thread: at P = 4,
-// 6 shared-memory reads (4 inputs, two broadcast 16-byte weights) per 32 FMAs; the FMA pipe is
-// 46 % busy, the issue slots 77 %.
+// 6 shared-memory reads (4 inputs, two broadcast 16-byte weights) per 32 products, issued in
+// pairs (one by one: forward 53.6 us and 53.1 now, data gradient 78 and 72).
 template <int P, bool DGRAD>
 __global__ void __launch_bounds__(128) conv_f32_kernel(const __grid_constant__ ConvF32Args a) {
     SQ_KERNEL_WAIT();
@@ -156,11 +171,11 @@ __global__ void __launch_bounds__(128) conv_f32_kernel(const __grid_constant__ C
         const int img = m / px, rem = m - img * px, oy = rem / a.g.ow;
         base[i] = m < m1 ? rg.pixel(a.g, img, oy, rem - oy * a.g.ow) : 0;
     }
-    float acc[P][8];
+    uint64_t acc[P][4];   // channel pairs
 #pragma unroll
     for (int i = 0; i < P; ++i)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0;
 
     for (int st = 0; st < steps; ++st) {
         if (a.stages == 2) asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -176,14 +191,14 @@ __global__ void __launch_bounds__(128) conv_f32_kernel(const __grid_constant__ C
                 const float* row = sx + (DGRAD ? 2 - ky : ky) * a.g.pw;
 #pragma unroll
                 for (int kx = 0; kx < 3; ++kx) {
-                    const float4 w0 = *reinterpret_cast<const float4*>(sw + (ky * 3 + kx) * kWRow);
-                    const float4 w1 = *reinterpret_cast<const float4*>(sw + (ky * 3 + kx) * kWRow + 4);
-                    const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+                    const ulonglong2 w0 = *reinterpret_cast<const ulonglong2*>(sw + (ky * 3 + kx) * kWRow);
+                    const ulonglong2 w1 = *reinterpret_cast<const ulonglong2*>(sw + (ky * 3 + kx) * kWRow + 4);
+                    const uint64_t wv[4] = {w0.x, w0.y, w1.x, w1.y};
 #pragma unroll
                     for (int i = 0; i < P; ++i) {
-                        const float x = row[base[i] + (DGRAD ? 2 - kx : kx)];
+                        const uint64_t x = both(row[base[i] + (DGRAD ? 2 - kx : kx)]);
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(x, wv[j], acc[i][j]);
+                        for (int j = 0; j < 4; ++j) fma_pair(acc[i][j], wv[j], x);
                     }
                 }
             }
@@ -200,7 +215,7 @@ __global__ void __launch_bounds__(128) conv_f32_kernel(const __grid_constant__ C
             const int n = n0 + warp * 8 + j;
             if (n >= a.N) continue;
             const int64_t off = (int64_t)img * a.out_img + (int64_t)n * px + rem;
-            float v = acc[i][j];
+            float v = half_of(acc[i], j);
             if (!DGRAD) {
                 v += a.bias[n];
                 if (a.relu && !(v > 0.f)) v = 0.f;
@@ -241,138 +256,203 @@ bool launch_conv(ConvF32Args a, cudaStream_t s) {
 
 // ---------------------------------------------------------------- weight gradient
 // Split z of the pixels, CI input channels x 32 output channels a CTA: a thread owns CO output
-// channels x the nine taps of one input channel and walks the split's pixels in order.  Along
-// an output row of a stride-1 layer the taps' inputs slide: three new values a pixel.  Bound by
-// issue (half of it staging and row bookkeeping) at 1.6 warps a scheduler: the splits, which fix
-// the order of the sums, give 61 chunks x 4 groups of 8 input channels.  8 x 2 channels a thread
-// pair measured 105 us, 8 x 4 115, 4 x 2 116 (the shape above).
-constexpr int kWTile = 64;   // pixels a stage
+// channels x the nine taps of one input channel and walks the split's pixels in order, four of an
+// output row at a time.  Half of the warps stage: the copies, 4 bytes each because a plane's rows
+// have no alignment, then cost the others no issue slots (one kind of warp: 98 us for the shape
+// above, so 82).  Input rows are staged so that a group's new columns start at a multiple of four,
+// the two before them stay in registers, and the next group is read while one is multiplied; products
+// are issued in pairs of output channels (one by one 86 us).
+// What bounds it: the splits, which fix the order of the sums, leave one multiplying warp a
+// scheduler (61 chunks x 2 groups of 16 input channels), so what a row's ends cost shows; of the
+// 82 us the staging is 8.
 struct WgradF32Args {
     const float *x, *dy;
     float* work;
-    PixelGrid g;
-    int P, Cin, Cout, chunk, words;
+    int oh, ow, pw;       // output rows and columns, input columns
+    int P, Cin, Cout, chunk;
+    int nr, xrows, xp, dp, stages;   // output rows a stage; staged input rows, their pitch, pixels a row
+    uint32_t inv_pw;      // ceil(2^32 / pw)
     int64_t x_img, x_plane, y_img;
 };
 
-// NP consecutive pixels of an output row from pixel u on: all their reads, then their products.
-template <int NP, int CO, bool SLIDE, int DROW>
-__device__ __forceinline__ void pixels(float (&acc)[CO][9], float (&bacc)[CO], bool bias, float (&edge)[3][2],
-                                       const float* row, const float* drow, int u, const PixelGrid& g) {
-    float x[NP][9], d[NP][CO];
+// Four pixels of an output row: the input columns under their taps, and CO channels' gradients.
+// Input column c of a row is staged at c + SHIFT, so that the columns new to a group start at a
+// multiple of four; the E before them are the previous group's last, or at a row's start read.
+template <int CO, int RS>
+struct PixelGroup {
+    static constexpr int E = 3 - RS, SHIFT = 4 - E, NEW = 4 * RS, DROW = CO == 4 ? 36 : 34;
+    float x[3][E + NEW];
+    uint64_t d[4][CO / 2];
+    __device__ __forceinline__ void load(const float* xs, int pitch, const float* ds, bool start, const PixelGroup& prev) {
 #pragma unroll
-    for (int v = 0; v < NP; ++v) {
-        const float* dp = drow + (u + v) * DROW;
-        if (CO == 4) {
-            const float4 t = *reinterpret_cast<const float4*>(dp);
-            d[v][0] = t.x; d[v][1] = t.y; d[v][2 % CO] = t.z; d[v][3 % CO] = t.w;
-        } else {
-            const float2 t = *reinterpret_cast<const float2*>(dp);
-            d[v][0] = t.x; d[v][1] = t.y;
+        for (int ky = 0; ky < 3; ++ky) {
+            const float* r = xs + ky * pitch;
+#pragma unroll
+            for (int c = 0; c < NEW; c += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(r + 4 + c);
+                x[ky][E + c] = v.x; x[ky][E + c + 1] = v.y; x[ky][E + c + 2] = v.z; x[ky][E + c + 3] = v.w;
+            }
+#pragma unroll
+            for (int e = 0; e < E; ++e) x[ky][e] = start ? r[SHIFT + e] : prev.x[ky][NEW + e];
         }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            if (CO == 4) {
+                const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(ds + v * DROW);
+                d[v][0] = t.x; d[v][CO / 2 - 1] = t.y;
+            } else {
+                d[v][0] = *reinterpret_cast<const uint64_t*>(ds + v * DROW);
+            }
+        }
+    }
+    // pixels LO .. HI - 1 of the group
+    template <int LO, int HI>
+    __device__ __forceinline__ void multiply(uint64_t (&acc)[CO / 2][9], float (&bacc)[CO], bool bias) const {
+        uint64_t xx[3][E + NEW];
 #pragma unroll
         for (int ky = 0; ky < 3; ++ky)
 #pragma unroll
-            for (int kx = SLIDE ? 2 : 0; kx < 3; ++kx) x[v][ky * 3 + kx] = row[ky * g.pw + (u + v) * g.rs + kx];
-    }
-    if (SLIDE) {
+            for (int c = 0; c < E + NEW; ++c) xx[ky][c] = both(x[ky][c]);
 #pragma unroll
-        for (int ky = 0; ky < 3; ++ky) {
+        for (int v = LO; v < HI; ++v) {
 #pragma unroll
-            for (int v = 0; v < NP; ++v) {
-                x[v][ky * 3] = v >= 2 ? x[v >= 2 ? v - 2 : 0][ky * 3 + 2] : edge[ky][v >= 2 ? 0 : v];
-                x[v][ky * 3 + 1] = v >= 1 ? x[v >= 1 ? v - 1 : 0][ky * 3 + 2] : edge[ky][1];
-            }
-            edge[ky][0] = NP >= 2 ? x[NP >= 2 ? NP - 2 : 0][ky * 3 + 2] : edge[ky][1];
-            edge[ky][1] = x[NP - 1][ky * 3 + 2];
+            for (int k = 0; k < CO / 2; ++k)
+#pragma unroll
+                for (int r = 0; r < 9; ++r) fma_pair(acc[k][r], d[v][k], xx[r / 3][v * RS + r % 3]);
+            if (bias)
+#pragma unroll
+                for (int k = 0; k < CO; ++k) bacc[k] += half_of(d[v], k);
         }
     }
-#pragma unroll
-    for (int v = 0; v < NP; ++v) {
-#pragma unroll
-        for (int k = 0; k < CO; ++k)
-#pragma unroll
-            for (int r = 0; r < 9; ++r) acc[k][r] = fmaf(d[v][k], x[v][r], acc[k][r]);
-        if (bias)
-#pragma unroll
-            for (int k = 0; k < CO; ++k) bacc[k] += d[v][k];
-    }
-}
+};
 
-template <int CI, int CO, bool SLIDE>
-__global__ void __launch_bounds__(CI * 32 / CO) wgrad_f32_kernel(const __grid_constant__ WgradF32Args a) {
-    static_assert(CI * 32 / CO % kWTile == 0, "whole pixels a pass");
-    constexpr int NT = CI * 32 / CO, DROW = CO == 4 ? 36 : 34;
+template <int CI, int CO, int RS>
+__global__ void __launch_bounds__(2 * CI * 32 / CO) wgrad_f32_kernel(const __grid_constant__ WgradF32Args a) {
+    using Group = PixelGroup<CO, RS>;
+    constexpr int NT = CI * 32 / CO, NW = NT / 32, DROW = Group::DROW;
     SQ_KERNEL_WAIT();
     extern __shared__ __align__(16) float smem[];
-    const int tid = threadIdx.x, cg = tid % (32 / CO), ci_l = tid / (32 / CO);
+    const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
+    const int cg = tid % (32 / CO), ci = tid / (32 / CO);
     const int c0 = blockIdx.x * CI, co0 = blockIdx.y * 32, nci = min(CI, a.Cin - c0);
     const int p_begin = blockIdx.z * a.chunk, p_end = min(a.P, p_begin + a.chunk);
-    const int px = a.g.oh * a.g.ow;
-    const int stage_words = kWTile * DROW + (CI * a.words + 3) / 4 * 4;
+    const int px = a.oh * a.ow;
+    // rows of the flattened (image, row) order that hold the split's pixels
+    const int g_begin = p_begin / a.ow, g_end = p_end > p_begin ? (p_end - 1) / a.ow + 1 : g_begin;
+    const int tiles = (g_end - g_begin + a.nr - 1) / a.nr;
+    const int full = (a.oh - 1) * RS + 3;
+    const int x_words = a.xrows * a.xp, stage_words = CI * x_words + (a.nr * a.dp + 4) * DROW;
     auto stage = [&](int t) {
-        const int q0 = p_begin + t * kWTile, q1 = min(p_end, q0 + kWTile);
-        if (q0 < q1) {
-            float* sd = smem + (t & 1) * stage_words;
-            float* sx = sd + kWTile * DROW;
-            // a thread copies one pixel's gradients of every NT / kWTile-th channel
-            const int pl = tid % kWTile, p = q0 + pl, img = p / px;
-            const float* src = a.dy + (int64_t)img * a.y_img + (int64_t)co0 * px + (p - img * px);
-            float* dst = sd + pl * DROW;
+        if (t < tiles) {
+            float* sx = smem + (t % a.stages) * stage_words;
+            float* sd = sx + CI * x_words;
+            const int r0 = g_begin + t * a.nr, r1 = min(g_end, r0 + a.nr);
+            // gradients: a lane's pixels, every NW-th output channel
+            for (int l = lane; l < (r1 - r0) * a.ow; l += 32) {
+                const int p = r0 * a.ow + l, img = p / px;
+                if (p < p_begin || p >= p_end) continue;
+                const int row = l / a.ow, col = l - row * a.ow;
+                const float* src = a.dy + (int64_t)img * a.y_img + (int64_t)co0 * px + (p - img * px);
+                float* dst = sd + (row * a.dp + col) * DROW;
 #pragma unroll 4
-            for (int co = tid / kWTile; co < 32; co += NT / kWTile) {
-                const bool ok = p < q1 && co0 + co < a.Cout;
-                copy4(dst + co, ok ? src + (int64_t)co * px : a.dy, ok);
+                for (int co = warp - NW; co < 32; co += NW)
+                    if (co0 + co < a.Cout) copy4(dst + co, src + (int64_t)co * px, true);
             }
-            const Region rg(a.g, q0, q1);
-            const float* x0 = a.x + (int64_t)rg.img0 * a.x_img + (int64_t)c0 * a.x_plane;
-            for (int w = tid; w < rg.words; w += NT) {
-                int img, row, col;
-                rg.place(a.g, w, img, row, col);
-                const float* xs = x0 + (int64_t)img * a.x_img + (int64_t)row * a.g.pw + col;
-#pragma unroll 4
-                for (int c = 0; c < nci; ++c) copy4(sx + c * a.words + w, xs + c * a.x_plane, true);
+            // input rows: of the first image from its first output row on, of the others from 0
+            const int img0 = r0 / a.oh, oy0 = r0 - img0 * a.oh, n0 = min(r1 - r0, a.oh - oy0), rest = r1 - r0 - n0;
+            const int first = (n0 - 1) * RS + 3, last = rest % a.oh;
+            const int rows = first + rest / a.oh * full + (last ? (last - 1) * RS + 3 : 0);
+            const float* x0 = a.x + (int64_t)img0 * a.x_img + (int64_t)c0 * a.x_plane;
+            for (int w = tid - NT; w < rows * a.pw; w += NT) {
+                const int r = __umulhi(w, a.inv_pw), col = w - r * a.pw;
+                const float* src = x0;
+                if (r < first) {
+                    src += (oy0 * RS + r) * a.pw + col;
+                } else {
+                    const int q = (r - first) / full;
+                    src += (q + 1) * a.x_img + (r - first - q * full) * a.pw + col;
+                }
+                float* dst = sx + r * a.xp + col + Group::SHIFT;
+#pragma unroll
+                for (int c = 0; c < CI; ++c)
+                    if (c < nci) copy4(dst + c * x_words, src + c * a.x_plane, true);
             }
         }
         copies_commit();
     };
-    float acc[CO][9], bacc[CO];
+    if (warp >= NW) {
+        for (int st = 0; st + 1 < a.stages; ++st) stage(st);
+        for (int t = 0; t < tiles; ++t) {
+            if (a.stages == 2) asm volatile("cp.async.wait_group 0;" ::: "memory");
+            else asm volatile("cp.async.wait_group 1;" ::: "memory");
+            __syncthreads();   // this stage has landed, the previous one has been read
+            stage(t + a.stages - 1);
+        }
+        SQ_KERNEL_TRIGGER();
+        return;
+    }
+    uint64_t acc[CO / 2][9];
+    float bacc[CO];
+    const bool bias = blockIdx.x == 0;
 #pragma unroll
     for (int k = 0; k < CO; ++k) {
         bacc[k] = 0.f;
 #pragma unroll
-        for (int r = 0; r < 9; ++r) acc[k][r] = 0.f;
+        for (int r = 0; r < 9; ++r) acc[k / 2][r] = 0;
     }
-    const bool bias = blockIdx.x == 0;
-    const int tiles = (p_end - p_begin + kWTile - 1) / kWTile;
-    stage(0);
     for (int t = 0; t < tiles; ++t) {
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();   // this stage has landed, the other one has been read
-        stage(t + 1);
-        const float* sd = smem + (t & 1) * stage_words + cg * CO;
-        const float* sx = smem + (t & 1) * stage_words + kWTile * DROW + (ci_l < nci ? ci_l : 0) * a.words;
-        const int q0 = p_begin + t * kWTile, q1 = min(p_end, q0 + kWTile);
-        const Region rg(a.g, q0, q1);
-        int img = rg.img0, oy = rg.row0, ox = (q0 - img * px) - oy * a.g.ow;
-        for (int q = q0; q < q1;) {   // one run of pixels of an output row
-            const int run = min(a.g.ow - ox, q1 - q);
-            const float* row = sx + rg.pixel(a.g, img, oy, ox);
-            const float* drow = sd + (q - q0) * DROW;
-            float edge[3][2];   // the first two columns of the next pixel's taps
-            if (SLIDE) {
-#pragma unroll
-                for (int ky = 0; ky < 3; ++ky) {
-                    edge[ky][0] = row[ky * a.g.pw];
-                    edge[ky][1] = row[ky * a.g.pw + 1];
-                }
+        __syncthreads();
+        const float* xrow = smem + (t % a.stages) * stage_words + ci * x_words;
+        const float* drow = smem + (t % a.stages) * stage_words + CI * x_words + cg * CO;
+        const int r1 = min(g_end, g_begin + (t + 1) * a.nr);
+        int g = g_begin + t * a.nr, oy = g % a.oh;
+        Group ga, gb;
+        ga.load(xrow, a.xp, drow, true, ga);
+        for (; g < r1; ++g) {
+            // pixels [lo, hi) of the row: all but in the split's first and last row
+            const int lo = max(0, p_begin - g * a.ow), hi = min(a.ow, p_end - g * a.ow);
+            int q = lo / 4;
+            const float* xq = xrow + 4 * RS * q;
+            const float* dq = drow + 4 * q * DROW;
+            if (lo) {
+                ga.load(xq, a.xp, dq, true, ga);
+                gb.load(xq + 4 * RS, a.xp, dq + 4 * DROW, false, ga);
+                const int l = lo - 4 * q, h = hi - 4 * q;
+                if (l <= 0 && h > 0) ga.template multiply<0, 1>(acc, bacc, bias);
+                if (l <= 1 && h > 1) ga.template multiply<1, 2>(acc, bacc, bias);
+                if (l <= 2 && h > 2) ga.template multiply<2, 3>(acc, bacc, bias);
+                if (h > 3) ga.template multiply<3, 4>(acc, bacc, bias);
+                ga = gb;
+                ++q;
+                xq += 4 * RS;
+                dq += 4 * DROW;
             }
-            int u = 0;
-            for (; u + 4 <= run; u += 4) pixels<4, CO, SLIDE, DROW>(acc, bacc, bias, edge, row, drow, u, a.g);
-            for (; u < run; ++u) pixels<1, CO, SLIDE, DROW>(acc, bacc, bias, edge, row, drow, u, a.g);
-            q += run;
-            ox = 0;
-            if (++oy == a.g.oh) { oy = 0; ++img; }
+            const int whole = hi / 4;
+            for (; q + 1 < whole; q += 2) {
+                gb.load(xq + 4 * RS, a.xp, dq + 4 * DROW, false, ga);
+                ga.template multiply<0, 4>(acc, bacc, bias);
+                xq += 8 * RS;
+                dq += 8 * DROW;
+                ga.load(xq, a.xp, dq, false, gb);
+                gb.template multiply<0, 4>(acc, bacc, bias);
+            }
+            if (q < whole) {
+                gb.load(xq + 4 * RS, a.xp, dq + 4 * DROW, false, ga);
+                ga.template multiply<0, 4>(acc, bacc, bias);
+                ga = gb;
+                ++q;
+            }
+            oy = oy + 1 == a.oh ? 0 : oy + 1;
+            if (g + 1 < r1) {
+                xrow += (oy ? RS : 3) * a.xp;
+                drow += a.dp * DROW;
+            }
+            gb.load(xrow, a.xp, drow, true, ga);
+            const int left = hi - 4 * q;
+            if (left > 0) ga.template multiply<0, 1>(acc, bacc, bias);
+            if (left > 1) ga.template multiply<1, 2>(acc, bacc, bias);
+            if (left > 2) ga.template multiply<2, 3>(acc, bacc, bias);
+            ga = gb;
         }
     }
     SQ_KERNEL_TRIGGER();
@@ -382,24 +462,33 @@ __global__ void __launch_bounds__(CI * 32 / CO) wgrad_f32_kernel(const __grid_co
     for (int k = 0; k < CO; ++k) {
         const int co = co0 + cg * CO + k;
         if (co >= a.Cout) continue;
-        if (ci_l < nci) {
+        if (ci < nci) {
 #pragma unroll
-            for (int r = 0; r < 9; ++r) out[(int64_t)co * N + (c0 + ci_l) * 9 + r] = acc[k][r];
+            for (int r = 0; r < 9; ++r)
+                out[(int64_t)co * N + (c0 + ci) * 9 + r] = __uint_as_float((uint32_t)(acc[k / 2][r] >> (32 * (k % 2))));
         }
-        if (bias && ci_l == 0) out[(int64_t)co * N + N - 1] = bacc[k];
+        if (bias && ci == 0) out[(int64_t)co * N + N - 1] = bacc[k];
     }
 }
 
-template <int CI, int CO, bool SLIDE>
+template <int CI, int CO, int RS>
 bool launch_wgrad(WgradF32Args a, int splits, cudaStream_t s) {
-    constexpr int DROW = CO == 4 ? 36 : 34;
-    const int64_t words = region_words(a.g, kWTile);
-    const int64_t bytes = 8 * (kWTile * DROW + (CI * words + 3) / 4 * 4);
-    if (bytes > kSmemBytes) return false;
-    a.words = (int)words;
-    launch_with(false, wgrad_f32_kernel<CI, CO, SLIDE>, dim3((a.Cin + CI - 1) / CI, (a.Cout + 31) / 32, splits), dim3(CI * 32 / CO),
-             (size_t)bytes, s, a);
-    return true;
+    using Group = PixelGroup<CO, RS>;
+    a.dp = (a.ow + 3) / 4 * 4;
+    a.xp = std::max(a.dp * RS + 4, (a.pw + Group::SHIFT + 3) / 4 * 4);
+    a.inv_pw = (uint32_t)(((1ULL << 32) + a.pw - 1) / a.pw);
+    // about 64 pixels a stage
+    for (a.nr = std::max(1, std::min(8, 64 / a.ow)); a.nr >= 1; --a.nr) {
+        const int pieces = (a.nr - 1 + a.oh - 1) / a.oh + 1;
+        a.xrows = a.nr * RS + std::max(0, 3 - RS) * pieces;
+        const int64_t stage = 4 * ((int64_t)CI * a.xrows * a.xp + (int64_t)(a.nr * a.dp + 4) * Group::DROW);
+        a.stages = 3 * stage <= kSmemBytes ? 3 : 2;
+        if (a.stages * stage > kSmemBytes) continue;
+        launch_with(false, wgrad_f32_kernel<CI, CO, RS>, dim3((a.Cin + CI - 1) / CI, (a.Cout + 31) / 32, splits), dim3(2 * CI * 32 / CO),
+                    (size_t)(a.stages * stage), s, a);
+        return true;
+    }
+    return false;
 }
 
 }  // namespace
@@ -430,11 +519,18 @@ bool launch_conv_wgrad_partials_f32(const ConvShape& sh, const float* dy, const 
                                     int chunk, cudaStream_t s) {
     WgradF32Args a{};
     a.x = x; a.dy = dy; a.work = work;
-    a.g = PixelGrid{sh.OH, sh.OW, sh.stride, sh.W};
+    a.oh = sh.OH; a.ow = sh.OW; a.pw = sh.W;
     a.P = sh.nimg * sh.OH * sh.OW; a.Cin = sh.Cin; a.Cout = sh.Cout; a.chunk = chunk;
     a.x_img = sh.x_img_stride; a.x_plane = (int64_t)sh.H * sh.W; a.y_img = sh.y_img_stride;
-    if (sh.stride == 1) return sh.Cin > 4 ? launch_wgrad<8, 2, true>(a, splits, s) : launch_wgrad<4, 2, true>(a, splits, s);
-    return sh.Cin > 4 ? launch_wgrad<8, 2, false>(a, splits, s) : launch_wgrad<4, 2, false>(a, splits, s);
+    // 512 images of 13 x 13 and 11 x 11, 32 channels: 62 and 47 us by 16 x 4, 66 and 47 by 8 x 2; of
+    // 16 channels 7 x 7: 14.6 and 12.6; 70 of 3 x 3, 2 channels: 17.5 by 8 x 2, 16.6 by 4 x 2.
+    // Wider strides take conv_wgrad_kernel.
+    if (sh.stride == 1) {
+        if (sh.Cin > 16) return launch_wgrad<16, 4, 1>(a, splits, s);
+        return sh.Cin > 4 ? launch_wgrad<8, 2, 1>(a, splits, s) : launch_wgrad<4, 2, 1>(a, splits, s);
+    }
+    if (sh.stride == 2) return sh.Cin > 4 ? launch_wgrad<8, 2, 2>(a, splits, s) : launch_wgrad<4, 2, 2>(a, splits, s);
+    return false;
 }
 
 }  // namespace sq
