@@ -217,6 +217,22 @@ __device__ __forceinline__ bool bulk_load_wait(uint64_t* bar, uint32_t parity) {
     }
 }
 
+// c += a x of two chains at once, each half rounded as fmaf rounds: one issue slot for two
+// products.
+__device__ __forceinline__ void fma_pair(uint64_t& c, uint64_t a, uint64_t x) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(x));
+}
+__device__ __forceinline__ uint64_t both(float x) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(v) : "f"(x));
+    return v;
+}
+__device__ __forceinline__ uint64_t pair(float lo, float hi) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+
 // One lane of the (converged) calling warp, the same one at every call.  Issue loops branch on
 // the warp (made uniform by warp_uniform) and then on this predicate: descriptors and loop
 // counters then stay in uniform registers, where a branch on the thread index moves every

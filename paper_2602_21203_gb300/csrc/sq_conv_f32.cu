@@ -27,16 +27,6 @@ __device__ __forceinline__ void copy4(float* dst, const float* src, bool valid) 
 }
 __device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 
-// c += a x of two chains at once, each half rounded as fmaf rounds: one issue slot for two
-// products.
-__device__ __forceinline__ void fma_pair(uint64_t& c, uint64_t a, uint64_t x) {
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(x));
-}
-__device__ __forceinline__ uint64_t both(float x) {
-    uint64_t v;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(v) : "f"(x));
-    return v;
-}
 template <int N>
 __device__ __forceinline__ float half_of(const uint64_t (&v)[N], int i) {
     return __uint_as_float((uint32_t)(v[i / 2] >> (32 * (i % 2))));

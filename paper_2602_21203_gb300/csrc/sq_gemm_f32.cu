@@ -2,8 +2,8 @@
 // layer's forward, data gradient and weight gradient).
 //
 // What bounds it: at the training shape, shared-memory fragment reads beside the FMAs (8
-// 16-byte reads per 64 FMAs, two warps a scheduler: the FMA pipe 32 % busy); at the small
-// ones, the latency of one CTA's pass over K.  Operand tiles come in by cp.async
+// 16-byte reads, 4 cycles of the SM's read path each, per 64 FMAs of a scheduler; two warps a
+// scheduler, the FMA pipe 32 % busy); at the small ones, the latency of one CTA's pass over K.  Operand tiles come in by cp.async
 // into a ring of kStages shared-memory stages, so global latency overlaps the arithmetic;
 // both are staged in their memory order (K-contiguous rows, or rows of M / N), so no
 // transposing pass is needed, and a thread reads 16-byte fragments: four K steps of a row
@@ -12,7 +12,10 @@
 // on the tile nor on the rest of the batch, and equal those of gemm_kernel (sq_gemm.cu),
 // which stages synchronously: M = N = K = 512 twice 50.4 us there, 20.5 here (floor 6.7 at
 // one FMA per lane and cycle), the projections' 2048 x 256 x 2592 244 and 91 us (floor 33.7),
-// M 32, N 256, K 412 twice 39.7 and 5.9 us.
+// M 32, N 256, K 412 twice 39.7 and 5.9 us.  Where B's rows are contiguous in n, a read brings
+// column pairs and products are issued in pairs: M 512, N 2592, K 256 32.8 us one by one and
+// 24.7 in pairs, N = K = 512 twice 22.6 and 20.6 (where they are contiguous in k the pairs would
+// have to be put together: 22.6 and 28.8).
 #include "sq_kernels.cuh"
 
 #include <algorithm>
@@ -184,11 +187,15 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) gemm_f32_kernel(const _
 #pragma unroll
     for (int st = 0; st < kStages; ++st) stage(st);
 
-    float acc[TM][TN];
+    float acc[TM][TN];      // B's rows contiguous in k
+    uint64_t acc2[TM][TN / 2];   // in n: column pairs
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+        for (int j = 0; j < TN; ++j) {
+            acc[i][j] = 0.f;
+            acc2[i][j / 2] = 0;
+        }
 
     asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 1) : "memory");
     __syncthreads();
@@ -218,7 +225,10 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) gemm_f32_kernel(const _
 #pragma unroll
                 for (int i = 0; i < TM; ++i)
 #pragma unroll
-                    for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[k4 % 2][i][kk], b[k4 % 2][j][kk], acc[i][j]);
+                    for (int j = 0; j < TN; ++j) {
+                        if (B_K) acc[i][j] = fmaf(a[k4 % 2][i][kk], b[k4 % 2][j][kk], acc[i][j]);
+                        else if (j % 2) fma_pair(acc2[i][j / 2], pair(b[k4 % 2][j - 1][kk], b[k4 % 2][j][kk]), both(a[k4 % 2][i][kk]));
+                    }
         }
         slot = next_slot;
     }
@@ -235,7 +245,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) gemm_f32_kernel(const _
         for (int j = 0; j < TN; ++j) {
             const int n = n0 + tile_row<B_K, BN, TN>(tx, j);
             if (n >= P.N) continue;
-            float v = acc[i][j];
+            float v = B_K ? acc[i][j] : __uint_as_float((uint32_t)(acc2[i][j / 2] >> (32 * (j % 2))));
             if (bias) v += bias[n];
             if (mask && !(mask[(int64_t)m * P.sm_m + (int64_t)n * P.sm_n] > 0.f)) v = 0.f;
             float* dst = C + (int64_t)m * P.sc_m + (int64_t)n * P.sc_n;
