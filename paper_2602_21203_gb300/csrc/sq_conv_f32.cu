@@ -94,11 +94,14 @@ struct ConvF32Args {
 // 32 P pixels x 32 output channels a CTA, P pixels (32 apart) x 8 channels a thread: at P = 4,
 // 6 shared-memory reads (4 inputs, two broadcast 16-byte weights) per 32 products, issued in
 // pairs (one by one: forward 53.6 us and 53.1 now, data gradient 78 and 72).
-template <int P, bool DGRAD>
-__global__ void __launch_bounds__(128) conv_f32_kernel(const __grid_constant__ ConvF32Args a) {
+// COPY threads stage, as in the weight gradient, beside those that multiply; with none all do both.
+// A small grid runs faster with them (32 images of 16 x 7 x 7, P = 1: forward 8.0 and 5.8 us, data
+// gradient 10.6 and 7.6), a full one has other warps to issue meanwhile (P = 4: 53 and 58 us).
+template <int P, int COPY, bool DGRAD>
+__global__ void __launch_bounds__(128 + COPY) conv_f32_kernel(const __grid_constant__ ConvF32Args a) {
     SQ_KERNEL_WAIT();
     extern __shared__ __align__(16) float smem[];
-    const int nt = blockDim.x, tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
+    const int nt = blockDim.x, nm = nt - COPY, tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
     const int m0 = blockIdx.x * 32 * P, m1 = min(a.M, m0 + 32 * P), n0 = blockIdx.y * 32;
     const Region rg(a.g, m0, m1);
     const int xwords = kChan * a.words, stage_words = kChan * 9 * kWRow + (xwords + 3) / 4 * 4;
@@ -119,12 +122,13 @@ __global__ void __launch_bounds__(128) conv_f32_kernel(const __grid_constant__ C
     __syncthreads();
     const float* in0 = a.in + (int64_t)rg.img0 * a.in_img;
     const int steps = (a.R + kChan - 1) / kChan;
+    const int ct = COPY ? tid - nm : tid, nc_t = COPY ? COPY : nt;   // place among the staging threads, their number
     auto stage = [&](int st) {
         if (st < steps) {
             float* sw = smem + (st % a.stages) * stage_words;
             float* sx = sw + kChan * 9 * kWRow;
             const int c0 = st * kChan, nc = min(kChan, a.R - c0);
-            for (int e = tid; e < kChan * 9 * 32; e += nt) {
+            for (int e = ct; e < kChan * 9 * 32; e += nc_t) {
                 int n, k;
                 const float* src;
                 if (!DGRAD) {
@@ -141,7 +145,7 @@ __global__ void __launch_bounds__(128) conv_f32_kernel(const __grid_constant__ C
                 copy4(sw + k * kWRow + n, ok ? src : a.w, ok);
             }
             const float* src0 = in0 + (int64_t)c0 * a.in_plane;
-            for (int w = tid; w < rg.words; w += nt) {
+            for (int w = ct; w < rg.words; w += nc_t) {
                 const int off = woff[w];
                 const float* src = src0 + (off < 0 ? 0 : off);
 #pragma unroll
@@ -151,7 +155,19 @@ __global__ void __launch_bounds__(128) conv_f32_kernel(const __grid_constant__ C
         }
         copies_commit();
     };
-    for (int st = 0; st + 1 < a.stages; ++st) stage(st);
+    auto next_stage = [&](int st) {
+        if (a.stages == 2) asm volatile("cp.async.wait_group 0;" ::: "memory");
+        else asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();   // this stage has landed, the previous one has been read
+        stage(st + a.stages - 1);
+    };
+    if (!COPY || tid >= nm)
+        for (int st = 0; st + 1 < a.stages; ++st) stage(st);
+    if (COPY && tid >= nm) {
+        for (int st = 0; st < steps; ++st) next_stage(st);
+        SQ_KERNEL_TRIGGER();
+        return;
+    }
 
     int base[P];
     const int px = a.g.oh * a.g.ow;
@@ -168,10 +184,8 @@ __global__ void __launch_bounds__(128) conv_f32_kernel(const __grid_constant__ C
         for (int j = 0; j < 4; ++j) acc[i][j] = 0;
 
     for (int st = 0; st < steps; ++st) {
-        if (a.stages == 2) asm volatile("cp.async.wait_group 0;" ::: "memory");
-        else asm volatile("cp.async.wait_group 1;" ::: "memory");
-        __syncthreads();   // this stage has landed, the previous one has been read
-        stage(st + a.stages - 1);
+        if (COPY) __syncthreads();
+        else next_stage(st);
         const float* sw = smem + (st % a.stages) * stage_words + warp * 8;
         const float* sx = smem + (st % a.stages) * stage_words + kChan * 9 * kWRow;
         const int nc = min(kChan, a.R - st * kChan);
@@ -221,7 +235,7 @@ template <bool DGRAD>
 bool launch_conv(ConvF32Args a, cudaStream_t s) {
     const int ny = (a.N + 31) / 32, threads = 32 * std::min(4, (a.N + 7) / 8);
     // P: 53 us at 4, 57 at 8, 62 at 2, 88 at 1 for the shape above; fewer pixels a thread where
-    // the CTAs would not fill two per SM (32 images of 16 x 7 x 7: 13.2, 9.4 and 8.0 us at 4, 2, 1)
+    // the CTAs would not fill two per SM (32 images of 16 x 7 x 7: 13.2, 7.2 and 5.8 us at 4, 2, 1)
     int p = 4;
     while (p > 1 && (int64_t)((a.M + 32 * p - 1) / (32 * p)) * ny < 2 * 152) p /= 2;
     for (; p >= 1; p /= 2) {
@@ -233,11 +247,11 @@ bool launch_conv(ConvF32Args a, cudaStream_t s) {
         a.stages = 3 * stage + table <= kSmemBytes ? 3 : 2;
         const int64_t bytes = a.stages * stage + table;
         if (bytes > kSmemBytes) continue;
-        const dim3 grid((a.M + 32 * p - 1) / (32 * p), ny), block(threads);
+        const dim3 grid((a.M + 32 * p - 1) / (32 * p), ny), block(threads + (p < 4 ? 128 : 0));
         switch (p) {
-            case 4: launch_k(conv_f32_kernel<4, DGRAD>, grid, block, (size_t)bytes, s, a); break;
-            case 2: launch_k(conv_f32_kernel<2, DGRAD>, grid, block, (size_t)bytes, s, a); break;
-            default: launch_k(conv_f32_kernel<1, DGRAD>, grid, block, (size_t)bytes, s, a); break;
+            case 4: launch_k(conv_f32_kernel<4, 0, DGRAD>, grid, block, (size_t)bytes, s, a); break;
+            case 2: launch_k(conv_f32_kernel<2, 128, DGRAD>, grid, block, (size_t)bytes, s, a); break;
+            default: launch_k(conv_f32_kernel<1, 128, DGRAD>, grid, block, (size_t)bytes, s, a); break;
         }
         return true;
     }
