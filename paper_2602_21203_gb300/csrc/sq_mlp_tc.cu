@@ -12,10 +12,12 @@
 //                     slabs through a shared-memory ring (mbarrier complete_tx)
 //   warp 0 / lane 0   MMA issuer: tcgen05.mma M = 128, N = NS (K = 16 per step) from
 //                     the activation region and the ring into tensor memory
-//   warps 0-3         epilogue, one thread per row: bias, LayerNorm statistics over the
-//                     whole row (each CTA's mean and centred sum of squares of its slice,
-//                     sent to every CTA of the cluster with st.async and combined in rank
-//                     order), ReLU; the BF16 result is written into this CTA's activation
+//   warps 0-3, 5-8    epilogue, two threads per row: bias, LayerNorm statistics over the
+//                     whole row (a sum in column order, so the first thread's work alone;
+//                     each CTA's mean and centred sum of squares of its slice, sent to
+//                     every CTA of the cluster with st.async and combined in rank order),
+//                     then half of the columns each: ReLU; the BF16 result is written into
+//                     this CTA's activation
 //                     region as the next layer's A operand and copied to the other CTAs of
 //                     the cluster with one shared-to-shared bulk copy each; saved FP32
 //                     activations leave through a per-warp transpose as coalesced rows,
@@ -28,6 +30,10 @@
 // Data that crosses CTAs travels by st.async and bulk copies that complete transaction
 // bytes on the receiver's mbarrier, so no cluster-scope fence or cluster-wide barrier is
 // needed between the layers, and the producer streams ahead undisturbed.
+// What bounds it: a chain of latencies at one CTA per SM.  Of the 40,000 cycles of M 512, kin 268,
+// H 512, nout 12 the copies between the CTAs (14 bytes a cycle into an SM) and the second layer's
+// products take 9,000, the first layer's operands 4,000, the statistics and their exchange 4,000
+// a layer.  One thread per row: 20.2 us (nout 101 twice 24.2, M 4096 22.3), two: 18.8 (22.5, 21.0).
 // Every wait is bounded; past the limit the waiting thread records a code in *err and
 // gives up, the CTA waits (bounded) for its copies in flight, frees its tensor memory and
 // returns.
@@ -47,7 +53,8 @@ namespace {
 constexpr int BM = 128;
 constexpr int SLAB = 64;                  // K elements per slab (128 bytes of BF16)
 constexpr int SLAB_BYTES = BM * 128;      // one activation slab: 128 rows x 128 B
-constexpr int kThreads = 160;
+constexpr int kThreads = 160;              // backward: an epilogue thread a row
+constexpr int kFwdThreads = 288;           // forward: two a row
 constexpr int STG_LD = 36;                // staging row stride (floats)
 constexpr int STG_BYTES = 4 * 32 * STG_LD * 4;
 constexpr int SMEM_LIMIT = 232448;
@@ -146,7 +153,13 @@ __device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
+// The end of a kernel: no CTA passes before all have arrived.  Orders no memory: what peers sent
+// has completed on this CTA's barriers.
+__device__ __forceinline__ void cluster_leave() {
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+__device__ __forceinline__ void fwd_bar() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 // Two floats into shared memory of a cluster CTA, completing 8 bytes of transaction count
 // on the barrier `bar` (a shared::cluster address in that CTA).
 __device__ __forceinline__ void st_async_v2(uint32_t addr, float x, float y, uint32_t bar) {
@@ -247,7 +260,28 @@ __device__ __forceinline__ void store_rows_coalesced(float* stg, const float (&v
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_constant__ MlpArgs a) {
+// The same for the forward, whose eight epilogue warps share the staging space: 16 columns at a
+// time, 16-byte units placed so that neither the rows written nor those read meet in a bank.
+__device__ __forceinline__ void store_rows_coalesced16(float* stg, const float (&v)[32], float* dst, int64_t ld,
+                                                       int row0, int M, int col, int lane) {
+#pragma unroll
+    for (int h = 0; h < 32; h += 16) {
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            *reinterpret_cast<float4*>(stg + lane * 16 + 4 * (j ^ (lane / 2 % 4))) =
+                make_float4(v[h + 4 * j], v[h + 4 * j + 1], v[h + 4 * j + 2], v[h + 4 * j + 3]);
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int rr = 8 * i + lane / 4;
+            const float4 x = *reinterpret_cast<const float4*>(stg + rr * 16 + 4 * (lane % 4 ^ (rr / 2 % 4)));
+            if (row0 + rr < M) *reinterpret_cast<float4*>(dst + (int64_t)(row0 + rr) * ld + col + h + 4 * (lane % 4)) = x;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kFwdThreads, 1) mlp_tc_kernel(const __grid_constant__ MlpArgs a) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int S = a.stages;
@@ -345,24 +379,30 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
             slot[1] = it;
         }
     } else {
-        const int r = warp * 32 + lane;                 // row of the block = tensor-memory lane
-        const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
+        // a warp reaches the 32 tensor-memory lanes of its number modulo 4; the second set of four
+        // warps takes the later half of the columns
+        const int quad = warp % 4, set = warp > 4 ? 1 : 0;
+        const int r = quad * 32 + lane;                 // row of the block = tensor-memory lane
+        const int et = set * 128 + r;
+        const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
+        const int c_mid = (NS / 32 + 1) / 2 * 32, c_lo = set ? c_mid : 0, c_hi = set ? NS : c_mid;
         // this CTA's slices of the bias, LayerNorm gain and shift of every hidden layer, and
-        // the output bias, staged by warps 1-3 while the first layer's operands arrive (the
-        // first epilogue's barrier orders them before any use)
+        // the output bias, staged by the warps that issue nothing while the first layer's operands
+        // arrive (the first epilogue's barrier orders them before any use)
         if (warp > 0) {
-            for (int i = threadIdx.x - 32; i < nh * 3 * NS; i += 96) {
+            const int t0 = set ? threadIdx.x - 64 : threadIdx.x - 32;
+            for (int i = t0; i < nh * 3 * NS; i += 224) {
                 const int l = i / (3 * NS), k = (i % (3 * NS)) / NS, j = i % NS;
                 const float* src = k == 0 ? P.bias[l] : (k == 1 ? P.g[l] : P.beta[l]);
                 par[i] = src[rank * NS + j];
             }
-            for (int j = threadIdx.x - 32; j < nop; j += 96) par[nh * 3 * NS + j] = j < a.nout ? P.bias[nh][j] : 0.f;
+            for (int j = t0; j < nop; j += 224) par[nh * 3 * NS + j] = j < a.nout ? P.bias[nh][j] : 0.f;
         }
         // the problem's output pointers, read once: P is reached through a generic pointer
         // into the parameter block, which the compiler would re-read after every store
         float* const p_out = P.out;
         const int64_t p_ldo = P.ldo;
-        float* stg_w = stg + warp * 32 * STG_LD;
+        float* stg_w = stg + (set * 4 + quad) * 32 * 16;
         int it0 = 0;                                     // weight slabs of the layers before
         bool dead = false;                               // the issuer gave up on a wait
         for (int l = 0; l <= nh; ++l) {
@@ -396,7 +436,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
             it0 += nk(l);
             mbar_wait(acc_full, l & 1, err, 34, wlim);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if (l == 0) epi_bar();   // the staged parameter slices
+            if (l == 0) fwd_bar();   // the staged parameter slices
             if (!last) {
                 // ------------------------------------------------------------ hidden layer epilogue
                 const int c0 = rank * NS;                 // this CTA's first column
@@ -408,36 +448,41 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
                 float* const s_mean = P.mean[l];
                 float* const s_rstd = P.rstd[l];
                 const bool s_ph = P.has_ph[l] != 0;
-                // statistics of this CTA's NS columns of the row: mean, then centred squares
-                float s1 = 0.f;
-                for (int c = 0; c < NS; c += 32) {
-                    float v[32], b[32];
-                    tmem_ld32(trow + c, v);
-                    ld_par32(pb + c, b);
+                // statistics of this CTA's NS columns of the row: mean, then centred squares (in order,
+                // so one thread a row; the second set joins where the columns are independent)
+                float mq = 0.f, m2 = 0.f;
+                if (set == 0) {
+                    float s1 = 0.f;
+                    for (int c = 0; c < NS; c += 32) {
+                        float v[32], b[32];
+                        tmem_ld32(trow + c, v);
+                        ld_par32(pb + c, b);
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) s1 += v[j] + b[j];
-                }
-                const float mq = s1 / (float)NS;
-                float m2 = 0.f;
-                for (int c = 0; c < NS; c += 32) {
-                    float v[32], b[32];
-                    tmem_ld32(trow + c, v);
-                    ld_par32(pb + c, b);
+                        for (int j = 0; j < 32; ++j) s1 += v[j] + b[j];
+                    }
+                    mq = s1 / (float)NS;
+                    m2 = 0.f;
+                    for (int c = 0; c < NS; c += 32) {
+                        float v[32], b[32];
+                        tmem_ld32(trow + c, v);
+                        ld_par32(pb + c, b);
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const float d = v[j] + b[j] - mq;
-                        m2 += d * d;
+                        for (int j = 0; j < 32; ++j) {
+                            const float d = v[j] + b[j] - mq;
+                            m2 += d * d;
+                        }
                     }
                 }
                 // the whole row's statistics: every CTA sends (mean, M2) of its slice to every
                 // CTA of the cluster; they are combined in rank order (Chan et al.'s pairwise
                 // update for equal counts: M2 = sum M2_q + NS sum (mean_q - mean)^2)
                 float mean = mq, var = m2 / (float)H;
+                float* buf = xbuf + (l & 1) * CL * BM * 2;
                 if (CL > 1) {
                     const int b = l & 1;
-                    float* buf = xbuf + b * CL * BM * 2;
                     const uint32_t mine = smem_u32(buf + (rank * BM + r) * 2), xb = xbar0 + 8 * b;
-                    for (int q = 0; q < CL; ++q) st_async_v2(mapa(mine, q), mq, m2, mapa(xb, q));
+                    if (set == 0)
+                        for (int q = 0; q < CL; ++q) st_async_v2(mapa(mine, q), mq, m2, mapa(xb, q));
                     mbar_wait<true>(xb, (l >> 1) & 1, err, 35, wlim);
                     // armed again for its next use (every CTA's sends of that use follow this
                     // CTA's sends of the next exchange, which follow all of its reads here)
@@ -451,16 +496,23 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
                         M2 += buf[(q * BM + r) * 2 + 1] + (float)NS * d * d;
                     }
                     var = M2 / (float)H;
+                } else if (set == 0) {
+                    buf[2 * r] = mean;
+                    buf[2 * r + 1] = var;
                 }
-                const float rstd = 1.0f / sqrtf(var + a.eps);
                 // the previous layer's TMA store has read this CTA's slabs before they are rewritten
                 if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-                epi_bar();
+                fwd_bar();
+                if (CL == 1 && set) {
+                    mean = buf[2 * r];
+                    var = buf[2 * r + 1];
+                }
+                const float rstd = 1.0f / sqrtf(var + a.eps);
                 // the last hidden layer feeds only this CTA's K slice of the output layer:
                 // kept locally, at the start of the activation region
                 const bool bcast = CL > 1 && l + 1 < nh;
                 const int kpos0 = (CL > 1 && l + 1 == nh) ? 0 : c0;
-                for (int c = 0; c < NS; c += 32) {
+                for (int c = c_lo; c < c_hi; c += 32) {
                     float v[32], y[32];
                     tmem_ld32(trow + c, v);
                     ld_par32(pb + c, y);
@@ -473,8 +525,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
 #pragma unroll
                         for (int j = 0; j < 32; ++j) y[j] = fmaxf(__fmaf_rn(y[j], (v[j] - mean) * rstd, bt[j]), 0.f);
                     }
-                    if (s_pre) store_rows_coalesced(stg_w, v, s_pre, H, m0 + warp * 32, M, c0 + c, lane);
-                    if (s_post) store_rows_coalesced(stg_w, y, s_post, H, m0 + warp * 32, M, c0 + c, lane);
+                    if (s_pre) store_rows_coalesced16(stg_w, v, s_pre, H, m0 + quad * 32, M, c0 + c, lane);
+                    if (s_post) store_rows_coalesced16(stg_w, y, s_post, H, m0 + quad * 32, M, c0 + c, lane);
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const int k = kpos0 + c + 8 * u;
@@ -487,11 +539,11 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
                                                   ((((k % SLAB) / 8) ^ (r & 7)) * 16)) = w;
                     }
                 }
-                if (H % SLAB)   // the K padding of the last slab reads as zero in the next layer
+                if (H % SLAB && set == 0)   // the K padding of the last slab reads as zero in the next layer
                     for (int k = H; k < hslabs * SLAB; k += 8)
                         *reinterpret_cast<uint4*>(smem + (k / SLAB) * SLAB_BYTES + r * 128 +
                                                   ((((k % SLAB) / 8) ^ (r & 7)) * 16)) = make_uint4(0u, 0u, 0u, 0u);
-                if (rank == 0 && m0 + r < M) {
+                if (rank == 0 && set == 0 && m0 + r < M) {
                     if (s_mean) s_mean[m0 + r] = mean;
                     if (s_rstd) s_rstd[m0 + r] = rstd;
                 }
@@ -499,7 +551,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
                 // reads them; tensor-memory reads before the next layer's MMAs
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                epi_bar();
+                fwd_bar();
                 if (threadIdx.x == 0) {
                     if (s_ph) {
                         for (int j = 0; j < (NS + SLAB - 1) / SLAB; ++j)
@@ -523,7 +575,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
                 const float* pob = par + nh * 3 * NS;
                 SQ_KERNEL_TRIGGER();
                 // this row's output (or partial output) into the idle weight ring, then coalesced
-                for (int c = 0; c < nop; c += 16) {
+                for (int c = 16 * set; c < nop; c += 32) {
                     float v[16];
                     tmem_ld16(trow + c, v);
 #pragma unroll
@@ -532,11 +584,11 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                epi_bar();
+                fwd_bar();
                 // four consecutive columns a thread: element e of the band is (row, 4 c4)
                 const int nq = (nout + 3) / 4;
                 if (CL == 1) {
-                    for (int e = threadIdx.x; e < BM * nq; e += BM) {
+                    for (int e = et; e < BM * nq; e += 256) {
                         const int row = e / nq, col = 4 * (e % nq);
                         const float4 x = *reinterpret_cast<const float4*>(ring_f + row * ldr + col);
                         const float4 bo = *reinterpret_cast<const float4*>(pob + col);
@@ -552,7 +604,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
                             bulk_s2s(mapa(recv + rank * bb, q), ring + q * bb, bb, mapa(out_bar, q));
                     mbar_wait<true>(out_bar, 0, err, 36, wlim);
                     const float* rv = reinterpret_cast<const float*>(smem + (size_t)NS * 256);
-                    for (int e = threadIdx.x; e < band * nq; e += BM) {
+                    for (int e = et; e < band * nq; e += 256) {
                         const int row = e / nq, col = 4 * (e % nq);
                         float4 v = *reinterpret_cast<const float4*>(pob + col);
                         for (int q = 0; q < CL; ++q) {
@@ -574,7 +626,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const __grid_consta
     if (threadIdx.x == 0)
         for (int i = (int)slot[2]; i < (int)slot[1]; ++i) mbar_wait(full(i % S), (i / S) & 1, err, 37, wlim);
     // no CTA of the cluster leaves while a peer may still write into its shared memory
-    if (CL > 1) cluster_sync_all();
+    if (CL > 1) cluster_leave();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0) {
@@ -1302,7 +1354,7 @@ int launch_mlp_tc(const MlpTcProblem* p, int n, int nh, int H, int nout, float e
         d.cta0 = ctas;
         ctas += (q.M + BM - 1) / BM * CL;
     }
-    launch_kc(mlp_tc_kernel, dim3(ctas), dim3(kThreads), (size_t)smem, s, dim3(CL), a);
+    launch_kc(mlp_tc_kernel, dim3(ctas), dim3(kFwdThreads), (size_t)smem, s, dim3(CL), a);
     return 0;
 }
 
