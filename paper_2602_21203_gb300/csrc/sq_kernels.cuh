@@ -138,6 +138,8 @@ struct LnBwdProblem {
     int rows, n;
     const float* dout; int64_t ld_dout;    // gradient w.r.t. the LN(+ReLU) output
     const float* out;  int64_t ld_out;     // forward output (ReLU mask) or null
+    const float* beta;                     // with out null: the shift, and the mask is fma(g, xhat, beta) > 0,
+                                           // the fused forward's rounding of its output; null: no mask
     const float* pre;  int64_t ld_pre;
     const float* mean; const float* rstd;
     const float* g;

@@ -252,7 +252,8 @@ void mlp_forward(squint_handle* h, MlpBufs& mb, const MlpRef* sets, int E, const
                     q.g[l] = ly.g; q.beta[l] = ly.beta;
                     if (keep) {
                         const int64_t off = ((int64_t)e * rows + r0) * H;
-                        q.save[l] = MlpTcSave{mb.pre[l] + off, mb.post[l] + off,
+                        // (no FP32 output: the GEMMs read the BF16 one, the backward rebuilds the mask from pre)
+                        q.save[l] = MlpTcSave{mb.pre[l] + off, nullptr,
                                               mb.posth.empty() ? nullptr : mb.posth[l] + off,
                                               mb.mean[l] + ((int64_t)e * rows + r0), mb.rstd[l] + ((int64_t)e * rows + r0)};
                     }
@@ -500,7 +501,8 @@ bool mlp_backward(squint_handle* h, const MlpBufs& mb, int r0, const MlpRef* set
             LnBwdProblem p{};
             p.rows = rows; p.n = ly.out;
             p.dout = h->dpost[l] + (int64_t)e * rows * ly.out; p.ld_dout = ly.out;
-            p.out = post(l, e).f; p.ld_out = ly.out;
+            if (mb.tc_saved) p.beta = ly.beta;
+            else { p.out = post(l, e).f; p.ld_out = ly.out; }
             p.pre = mb.pre[l] + ((int64_t)e * R + r0) * ly.out; p.ld_pre = ly.out;
             p.mean = mb.mean[l] + (int64_t)e * R + r0; p.rstd = mb.rstd[l] + (int64_t)e * R + r0;
             p.g = ly.g;

@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256) ln_bwd_row_kernel(LnBwdBatch b, int want_
     float* my = acc + (size_t)warp * 3 * P.n;
     if (row < P.rows && P.n <= 32 * kVpt) {
         const float* dout = P.dout + (int64_t)row * P.ld_dout;
-        const float* out = P.out ? P.out + (int64_t)row * P.ld_out : nullptr;
+        const float* msk = P.beta ? P.beta : P.out ? P.out + (int64_t)row * P.ld_out : nullptr;
         const float* pre = P.pre + (int64_t)row * P.ld_pre;
         const float mean = P.mean[row], rstd = P.rstd[row];
         float dn[kVpt], xh[kVpt], gg[kVpt];
@@ -120,10 +120,11 @@ __global__ void __launch_bounds__(256) ln_bwd_row_kernel(LnBwdBatch b, int want_
             const int j = lane + 32 * k;
             const bool in = j < P.n;
             const float d = in ? dout[j] : 0.f;
-            const float o = (in && out) ? out[j] : 1.f;
-            dn[k] = (out && !(o > 0.f)) ? 0.f : d;
             xh[k] = in ? (pre[j] - mean) * rstd : 0.f;
             gg[k] = in ? P.g[j] : 0.f;
+            float o = (in && msk) ? msk[j] : 1.f;
+            if (P.beta) o = __fmaf_rn(gg[k], xh[k], o);
+            dn[k] = (msk && !(o > 0.f)) ? 0.f : d;
         }
         float s1 = 0.f, s2 = 0.f;
 #pragma unroll
@@ -154,11 +155,14 @@ __global__ void __launch_bounds__(256) ln_bwd_row_kernel(LnBwdBatch b, int want_
         const float* out = P.out ? P.out + (int64_t)row * P.ld_out : nullptr;
         const float* pre = P.pre + (int64_t)row * P.ld_pre;
         const float mean = P.mean[row], rstd = P.rstd[row];
+        auto masked = [&](int j, float xh) {
+            return out ? !(out[j] > 0.f) : P.beta && !(__fmaf_rn(P.g[j], xh, P.beta[j]) > 0.f);
+        };
         float s1 = 0.f, s2 = 0.f;
         for (int j = lane; j < P.n; j += 32) {
-            const float dn = (out && !(out[j] > 0.f)) ? 0.f : dout[j];
-            const float dxh = dn * P.g[j];
             const float xh = (pre[j] - mean) * rstd;
+            const float dn = masked(j, xh) ? 0.f : dout[j];
+            const float dxh = dn * P.g[j];
             s1 += dxh;
             s2 += dxh * xh;
         }
@@ -166,8 +170,8 @@ __global__ void __launch_bounds__(256) ln_bwd_row_kernel(LnBwdBatch b, int want_
         const float m2 = warp_sum(s2) / (float)P.n;
         float* dpre = P.dpre + (int64_t)row * P.ld_dpre;
         for (int j = lane; j < P.n; j += 32) {
-            const float dn = (out && !(out[j] > 0.f)) ? 0.f : dout[j];
             const float xh = (pre[j] - mean) * rstd;
+            const float dn = masked(j, xh) ? 0.f : dout[j];
             const float v = rstd * (dn * P.g[j] - m1 - xh * m2);
             dpre[j] = v;
             if (P.dpre_bf) P.dpre_bf[(int64_t)row * P.ld_dpre_bf + j] = __float2bfloat16_rn(v);

@@ -52,6 +52,7 @@ namespace {
 
 constexpr int BM = 128;
 constexpr int SLAB = 64;                  // K elements per slab (128 bytes of BF16)
+constexpr int kMaxSlabs = 8;              // of a hidden layer (wider ones do not fit in shared memory)
 constexpr int SLAB_BYTES = BM * 128;      // one activation slab: 128 rows x 128 B
 constexpr int kThreads = 160;              // backward: an epilogue thread a row
 constexpr int kFwdThreads = 288;           // forward: two a row
@@ -293,12 +294,13 @@ __global__ void __launch_bounds__(kFwdThreads, 1) mlp_tc_kernel(const __grid_con
     float* xbuf = stg + 4 * 32 * STG_LD;                                 // [2][CL][BM][2]: (mean, M2) of each CTA
     float* par = xbuf + 2 * CL * BM * 2;                                 // bias, g, beta slices; output bias
     uint64_t* bars = reinterpret_cast<uint64_t*>(par + a.par_floats);
-    uint32_t* slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 6);     // tmem address, issued, consumed
+    uint32_t* slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 5 + kMaxSlabs);     // tmem address, issued, consumed
     const uint32_t bar0 = smem_u32(bars);
     auto full = [&](int s) { return bar0 + 8 * s; };
     auto empty = [&](int s) { return bar0 + 8 * (S + s); };
-    const uint32_t x_full = bar0 + 8 * (2 * S), acc_full = x_full + 8, a_ready = x_full + 16;
-    const uint32_t xbar0 = x_full + 24, out_bar = x_full + 40;
+    const uint32_t x_full = bar0 + 8 * (2 * S), acc_full = x_full + 8;
+    const uint32_t xbar0 = x_full + 16, out_bar = x_full + 32;
+    auto a_ready = [&](int slab) { return x_full + 40 + 8 * slab; };   // a slab of the activations has arrived
 
     int pi = 0;
     while (pi + 1 < a.n_probs && (int)blockIdx.x >= a.p[pi + 1].cta0) ++pi;
@@ -321,7 +323,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) mlp_tc_kernel(const __grid_con
         }
         mbar_init(x_full, 1);
         mbar_init(acc_full, 1);
-        mbar_init(a_ready, 1);
+        for (int i = 0; i < kMaxSlabs; ++i) mbar_init(a_ready(i), 1);
         mbar_init(xbar0, 1);
         mbar_init(xbar0 + 8, 1);
         mbar_init(out_bar, 1);
@@ -380,12 +382,12 @@ __global__ void __launch_bounds__(kFwdThreads, 1) mlp_tc_kernel(const __grid_con
         }
     } else {
         // a warp reaches the 32 tensor-memory lanes of its number modulo 4; the second set of four
-        // warps takes the later half of the columns
+        // warps takes the later half of each slab's columns
         const int quad = warp % 4, set = warp > 4 ? 1 : 0;
         const int r = quad * 32 + lane;                 // row of the block = tensor-memory lane
         const int et = set * 128 + r;
+        const int nsl = (NS + SLAB - 1) / SLAB;         // slabs of the slice
         const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
-        const int c_mid = (NS / 32 + 1) / 2 * 32, c_lo = set ? c_mid : 0, c_hi = set ? NS : c_mid;
         // this CTA's slices of the bias, LayerNorm gain and shift of every hidden layer, and
         // the output bias, staged by the warps that issue nothing while the first layer's operands
         // arrive (the first epilogue's barrier orders them before any use)
@@ -410,16 +412,14 @@ __global__ void __launch_bounds__(kFwdThreads, 1) mlp_tc_kernel(const __grid_con
             // ---------------------------------------------------------------- MMA issue
             if (warp == 0 && elect_one()) {
                 const bool gave_up = dead;
-                if (!dead) {
-                    if (l == 0) dead = !mbar_wait(x_full, 0, err, 31, wlim);
-                    else dead = !mbar_wait<true>(a_ready, (l - 1) & 1, err, 32, wlim);
-                }
+                if (!dead && l == 0) dead = !mbar_wait(x_full, 0, err, 31, wlim);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t idesc = idesc_bf16_kk(BM, last ? nop : NS);
                 const int nkl = nk(l);
                 int kb = 0, s = it0 % S;
                 uint32_t ph = (uint32_t)(it0 / S) & 1;
                 for (; kb < nkl && !dead; ++kb) {
+                    if (l > 0 && !mbar_wait<true>(a_ready(kb), (l - 1) & 1, err, 32, wlim)) { dead = true; break; }
                     if (!mbar_wait(full(s), ph, err, 33, wlim)) { dead = true; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t as = a_base + kb * SLAB_BYTES, bs = ring + s * a.stage_bytes;
@@ -512,61 +512,65 @@ __global__ void __launch_bounds__(kFwdThreads, 1) mlp_tc_kernel(const __grid_con
                 // kept locally, at the start of the activation region
                 const bool bcast = CL > 1 && l + 1 < nh;
                 const int kpos0 = (CL > 1 && l + 1 == nh) ? 0 : c0;
-                for (int c = c_lo; c < c_hi; c += 32) {
-                    float v[32], y[32];
-                    tmem_ld32(trow + c, v);
-                    ld_par32(pb + c, y);
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] += y[j];
-                    ld_par32(pg + c, y);
-                    {   // g xhat + beta rounded once: the backward rebuilds the ReLU mask the same way
-                        float bt[32];
-                        ld_par32(pbeta + c, bt);
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) y[j] = fmaxf(__fmaf_rn(y[j], (v[j] - mean) * rstd, bt[j]), 0.f);
-                    }
-                    if (s_pre) store_rows_coalesced16(stg_w, v, s_pre, H, m0 + quad * 32, M, c0 + c, lane);
-                    if (s_post) store_rows_coalesced16(stg_w, y, s_post, H, m0 + quad * 32, M, c0 + c, lane);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int k = kpos0 + c + 8 * u;
-                        uint4 w;
-                        w.x = pack_bf16(y[8 * u], y[8 * u + 1]);
-                        w.y = pack_bf16(y[8 * u + 2], y[8 * u + 3]);
-                        w.z = pack_bf16(y[8 * u + 4], y[8 * u + 5]);
-                        w.w = pack_bf16(y[8 * u + 6], y[8 * u + 7]);
-                        *reinterpret_cast<uint4*>(smem + (k / SLAB) * SLAB_BYTES + r * 128 +
-                                                  ((((k % SLAB) / 8) ^ (r & 7)) * 16)) = w;
-                    }
-                }
-                if (H % SLAB && set == 0)   // the K padding of the last slab reads as zero in the next layer
-                    for (int k = H; k < hslabs * SLAB; k += 8)
-                        *reinterpret_cast<uint4*>(smem + (k / SLAB) * SLAB_BYTES + r * 128 +
-                                                  ((((k % SLAB) / 8) ^ (r & 7)) * 16)) = make_uint4(0u, 0u, 0u, 0u);
+                // the slabs that peers send
+                if (bcast && warp == 1 && lane < hslabs && lane / nsl != rank) mbar_expect_tx(a_ready(lane), SLAB_BYTES);
                 if (rank == 0 && set == 0 && m0 + r < M) {
                     if (s_mean) s_mean[m0 + r] = mean;
                     if (s_rstd) s_rstd[m0 + r] = rstd;
                 }
-                // the activation writes before the async proxy (MMA, TMA store, bulk copies)
-                // reads them; tensor-memory reads before the next layer's MMAs
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                fwd_bar();
-                if (threadIdx.x == 0) {
-                    if (s_ph) {
-                        for (int j = 0; j < (NS + SLAB - 1) / SLAB; ++j)
-                            tma_store_2d(&P.tph[l], a_base + (kpos0 / SLAB + j) * SLAB_BYTES, c0 + j * SLAB, m0);
-                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                // slab by slab, so that one is on its way to the other CTAs while the next is formed
+                for (int j = 0; j < nsl; ++j) {
+                    const int c = j * SLAB + 32 * set;
+                    if (c < NS) {
+                        float v[32], y[32];
+                        tmem_ld32(trow + c, v);
+                        ld_par32(pb + c, y);
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) v[j] += y[j];
+                        ld_par32(pg + c, y);
+                        {   // g xhat + beta rounded once: the backward rebuilds the ReLU mask the same way
+                            float bt[32];
+                            ld_par32(pbeta + c, bt);
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) y[j] = fmaxf(__fmaf_rn(y[j], (v[j] - mean) * rstd, bt[j]), 0.f);
+                        }
+                        if (s_pre) store_rows_coalesced16(stg_w, v, s_pre, H, m0 + quad * 32, M, c0 + c, lane);
+                        if (s_post) store_rows_coalesced16(stg_w, y, s_post, H, m0 + quad * 32, M, c0 + c, lane);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int k = kpos0 + c + 8 * u;
+                            uint4 w;
+                            w.x = pack_bf16(y[8 * u], y[8 * u + 1]);
+                            w.y = pack_bf16(y[8 * u + 2], y[8 * u + 3]);
+                            w.z = pack_bf16(y[8 * u + 4], y[8 * u + 5]);
+                            w.w = pack_bf16(y[8 * u + 6], y[8 * u + 7]);
+                            *reinterpret_cast<uint4*>(smem + (k / SLAB) * SLAB_BYTES + r * 128 +
+                                                      ((((k % SLAB) / 8) ^ (r & 7)) * 16)) = w;
+                        }
+                    } else {   // the K padding of the last slab reads as zero in the next layer
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            *reinterpret_cast<uint4*>(smem + (kpos0 / SLAB + j) * SLAB_BYTES + r * 128 +
+                                                      (((4 * set + u) ^ (r & 7)) * 16)) = make_uint4(0u, 0u, 0u, 0u);
                     }
-                    if (bcast) {
-                        // this CTA's slice (whole slabs) into the same place of every other
-                        // CTA's activation region; each copy completes on the receiver's barrier
-                        const uint32_t src = a_base + (c0 / SLAB) * SLAB_BYTES, bytes = (uint32_t)NS * 256;
-                        for (int q = 0; q < CL; ++q)
-                            if (q != rank) bulk_s2s(mapa(src, q), src, bytes, mapa(a_ready, q));
-                        mbar_expect_tx(a_ready, (uint32_t)(CL - 1) * bytes);
-                    } else {
-                        mbar_arrive_local(a_ready);
+                    // the activation writes before the async proxy (MMA, TMA store, bulk copies)
+                    // reads them; tensor-memory reads before the next layer's MMAs
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    fwd_bar();
+                    if (threadIdx.x == 0) {
+                        const int slab = kpos0 / SLAB + j;
+                        const uint32_t src = a_base + slab * SLAB_BYTES;
+                        // the same place of every other CTA's activation region; each copy
+                        // completes on the receiver's barrier
+                        if (bcast)
+                            for (int q = 0; q < CL; ++q)
+                                if (q != rank) bulk_s2s(mapa(src, q), src, SLAB_BYTES, mapa(a_ready(slab), q));
+                        mbar_arrive_local(a_ready(slab));
+                        if (s_ph) {
+                            tma_store_2d(&P.tph[l], src, c0 + j * SLAB, m0);
+                            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                        }
                     }
                 }
             } else {
@@ -1150,6 +1154,7 @@ bool plan(int H, int CL, int nh, int nop, int kin, int* a_bytes, int* stage_byte
     *a_bytes = std::max(k0, hs) * SLAB_BYTES;
     *stage_bytes = std::max(NS, nop) * 128;
     *par_floats = (nh * 3 * NS + nop + 3) / 4 * 4;
+    if (hs > kMaxSlabs) return false;
     const int fixed = 1024 + STG_BYTES + 2 * CL * BM * 2 * 4 + *par_floats * 4 + 256;
     const int n = (SMEM_LIMIT - fixed - *a_bytes) / *stage_bytes;
     *stages = std::min(n, 8);
