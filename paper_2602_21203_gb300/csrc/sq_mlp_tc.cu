@@ -17,9 +17,9 @@
 //                     each CTA's mean and centred sum of squares of its slice, sent to
 //                     every CTA of the cluster with st.async and combined in rank order),
 //                     then half of the columns each: ReLU; the BF16 result is written into
-//                     this CTA's activation
-//                     region as the next layer's A operand and copied to the other CTAs of
-//                     the cluster with one shared-to-shared bulk copy each; saved FP32
+//                     this CTA's activation region as the next layer's A operand and each slab copied to the
+//                     other CTAs of the cluster with a shared-to-shared bulk copy each, while
+//                     the next slab is formed and earlier ones are multiplied; saved FP32
 //                     activations leave through a per-warp transpose as coalesced rows,
 //                     the BF16 copy by a TMA store of the CTA's own slabs
 //   output layer      K split over the cluster (each CTA multiplies its own column slice
@@ -30,10 +30,11 @@
 // Data that crosses CTAs travels by st.async and bulk copies that complete transaction
 // bytes on the receiver's mbarrier, so no cluster-scope fence or cluster-wide barrier is
 // needed between the layers, and the producer streams ahead undisturbed.
-// What bounds it: a chain of latencies at one CTA per SM.  Of the 40,000 cycles of M 512, kin 268,
+// What bounds it: a chain of latencies at one CTA per SM.  Of the 38,000 cycles of M 512, kin 268,
 // H 512, nout 12 the copies between the CTAs (14 bytes a cycle into an SM) and the second layer's
-// products take 9,000, the first layer's operands 4,000, the statistics and their exchange 4,000
-// a layer.  One thread per row: 20.2 us (nout 101 twice 24.2, M 4096 22.3), two: 18.8 (22.5, 21.0).
+// products take 8,000, the first layer's operands 4,000, the statistics and their exchange 4,000
+// a layer.  One thread per row: 20.2 us (nout 101 twice 24.2, M 4096 22.3), two: 18.8 (22.5, 21.0),
+// and with the slabs sent and multiplied one by one, not the slice at once: 17.9 (21.6, 20.2).
 // Every wait is bounded; past the limit the waiting thread records a code in *err and
 // gives up, the CTA waits (bounded) for its copies in flight, frees its tensor memory and
 // returns.
