@@ -309,19 +309,24 @@ __global__ void __launch_bounds__(kConvThreads) conv32_tc_kernel(const __grid_co
 // ---------------------------------------------------------------- weight gradient
 // D_tap[co, ci] += sum_q dy[q, co] x[q + origin(tap), ci] over the virtual grid of
 // the input's padded row width (dy = 0 outside the valid outputs), origin(ky, kx) =
-// (2 + ky) Wp + 2 + kx.  A = dy^T, MN-major: the threads copy dy's 16-byte pixel chunks
+// (2 + ky) Wp + 2 + kx.  A = dy^T, MN-major: four warps copy dy's 16-byte pixel chunks
 // unchanged into four channel planes of kq pixel rows (no transpose); rows 32..127 of the
 // 128-row MMA read whatever follows in shared memory (inside the allocation: the dy
 // buffers come first) and land in accumulator rows that are never read.  B stacks the
 // three horizontal taps: shared memory holds
-// twelve slots (kx, channel plane), slot (kx, p) = rows origin(0, kx) + [0, slot_rows)
-// of plane p, SLOT apart, so one MN-major operand of N = 96 (kx, ci) starting ky Wp
+// twelve slots (kx, channel plane), slot (kx, p) = rows origin(0, kx) + [0, x_rows)
+// of plane p, slot_rows apart, so one MN-major operand of N = 96 (kx, ci) starting ky Wp
 // rows into every slot covers taps (ky, 0..2); its accumulator columns ky 96 + kx 32 +
 // ci are tap 32 + ci.  Three MMAs per 16 pixels instead of nine.
+// What bounds it, for 512 images of 15 x 15, four to a CTA: the products (3,000 cycles an image)
+// and the fixed start and end (5,000).  The next image is staged while one is multiplied; four
+// more warps copy the input with 16-byte asynchronous copies, where tensor copies of its 16-byte
+// plane rows took 4,800 cycles an image to issue; the end reads the accumulators by three
+// warps and stores 16 bytes a thread.  20.2 us before, 11.5 now (11 x 11: 17.9 and 9.3).
 struct WgradArgs {
-    CUtensorMap tin;                 // layer input planes, dims {8, 4, nimg * in_rows}, box {8, 1, box_rows}
+    const __nv_bfloat16* x;          // padded-HWC layer input
     const __nv_bfloat16* dy;         // padded-HWC gradient at the layer's pre-activation (grid out_w + 4)
-    int nimg, in_rows, Wp, out_h, out_w, kq, slot_rows, box_rows, per_cta;
+    int nimg, in_rows, Wp, out_h, out_w, kq, slot_rows, x_rows, per_cta;
     float* work;                     // [ctas, 32, 289]: partial dW (co, ci*9 + tap) and db (col 288)
     int* err;
 };
@@ -335,7 +340,9 @@ __host__ __device__ inline uint32_t wgrad_operand_bytes(uint32_t xbytes, uint32_
     return ops > kWgTileBytes ? ops : kWgTileBytes;
 }
 
-__global__ void __launch_bounds__(128) wgrad32_tc_kernel(const __grid_constant__ WgradArgs a) {
+// Threads 0-127 stage dy, 128-255 the input, warp 8 issues the products.
+constexpr int kWgThreads = 288;
+__global__ void __launch_bounds__(kWgThreads) wgrad32_tc_kernel(const __grid_constant__ WgradArgs a) {
     SQ_KERNEL_WAIT();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -348,15 +355,14 @@ __global__ void __launch_bounds__(128) wgrad32_tc_kernel(const __grid_constant__
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + wgrad_operand_bytes(xbytes, dybytes));
     float* red = reinterpret_cast<float*>(bars + 8);             // [128][8] bias partials
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(red + 128 * 8);
-    const uint32_t tma_bar[2] = {smem_u32(bars), smem_u32(bars + 1)};
-    const uint32_t mma_bar[2] = {smem_u32(bars + 2), smem_u32(bars + 3)};
-    const uint32_t done_bar = smem_u32(bars + 4);
+    const uint32_t mma_bar[2] = {smem_u32(bars), smem_u32(bars + 1)};
+    const uint32_t done_bar = smem_u32(bars + 2);
     const int warp = warp_uniform((int)threadIdx.x / 32), lane = threadIdx.x % 32;
     const int i0 = blockIdx.x * a.per_cta, i1 = min(a.nimg, i0 + a.per_cta);
 
     if (warp == 0) tmem_alloc(smem_u32(tmem_slot), 512);
     if (threadIdx.x == 32) {
-        for (int b = 0; b < 2; ++b) { mbar_init(tma_bar[b], 1); mbar_init(mma_bar[b], 1); }
+        for (int b = 0; b < 2; ++b) mbar_init(mma_bar[b], 1);
         mbar_init(done_bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -371,30 +377,34 @@ __global__ void __launch_bounds__(128) wgrad32_tc_kernel(const __grid_constant__
     bool ok = true;
     constexpr uint32_t idesc = idesc_bf16(128, 3 * kCh, true, true);
 
-    // Every thread runs every iteration (the barriers inside must match); a wait that
-    // gives up only records the error and stops further MMA issue.
-    for (int i = i0; i < i1; ++i) {
-        const int li = i - i0, b = li & 1;
-        if (li >= 2 && !mbar_wait(mma_bar[b], ((li - 2) >> 1) & 1, a.err, 21)) ok = false;
-        if (warp == 0 && elect_one() && ok) {
-            const int boxes = a.slot_rows / a.box_rows;
-            const int row0 = i * a.in_rows + 2 * a.Wp + 2;
-            mbar_expect_tx(tma_bar[b], xbytes);
-            for (int kx = 0; kx < 3; ++kx)
-                for (int c = 0; c < 4; ++c)
-                    for (int bb = 0; bb < boxes; ++bb)
-                        tma_load_3d(smem_u32(xs[b]) + (kx * 4 + c) * slot + bb * a.box_rows * 16, &a.tin, 0, c,
-                                    row0 + kx + bb * a.box_rows, tma_bar[b]);
+    const int64_t x_end = (int64_t)a.nimg * a.in_rows;
+    auto stage = [&](int i) {
+        const int b = (i - i0) & 1;
+        if (warp >= 4) {
+            // the input's 16-byte chunks, once per horizontal tap; rows behind the last image read as
+            // zero.  (A pixel's four chunks land slot bytes apart, an odd multiple of 32: no bank
+            // conflict.  Tensor copies of 16-byte rows would take 1.3 cycles a row, three times this.)
+            const int64_t row0 = (int64_t)i * a.in_rows + 2 * a.Wp + 2;
+            const uint32_t dst = smem_u32(xs[b]) + cc * slot;
+            for (int row = (threadIdx.x - 128) / 4; row < a.x_rows; row += 32) {
+#pragma unroll
+                for (int kx = 0; kx < 3; ++kx) {
+                    const bool in = row0 + kx + row < x_end;
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst + kx * 4 * slot + row * 16),
+                                 "l"(in ? a.x + (row0 + kx + row) * kCh + cc * 8 : a.x), "r"(in ? 16 : 0) : "memory");
+                }
+            }
+            return;
         }
         // stage dy: the 16-byte chunk of channels 8 cc .. 8 cc + 7 of pixel q at cc PLANE + 16 q
         // (zero outside the valid outputs); a thread's loads for eight pixels are issued
         // before any of them is stored
         uint8_t* d = ds[b];
-        for (int j0 = threadIdx.x; j0 < a.kq * 4; j0 += 8 * blockDim.x) {
+        for (int j0 = threadIdx.x; j0 < a.kq * 4; j0 += 8 * 128) {
             uint4 v4[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const int j = j0 + u * blockDim.x;
+                const int j = j0 + u * 128;
                 const int q = j >> 2;
                 const int oy = q / a.Wp, ox = q - (q / a.Wp) * a.Wp;
                 v4[u] = make_uint4(0, 0, 0, 0);
@@ -404,7 +414,7 @@ __global__ void __launch_bounds__(128) wgrad32_tc_kernel(const __grid_constant__
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const int j = j0 + u * blockDim.x;
+                const int j = j0 + u * 128;
                 if (j >= a.kq * 4) break;
                 const int q = j >> 2;
                 const __nv_bfloat16* hv = reinterpret_cast<const __nv_bfloat16*>(&v4[u]);
@@ -413,13 +423,17 @@ __global__ void __launch_bounds__(128) wgrad32_tc_kernel(const __grid_constant__
                 for (int k = 0; k < 8; ++k) bsum[k] += __bfloat162float(hv[k]);
             }
         }
+    };
+    // Every thread runs every iteration (the barriers inside must match); a wait that gives up
+    // only records the error and stops this thread's staging.
+    if (warp < 8 && i0 < i1) stage(i0);
+    for (int i = i0; i < i1; ++i) {
+        const int li = i - i0, b = li & 1;
+        asm volatile("cp.async.wait_all;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
-        if (warp == 1 && elect_one()) {
-            if (!ok || !mbar_wait(tma_bar[b], (li >> 1) & 1, a.err, 22)) {
-                ok = false;
-            } else {
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (warp == 8) {
+            if (elect_one()) {
                 // descriptors built once; each MMA adds its start offset in 16-byte units
                 // (shared-memory addresses stay below 2^18: the 14-bit field never carries)
                 const uint64_t a0 = plain_desc(smem_u32(ds[b]), 128, dplane);
@@ -429,12 +443,16 @@ __global__ void __launch_bounds__(128) wgrad32_tc_kernel(const __grid_constant__
                     for (int ky = 0; ky < 3; ++ky)
                         mma_bf16(tmem + ky * 3 * kCh, a0 + (uint64_t)(k * 16), b0 + (uint64_t)(k * 16 + ky * a.Wp),
                                  idesc, (i > i0 || k > 0) ? 1u : 0u);
+                mma_commit(mma_bar[b]);
             }
-            mma_commit(mma_bar[b]);
+            __syncwarp();
+        } else if (i + 1 < i1) {
+            // the next image, into the buffers that the products of the one before have read
+            if (li >= 1 && !mbar_wait(mma_bar[b ^ 1], ((li - 1) >> 1) & 1, a.err, 21)) ok = false;
+            if (ok) stage(i + 1);
         }
-        __syncwarp();
     }
-    if (warp == 1 && elect_one()) mma_commit(done_bar);
+    if (warp == 8 && elect_one()) mma_commit(done_bar);
     __syncwarp();
     SQ_KERNEL_TRIGGER();
     const bool have = mbar_wait(done_bar, 0, a.err, 23) && ok && i1 > i0;
@@ -442,20 +460,22 @@ __global__ void __launch_bounds__(128) wgrad32_tc_kernel(const __grid_constant__
     // bias partials: reduce the 32 threads of each chunk in a fixed order.  The partial
     // tile [co][ci * 9 + tap | bias] is assembled in shared memory (the operand buffers are
     // idle once the last MMA has completed) and stored by all threads, coalesced.
+    if (threadIdx.x < 128) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) red[threadIdx.x * 8 + k] = bsum[k];
+        for (int k = 0; k < 8; ++k) red[threadIdx.x * 8 + k] = bsum[k];
+    }
     __syncthreads();
     constexpr int NW = kCh * 9 + 1;
     float* tile = reinterpret_cast<float*>(smem);   // [kCh][NW]
-    if (threadIdx.x < kCh) {
-        const int co = threadIdx.x;
+    if (warp == 1) {
+        const int co = lane;
         float s = 0.f;
         for (int t = co / 8; t < 128; t += 4) s += red[t * 8 + (co % 8)];
         tile[co * NW + kCh * 9] = s;
     }
-    if (warp == 0) {
+    if (warp % 4 == 0) {   // lanes 0-31 of the accumulators: a row ky of taps each
         const int co = lane;
-        for (int tap = 0; tap < 9; ++tap) {
+        for (int tap = 3 * (warp / 4); tap < 3 * (warp / 4) + 3; ++tap) {
             uint32_t r0[16], r1[16];
             tmem_ld16(tmem + tap * kCh, r0);
             tmem_ld16(tmem + tap * kCh + 16, r1);
@@ -468,7 +488,12 @@ __global__ void __launch_bounds__(128) wgrad32_tc_kernel(const __grid_constant__
     }
     __syncthreads();
     float* out = a.work + (int64_t)blockIdx.x * kCh * NW;
-    for (int e = threadIdx.x; e < kCh * NW; e += blockDim.x) out[e] = tile[e];
+    if (reinterpret_cast<uintptr_t>(out) % 16 == 0) {
+        for (int e = threadIdx.x; e < kCh * NW / 4; e += kWgThreads)
+            reinterpret_cast<float4*>(out)[e] = reinterpret_cast<const float4*>(tile)[e];
+    } else {
+        for (int e = threadIdx.x; e < kCh * NW; e += kWgThreads) out[e] = tile[e];
+    }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0) {
@@ -1103,12 +1128,12 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 }
 
 // Planes of a padded-HWC tensor: dims {8 channels, 4 planes, rows}, box {8, 1, 128}.
-bool plane_map(CUtensorMap* m, const __nv_bfloat16* base, int64_t rows, int box_rows = 128) {
+bool plane_map(CUtensorMap* m, const __nv_bfloat16* base, int64_t rows) {
     auto fn = encode_fn();
-    if (!fn || (reinterpret_cast<uintptr_t>(base) & 15) || box_rows < 8 || box_rows > 256) return false;
+    if (!fn || (reinterpret_cast<uintptr_t>(base) & 15)) return false;
     cuuint64_t dims[3] = {8, 4, (cuuint64_t)rows};
     cuuint64_t strides[2] = {16, 64};
-    cuuint32_t box[3] = {8, 1, (cuuint32_t)box_rows};
+    cuuint32_t box[3] = {8, 1, 128};
     cuuint32_t estr[3] = {1, 1, 1};
     std::memset(m, 0, sizeof(*m));
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16*>(base), dims, strides, box, estr,
@@ -1163,19 +1188,18 @@ int launch_wgrad32_tc_partials(const WgradTc& c, int per_cta, float* work, int* 
     WgradArgs a;
     std::memset(&a, 0, sizeof(a));
     a.kq = round_up(c.out_h * c.Wp, 16);
-    // a slot covers the rows every K step of every vertical tap reads: kq + 2 Wp, loaded in
-    // equal boxes of at most 256 rows, a multiple of 8 rows (128 B) each
-    const int need = a.kq + 2 * c.Wp;
-    const int nb = (need + 255) / 256;
-    a.box_rows = round_up((need + nb - 1) / nb, 8);
-    a.slot_rows = nb * a.box_rows;
+    // a slot covers the rows every K step of every vertical tap reads: kq + 2 Wp
+    a.x_rows = a.kq + 2 * c.Wp;
+    a.slot_rows = (a.x_rows + 5) / 8 * 8 + 2;
+    if (wgrad_smem(a.slot_rows, a.kq) > 220 * 1024) a.slot_rows = a.x_rows;   // the largest images: any pitch that fits
     if (wgrad_smem(a.slot_rows, a.kq) > 220 * 1024 || (a.kq / 8) * 512 + 2048 > kDyBytesMax + 2048) return -1;
-    if (!plane_map(&a.tin, c.x, (int64_t)c.nimg * c.in_rows, a.box_rows)) return -2;
+    if (reinterpret_cast<uintptr_t>(c.x) & 15) return -2;
+    a.x = c.x;
     a.per_cta = per_cta;
     const int grid = (c.nimg + per_cta - 1) / per_cta;
     a.dy = c.dy; a.nimg = c.nimg; a.in_rows = c.in_rows; a.Wp = c.Wp; a.out_h = c.out_h; a.out_w = c.out_w;
     a.work = work; a.err = err;
-    launch_k(wgrad32_tc_kernel, dim3(grid), dim3(128), wgrad_smem(a.slot_rows, a.kq), s, a);
+    launch_k(wgrad32_tc_kernel, dim3(grid), dim3(kWgThreads), wgrad_smem(a.slot_rows, a.kq), s, a);
     return 0;
 }
 
