@@ -275,7 +275,7 @@ __device__ float block_sum(float v, float* sh) {
 }
 
 // ---------------------------------------------------------------- C51 target
-// One warp per sample (kHeadRows samples a block, V atoms a lane: atom j = lane + 32 k):
+// One warp per sample (kC51Rows samples a block, V atoms a lane: atom j = lane + 32 k):
 // average of the target critics' categorical distributions, projected onto the fixed
 // support as m_j = sum_i P_i max(0, 1 - |b_i - j|)   (linear interpolation between the
 // two neighbouring atoms of b_i = (clip(r + gamma (1-d)(z_i - alpha log pi')) - v_min)/dz),
@@ -283,14 +283,18 @@ __device__ float block_sum(float v, float* sh) {
 // critic with the smaller mean (ties to critic 0).  MSE critics (K = 1): y = r + gamma
 // (1-d)(Q_bar - alpha log pi') with Q_bar the average (or, with clipped double Q, the
 // minimum) of the target outputs.  Softmax statistics by warp shuffles, no block barrier.
-constexpr int kHeadRows = 8;
+constexpr int kHeadRows = 8;   // samples a block of the other per-sample kernels
+// The target's projection walks all K atoms for each of a lane's V: one warp a scheduler, and one
+// read of an atom for the V of them (512 rows of 101 atoms, two critics, in the update, waiting for
+// its inputs included: 13.0 us with eight rows a block and a walk for each, 11.8 now).
+constexpr int kC51Rows = 4;
 
 template <int V>
-__global__ void __launch_bounds__(32 * kHeadRows) c51_target_kernel(C51TargetArgs a) {
+__global__ void __launch_bounds__(32 * kC51Rows) c51_target_kernel(C51TargetArgs a) {
     SQ_KERNEL_ENTRY();
-    __shared__ float sp[kHeadRows][32 * V], sb[kHeadRows][32 * V];
+    __shared__ float2 spb[kC51Rows][32 * V];   // an atom's probability and its projected place
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const int row = blockIdx.x * kHeadRows + warp;
+    const int row = blockIdx.x * kC51Rows + warp;
     if (a.steps && blockIdx.x == 0 && threadIdx.x == 0) {
         const int act = (((uint64_t)*a.update_idx + 1) % (uint64_t)a.policy_freq) == 0;
         a.steps[0] += 1;
@@ -374,18 +378,21 @@ __global__ void __launch_bounds__(32 * kHeadRows) c51_target_kernel(C51TargetArg
         const float zj = a.v_min + (float)j * dz;
         float tz = r + a.gamma * nd * (zj - alpha * lp);
         tz = fminf(fmaxf(tz, a.v_min), a.v_max);
-        sp[warp][j] = pb[k] / n_used;
-        sb[warp][j] = fminf(fmaxf((tz - a.v_min) / dz, 0.f), (float)(K - 1));
+        spb[warp][j] = make_float2(pb[k] / n_used, fminf(fmaxf((tz - a.v_min) / dz, 0.f), (float)(K - 1)));
     }
     __syncwarp();
+    float acc[V];
 #pragma unroll
-    for (int k = 0; k < V; ++k) {
-        const int j = lane + 32 * k;
-        if (j >= K) break;
-        float acc = 0.f;
-        for (int i = 0; i < K; ++i) acc += sp[warp][i] * fmaxf(0.f, 1.0f - fabsf(sb[warp][i] - (float)j));
-        a.m[(int64_t)row * K + j] = acc;
+    for (int k = 0; k < V; ++k) acc[k] = 0.f;
+#pragma unroll 4
+    for (int i = 0; i < K; ++i) {
+        const float2 x = spb[warp][i];
+#pragma unroll
+        for (int k = 0; k < V; ++k) acc[k] += x.x * fmaxf(0.f, 1.0f - fabsf(x.y - (float)(lane + 32 * k)));
     }
+#pragma unroll
+    for (int k = 0; k < V; ++k)
+        if (lane + 32 * k < K) a.m[(int64_t)row * K + lane + 32 * k] = acc[k];
 }
 
 // ---------------------------------------------------------------- cross entropy
@@ -553,63 +560,71 @@ __device__ __forceinline__ float softplusf(float x) { return fmaxf(x, 0.f) + log
 
 // log_std = lo + (hi-lo)/2 (tanh(raw)+1); u = mu + std eps; a = tanh(u);
 // log pi = sum_k [-eps^2/2 - log_std - log(2 pi)/2 - 2 (log 2 - u - softplus(-2u))].
-__global__ void actor_head_kernel(ActorHeadArgs a) {
+// G threads a row (a power of two, at least A where A <= 32): a draw, three exponentials and two
+// hyperbolic tangents an action are a long chain, so the actions go side by side; the log
+// probability adds their terms in action order.  (512 rows of 6 actions in the update: 6.0 us with
+// one thread a row, 4.0 with eight; the backward, all actions side by side, 6.7 and 4.1.)
+template <int G>
+__global__ void __launch_bounds__(128) actor_head_kernel(ActorHeadArgs a) {
     SQ_KERNEL_ENTRY();
-    const int row = a.row0 + blockIdx.x * blockDim.x + threadIdx.x;
-    if (row >= a.rows) return;
-    const bool tgt = row < a.B;
+    const int row = a.row0 + (blockIdx.x * 128 + threadIdx.x) / G, k0 = threadIdx.x % G;
+    const bool in = row < a.rows, tgt = row < a.B;
     const int el = tgt ? row : row - a.B;
     const uint64_t u = a.update_idx ? (uint64_t)*a.update_idx : 0;
     const float* o = a.out + (int64_t)row * a.ld_out;
     float lp = 0.f;
-    for (int k = 0; k < a.A; ++k) {
-        const float eps = a.eps_in ? a.eps_in[(int64_t)row * a.A + k]
-                                   : normal_draw(a.seed, (uint32_t)el, tgt ? kStreamEpsTarget : kStreamEpsActor, u, k);
-        const float mu = o[k], raw = o[a.A + k];
-        const float ls = a.lo + 0.5f * (a.hi - a.lo) * (tanhf(raw) + 1.0f);
-        const float sd = expf(ls);
-        const float uu = mu + sd * eps;
-        const float act = tanhf(uu);
-        lp += -0.5f * eps * eps - ls - 0.91893853320467274f - 2.0f * (0.69314718055994531f - uu - softplusf(-2.0f * uu));
-        if (a.eps) a.eps[(int64_t)row * a.A + k] = eps;
-        if (tgt) {
-            a.a_dst0[(int64_t)row * a.ld0 + k] = act;
-            if (a.a_dst0_h) a.a_dst0_h[(int64_t)row * a.ld0_h + k] = __float2bfloat16_rn(act);
-        } else {
-            a.a_dst1[(int64_t)el * a.ld1 + k] = act;
-            if (a.a_dst1_h) a.a_dst1_h[(int64_t)el * a.ld1_h + k] = __float2bfloat16_rn(act);
+    for (int kb = 0; kb < a.A; kb += G) {
+        const int k = kb + k0;
+        float term = 0.f;
+        if (in && k < a.A) {
+            const float eps = a.eps_in ? a.eps_in[(int64_t)row * a.A + k]
+                                       : normal_draw(a.seed, (uint32_t)el, tgt ? kStreamEpsTarget : kStreamEpsActor, u, k);
+            const float mu = o[k], raw = o[a.A + k];
+            const float ls = a.lo + 0.5f * (a.hi - a.lo) * (tanhf(raw) + 1.0f);
+            const float sd = expf(ls);
+            const float uu = mu + sd * eps;
+            const float act = tanhf(uu);
+            term = -0.5f * eps * eps - ls - 0.91893853320467274f - 2.0f * (0.69314718055994531f - uu - softplusf(-2.0f * uu));
+            if (a.eps) a.eps[(int64_t)row * a.A + k] = eps;
+            if (tgt) {
+                a.a_dst0[(int64_t)row * a.ld0 + k] = act;
+                if (a.a_dst0_h) a.a_dst0_h[(int64_t)row * a.ld0_h + k] = __float2bfloat16_rn(act);
+            } else {
+                a.a_dst1[(int64_t)el * a.ld1 + k] = act;
+                if (a.a_dst1_h) a.a_dst1_h[(int64_t)el * a.ld1_h + k] = __float2bfloat16_rn(act);
+            }
         }
+        for (int i = 0; i < min(G, a.A - kb); ++i) lp += __shfl_sync(0xffffffffu, term, i, G);
     }
-    a.logp[row] = lp;
+    if (in && k0 == 0) a.logp[row] = lp;
 }
 
 // Reparameterised backward: du = da (1 - a^2) + dlogp 2a; dlog_std = du std eps - dlogp;
 // draw = dlog_std (hi-lo)/2 (1 - tanh(raw)^2).
-__global__ void actor_head_bwd_kernel(ActorHeadBwdArgs a) {
+__global__ void __launch_bounds__(128) actor_head_bwd_kernel(ActorHeadBwdArgs a) {   // a thread an action
     SQ_KERNEL_ENTRY();
     if (a.do_actor && !*a.do_actor) return;
-    const int row = blockIdx.x * blockDim.x + threadIdx.x;
-    if (row >= a.B) return;
+    const int64_t e = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    if (e >= (int64_t)a.B * a.A) return;
+    const int row = (int)(e / a.A), k = (int)(e - (int64_t)row * a.A);
     const float dlogp = a.dlogp_rows ? a.dlogp_rows[row] : expf(*a.log_alpha) / (float)a.B;
     const float* o = a.out + (int64_t)row * a.ld_out;
-    for (int k = 0; k < a.A; ++k) {
-        const float eps = a.eps[(int64_t)row * a.A + k];
-        const float mu = o[k], raw = o[a.A + k];
-        const float th = tanhf(raw);
-        const float sd = expf(a.lo + 0.5f * (a.hi - a.lo) * (th + 1.0f));
-        const float act = tanhf(mu + sd * eps);
-        const int64_t ldd = a.ld_da ? a.ld_da : a.A;
-        float dq = a.da[(int64_t)row * ldd + k];
-        if (a.da2) dq += a.da2[(int64_t)row * ldd + k];
-        const float du = dq * (1.0f - act * act) + dlogp * 2.0f * act;
-        const float dls = du * sd * eps - dlogp;
-        const float draw = dls * 0.5f * (a.hi - a.lo) * (1.0f - th * th);
-        a.dout[(int64_t)row * 2 * a.A + k] = du;
-        a.dout[(int64_t)row * 2 * a.A + a.A + k] = draw;
-        if (a.dout_bf) {
-            a.dout_bf[(int64_t)row * a.ld_dout_bf + k] = __float2bfloat16_rn(du);
-            a.dout_bf[(int64_t)row * a.ld_dout_bf + a.A + k] = __float2bfloat16_rn(draw);
-        }
+    const float eps = a.eps[e];
+    const float mu = o[k], raw = o[a.A + k];
+    const float th = tanhf(raw);
+    const float sd = expf(a.lo + 0.5f * (a.hi - a.lo) * (th + 1.0f));
+    const float act = tanhf(mu + sd * eps);
+    const int64_t ldd = a.ld_da ? a.ld_da : a.A;
+    float dq = a.da[(int64_t)row * ldd + k];
+    if (a.da2) dq += a.da2[(int64_t)row * ldd + k];
+    const float du = dq * (1.0f - act * act) + dlogp * 2.0f * act;
+    const float dls = du * sd * eps - dlogp;
+    const float draw = dls * 0.5f * (a.hi - a.lo) * (1.0f - th * th);
+    a.dout[(int64_t)row * 2 * a.A + k] = du;
+    a.dout[(int64_t)row * 2 * a.A + a.A + k] = draw;
+    if (a.dout_bf) {
+        a.dout_bf[(int64_t)row * a.ld_dout_bf + k] = __float2bfloat16_rn(du);
+        a.dout_bf[(int64_t)row * a.ld_dout_bf + a.A + k] = __float2bfloat16_rn(draw);
     }
 }
 
@@ -1003,14 +1018,19 @@ void launch_colsum(const ColSumProblem* p, int n, cudaStream_t s) {
     }
 }
 void launch_actor_head(const ActorHeadArgs& a, cudaStream_t s) {
-    if (a.rows > a.row0) launch_k(actor_head_kernel, dim3((a.rows - a.row0 + 127) / 128), dim3(128), 0, s, a);
+    if (a.rows <= a.row0) return;
+    const int g = a.A <= 8 ? 8 : a.A <= 16 ? 16 : 32, per = 128 / g;
+    const dim3 grid((unsigned)(((int64_t)a.rows - a.row0 + per - 1) / per));
+    if (g == 8) launch_k(actor_head_kernel<8>, grid, dim3(128), 0, s, a);
+    else if (g == 16) launch_k(actor_head_kernel<16>, grid, dim3(128), 0, s, a);
+    else launch_k(actor_head_kernel<32>, grid, dim3(128), 0, s, a);
 }
 void launch_actor_head_bwd(const ActorHeadBwdArgs& a, cudaStream_t s) {
-    launch_k(actor_head_bwd_kernel, dim3((a.B + 127) / 128), dim3(128), 0, s, a);
+    launch_k(actor_head_bwd_kernel, dim3((unsigned)(((int64_t)a.B * a.A + 127) / 128)), dim3(128), 0, s, a);
 }
 // atoms per lane: 4 up to 128 atoms, 8 up to 256 (the most a configuration takes)
 void launch_c51_target(const C51TargetArgs& a, cudaStream_t s) {
-    const dim3 g((a.B + kHeadRows - 1) / kHeadRows), t(32 * kHeadRows);
+    const dim3 g((a.B + kC51Rows - 1) / kC51Rows), t(32 * kC51Rows);
     if (a.K <= 128) launch_k(c51_target_kernel<4>, g, t, 0, s, a);
     else launch_k(c51_target_kernel<8>, g, t, 0, s, a);
 }
