@@ -790,12 +790,13 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
     float* colacc = xbuf + 2 * CL * BM * 2;                              // [4 warps][3][NS] column sums
     float* par = colacc + 4 * 3 * NS;                                    // g (then beta) slices of the hidden layers
     uint64_t* bars = reinterpret_cast<uint64_t*>(par + ((2 * nh * NS + 3) / 4) * 4);
-    uint32_t* slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 6);     // tmem address, issued, consumed
+    uint32_t* slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 5 + kMaxSlabs);     // tmem address, issued, consumed
     const uint32_t bar0 = smem_u32(bars);
     auto full = [&](int s) { return bar0 + 8 * s; };
     auto empty = [&](int s) { return bar0 + 8 * (S + s); };
-    const uint32_t a0_full = bar0 + 8 * (2 * S), acc_full = a0_full + 8, a_ready = a0_full + 16;
-    const uint32_t xbar0 = a0_full + 24, out_bar = a0_full + 40;
+    const uint32_t a0_full = bar0 + 8 * (2 * S), acc_full = a0_full + 8;
+    const uint32_t xbar0 = a0_full + 16, out_bar = a0_full + 32;
+    auto a_ready = [&](int slab) { return a0_full + 40 + 8 * slab; };
 
     int pi = 0;
     while (pi + 1 < a.n_probs && (int)blockIdx.x >= a.p[pi + 1].cta0) ++pi;
@@ -819,7 +820,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
         }
         mbar_init(a0_full, 1);
         mbar_init(acc_full, 1);
-        mbar_init(a_ready, 1);
+        for (int i = 0; i < kMaxSlabs; ++i) mbar_init(a_ready(i), 1);
         mbar_init(xbar0, 1);
         mbar_init(xbar0 + 8, 1);
         mbar_init(out_bar, 1);
@@ -877,6 +878,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
     } else {
         const int r = warp * 32 + lane;
         const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
+        const int nsl = NS / SLAB;
         float* stg_w = stg + warp * 32 * STG_LD;
         const bool rebuild = P.beta[0] != nullptr;   // the ReLU mask from pre, g and beta
         if (warp > 0)
@@ -905,15 +907,13 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
             // ---------------------------------------------------------------- MMA issue
             if (warp == 0 && elect_one()) {
                 const bool gave_up = dead;
-                if (!dead) {
-                    if (st == 0) dead = !mbar_wait(a0_full, 0, err, 41, wlim);
-                    else dead = !mbar_wait<true>(a_ready, (st - 1) & 1, err, 42, wlim);
-                }
+                if (!dead && st == 0) dead = !mbar_wait(a0_full, 0, err, 41, wlim);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t idesc = idesc_bf16_kn(BM, fin ? nfin : NS);
                 int kb = 0, s = it0 % S;
                 uint32_t ph = (uint32_t)(it0 / S) & 1;
                 for (; kb < nk(st) && !dead; ++kb) {
+                    if (st > 0 && !mbar_wait<true>(a_ready(kb), (st - 1) & 1, err, 42, wlim)) { dead = true; break; }
                     if (!mbar_wait(full(s), ph, err, 43, wlim)) { dead = true; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t as = a_base + kb * SLAB_BYTES, bs = ring + s * a.stage_bytes;
@@ -1003,35 +1003,48 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
                 // the output columns, only its own slice (kept at the start) when it splits K
                 const bool bcast = CL > 1 && !(last_hidden && (ksplit || nsteps == nh));
                 const int kpos0 = (CL > 1 && last_hidden && ksplit && nsteps > nh) ? 0 : c0;
-                for (int c = 0; c < NS; c += 32) {
-                    float xh[32], v[32];
-                    {
-                        float dxh[32];
-                        tmem_ld32(trow + NS + c, xh);
-                        tmem_ld32(trow + 2 * NS + c, dxh);
+                // the slabs that peers send
+                if (bcast && warp == 1 && lane < hslabs && lane / nsl != rank) mbar_expect_tx(a_ready(lane), SLAB_BYTES);
+                // slab by slab, as in the forward (a slice is whole slabs)
+                for (int sl = 0; sl < nsl; ++sl) {
+                    for (int c = sl * SLAB; c < (sl + 1) * SLAB; c += 32) {
+                        float xh[32], v[32];
+                        {
+                            float dxh[32];
+                            tmem_ld32(trow + NS + c, xh);
+                            tmem_ld32(trow + 2 * NS + c, dxh);
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) v[j] = rstd * (dxh[j] - m1 - xh[j] * m2);   // dpre
+                            for (int j = 0; j < 32; ++j) v[j] = rstd * (dxh[j] - m1 - xh[j] * m2);   // dpre
+                        }
+                        if (s_col) colacc[(warp * 3 + 2) * NS + c + lane] = warp_col_sum(stg_w, v, lane);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int k = kpos0 + c + 8 * u;
+                            uint4 w;
+                            w.x = pack_bf16(v[8 * u], v[8 * u + 1]);
+                            w.y = pack_bf16(v[8 * u + 2], v[8 * u + 3]);
+                            w.z = pack_bf16(v[8 * u + 4], v[8 * u + 5]);
+                            w.w = pack_bf16(v[8 * u + 6], v[8 * u + 7]);
+                            *reinterpret_cast<uint4*>(smem + (k / SLAB) * SLAB_BYTES + r * 128 +
+                                                      ((((k % SLAB) / 8) ^ (r & 7)) * 16)) = w;
+                        }
                     }
-                    if (s_col) colacc[(warp * 3 + 2) * NS + c + lane] = warp_col_sum(stg_w, v, lane);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int k = kpos0 + c + 8 * u;
-                        uint4 w;
-                        w.x = pack_bf16(v[8 * u], v[8 * u + 1]);
-                        w.y = pack_bf16(v[8 * u + 2], v[8 * u + 3]);
-                        w.z = pack_bf16(v[8 * u + 4], v[8 * u + 5]);
-                        w.w = pack_bf16(v[8 * u + 6], v[8 * u + 7]);
-                        *reinterpret_cast<uint4*>(smem + (k / SLAB) * SLAB_BYTES + r * 128 +
-                                                  ((((k % SLAB) / 8) ^ (r & 7)) * 16)) = w;
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    epi_bar();
+                    if (threadIdx.x == 0) {
+                        const int slab = kpos0 / SLAB + sl;
+                        const uint32_t src = a_base + slab * SLAB_BYTES;
+                        if (bcast)
+                            for (int q = 0; q < CL; ++q)
+                                if (q != rank) bulk_s2s(mapa(src, q), src, SLAB_BYTES, mapa(a_ready(slab), q));
+                        mbar_arrive_local(a_ready(slab));
+                        if (s_dp) {
+                            tma_store_2d(&P.tdp[lh], src, c0 + sl * SLAB, m0);
+                            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                        }
                     }
                 }
-                if (H % SLAB)
-                    for (int k = H; k < hslabs * SLAB; k += 8)
-                        *reinterpret_cast<uint4*>(smem + (k / SLAB) * SLAB_BYTES + r * 128 +
-                                                  ((((k % SLAB) / 8) ^ (r & 7)) * 16)) = make_uint4(0u, 0u, 0u, 0u);
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                epi_bar();
                 if (s_col) {   // this row block's column sums of the slice, warps added in order
                     for (int i = threadIdx.x; i < 3 * NS; i += BM) {
                         const int k = i / NS, j = i % NS;
@@ -1040,21 +1053,6 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
                         s_col[((int64_t)rb * 3 + k) * H + c0 + j] = t;
                     }
                     epi_bar();   // read before the next layer's column sums overwrite them
-                }
-                if (threadIdx.x == 0) {
-                    if (s_dp) {
-                        for (int j = 0; j < (NS + SLAB - 1) / SLAB; ++j)
-                            tma_store_2d(&P.tdp[lh], a_base + (kpos0 / SLAB + j) * SLAB_BYTES, c0 + j * SLAB, m0);
-                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                    }
-                    if (bcast) {
-                        const uint32_t src = a_base + (c0 / SLAB) * SLAB_BYTES, bytes = (uint32_t)NS * 256;
-                        for (int q = 0; q < CL; ++q)
-                            if (q != rank) bulk_s2s(mapa(src, q), src, bytes, mapa(a_ready, q));
-                        mbar_expect_tx(a_ready, (uint32_t)(CL - 1) * bytes);
-                    } else {
-                        mbar_arrive_local(a_ready);
-                    }
                 }
             } else if (!ksplit) {
                 // ------------------------------------------------------------ final step, split over columns
@@ -1103,7 +1101,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
     __syncthreads();
     if (threadIdx.x == 0)
         for (int i = (int)slot[2]; i < (int)slot[1]; ++i) mbar_wait(full(i % S), (i / S) & 1, err, 47, wlim);
-    if (CL > 1) cluster_sync_all();
+    if (CL > 1) cluster_leave();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0) {
@@ -1187,6 +1185,7 @@ bool plan_bwd(int H, int CL, int nh, int nko, int nfin, bool ksplit, int* a_byte
     if (ksplit && CL > 1) *a_bytes = std::max(*a_bytes, (NS * 256 + BM * *ldr * 4 + 1023) / 1024 * 1024);
     *stage_bytes = std::max(NS, nfin) * 128;
     const int fixed = 1024 + STG_BYTES + 2 * CL * BM * 2 * 4 + 4 * 3 * NS * 4 + ((2 * nh * NS + 3) / 4) * 16 + 256;
+    if (hs > kMaxSlabs) return false;
     const int n = (SMEM_LIMIT - fixed - *a_bytes) / *stage_bytes;
     *stages = std::min(n, 8);
     *smem = fixed + *a_bytes + *stages * *stage_bytes;
