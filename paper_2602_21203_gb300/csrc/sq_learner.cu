@@ -513,7 +513,7 @@ bool mlp_backward(squint_handle* h, const MlpBufs& mb, int r0, const MlpRef* set
             lb[e] = p;
         }
         {
-            ProfScope ps(h, s, "layernorm_bwd", 4.0 * E * rows * sets[0][l].out * (grads ? 9.0 : 5.0), 1);
+            ProfScope ps(h, s, "layernorm_bwd", 4.0 * E * rows * sets[0][l].out * ((grads ? 9.0 : 5.0) - (mb.tc_saved ? 1.0 : 0.0)), 1);
             launch_ln_bwd(lb, E, h->ln_work, s);
         }
         if (grads) {
