@@ -130,9 +130,12 @@ __device__ __forceinline__ void fragment(float (&f)[T][4], const float* s, int t
     }
 }
 
-// BM x BN outputs a CTA, TM x TN a thread (TM, TN in {2, 4}); a warp covers 4 x 8 threads.
+// BM x BN outputs a CTA, TM x TN a thread (TM, TN in {2, 4}); a warp covers 4 x 8 threads.  Three
+// CTAs of the large tile to an SM: left to itself the compiler takes 254 registers where A and B
+// are contiguous in m and n, two CTAs, and 328 tiles (M 256, N 2592, K 512) wait for a second
+// wave: 30.2 us, 26.7 with three.  (Four: 26.7 too, but the FP32 update 5,167 us against 5,069.)
 template <int BM, int BN, int TM, int TN, int BK, bool A_K, bool B_K>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN)) gemm_f32_kernel(const __grid_constant__ GemmF32Batch gb) {
+__global__ void __launch_bounds__((BM / TM) * (BN / TN), BN < 64 ? 1 : 3) gemm_f32_kernel(const __grid_constant__ GemmF32Batch gb) {
     constexpr int NTHR = (BM / TM) * (BN / TN);
     constexpr int WN = BN / (8 * TN);
     constexpr int A_FLOATS = A_K ? BM * (BK + 4) : BK * (BM + 4);
