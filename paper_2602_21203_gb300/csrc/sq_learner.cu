@@ -271,7 +271,7 @@ void mlp_forward(squint_handle* h, MlpBufs& mb, const MlpRef* sets, int E, const
             }
         }
     }
-    mb.tc_saved = false;
+    if (keep) mb.tc_saved = false;
     for (int l = 0; l <= nh; ++l) {
         // the hidden layers' LayerNorm (+ReLU) problems; on the tensor-core path the GEMM
         // computes them in its epilogue
