@@ -1232,18 +1232,20 @@ __global__ void __launch_bounds__(32 * kCastRows) cast_rows_kernel(CastBatch cb)
 
 // The same for one matrix, with the column sums of 32 rows at a time: a warp takes rows w, w + 8,
 // ... of a block's 32 in order, four columns a lane, and the block adds its warps in order into
-// part[block][cols].
-__global__ void __launch_bounds__(256) cast_colsum_kernel(CastItem c, float* __restrict__ part) {
+// part[row block][cols].  CTA b: columns 128 (b % col_tiles) on of row block b / col_tiles (a grid's
+// y dimension ends at 65,535 row blocks).
+__global__ void __launch_bounds__(256) cast_colsum_kernel(CastItem c, int col_tiles, float* __restrict__ part) {
     SQ_KERNEL_ENTRY();
     __shared__ float4 sums[8][32];
     const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
-    const int col = blockIdx.x * 128 + 4 * lane;
+    const int row_block = blockIdx.x / col_tiles, row0 = row_block * 32 + warp;
+    const int col = (blockIdx.x - row_block * col_tiles) * 128 + 4 * lane;
     const int cols = c.cols, ld = (int)c.dst_ld;
     const bool vec = ((reinterpret_cast<uintptr_t>(c.src) & 15) | (c.src_ld & 3)) == 0 && col + 3 < cols;
     float4 v[4], s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        const int r = blockIdx.y * 32 + warp + 8 * u;
+        const int r = row0 + 8 * u;
         const float* p = c.src + (int64_t)r * c.src_ld + col;
         v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (r >= c.rows) continue;
@@ -1253,7 +1255,7 @@ __global__ void __launch_bounds__(256) cast_colsum_kernel(CastItem c, float* __r
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        const int r = blockIdx.y * 32 + warp + 8 * u;
+        const int r = row0 + 8 * u;
         s.x += v[u].x; s.y += v[u].y; s.z += v[u].z; s.w += v[u].w;
         if (r >= c.rows) continue;
         __nv_bfloat16* d = c.dst + (int64_t)r * c.dst_ld + col;
@@ -1278,7 +1280,7 @@ __global__ void __launch_bounds__(256) cast_colsum_kernel(CastItem c, float* __r
         const float4 t = sums[w][lane];
         s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
     }
-    float* out = part + (int64_t)blockIdx.y * cols + col;
+    float* out = part + (int64_t)row_block * cols + col;
     const float f[4] = {s.x, s.y, s.z, s.w};
 #pragma unroll
     for (int k = 0; k < 4; ++k)
@@ -1291,7 +1293,8 @@ int64_t cast_colsum_workspace(int rows, int cols) { return (int64_t)((rows + 31)
 void launch_cast_colsum(const CastItem& c, float* out, float* work, cudaStream_t s) {
     const int blocks = (c.rows + 31) / 32;
     if (!blocks || !c.cols) return;
-    launch_k(cast_colsum_kernel, dim3((unsigned)((c.dst_ld + 127) / 128), blocks), dim3(256), 0, s, c, work);
+    const int col_tiles = (int)((c.dst_ld + 127) / 128);
+    launch_k(cast_colsum_kernel, dim3((unsigned)((int64_t)blocks * col_tiles)), dim3(256), 0, s, c, col_tiles, work);
     const ColSumProblem p{blocks, c.cols, work, c.cols, out};
     launch_colsum(&p, 1, s);
 }

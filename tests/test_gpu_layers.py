@@ -128,3 +128,23 @@ def test_ce_mean(rows, K):
     got = ops.ce_mean_bwd(logits, m, torch.full((), 0.75, device="cuda"))
     # the same products with the scale rounded on the device: one more rounding of 0.75 / rows
     assert bool(((got - d).abs() <= 2 * U * d.abs() + 1e-45).all())
+
+
+# one row block (32 rows) more than a grid's y dimension counts
+MANY = 32 * 65535 + 1
+
+
+def test_linear_bf16_backward_over_many_rows():
+    from paper_2602_21203_gb300 import ops
+    x, w, dy = _rand(MANY, 8, seed=1), _rand(9, 8, seed=2), _rand(MANY, 9, seed=3)
+    _, xs, ws = ops.linear_bf16_fwd(x, w, None)
+    _dirty()
+    dx, dw, db = ops.linear_bf16_bwd(dy, xs, ws)
+    dyh = ops.cast_bf16(dy)
+    assert torch.equal(dx, ops.gemm(dyh, ws.t(), M=MANY, N=8, K=9))
+    assert torch.equal(dw, ops.gemm(dyh.t(), xs.t(), M=9, N=8, K=MANY))
+    _sum_close(db, dy, MANY)
+
+
+def test_mlp_head_backward_over_many_rows():
+    test_mlp_head_layer(MANY, 8, 32, 1, 3)
