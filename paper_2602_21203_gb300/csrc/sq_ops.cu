@@ -19,6 +19,9 @@ namespace {
 
 int launch_status() { return cudaGetLastError() == cudaSuccess ? SQUINT_OK : SQUINT_ECUDA; }
 
+// The error flag of the tensor-core kernels; the first call sets their attributes.  Anything that
+// sets a kernel's attributes comes before a call's first launch: cudaFuncSetAttribute takes back a
+// refused launch's error, and launch_status() would not see it.
 int* tc_error_flag() {
     static int* flag = nullptr;
     static std::once_flag once;
@@ -210,6 +213,8 @@ int squint_op_gemm_fp8(int M, int N, int K, const void* A, int64_t lda, const vo
         return SQUINT_EINVAL;
     }
     if (M == 0 || N == 0) return SQUINT_OK;
+    int* err = tc_error_flag();
+    if (!err) return SQUINT_ECUDA;
     cudaStream_t s = (cudaStream_t)stream;
     char* w = static_cast<char*>(work);
     float* part = reinterpret_cast<float*>(w);
@@ -226,8 +231,6 @@ int squint_op_gemm_fp8(int M, int N, int K, const void* A, int64_t lda, const vo
     g.b[0] = TcOperand{b8, pad16(K), false};
     g.bias = bias; g.c = C; g.ldc = ldc;
     g.fp8 = 1; g.scale_a = scales; g.scale_b = scales + 1;
-    int* err = tc_error_flag();
-    if (!err) return SQUINT_ECUDA;
     if (launch_tc_gemm(&g, 1, err, s) != 0) return SQUINT_EINVAL;
     return launch_status();
 }
@@ -461,13 +464,13 @@ int squint_op_linear_bf16_fwd(int M, int N, int K, const float* x, int64_t ldx, 
     if (M < 0 || N < 1 || K < 1 || !x || !w || !xh || !wh || !y || ldx < K || ldw < K || ldxh < K || ldwh < K)
         return SQUINT_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
+    int* err = tc_error_flag();
+    if (!err) return SQUINT_ECUDA;
     const CastItem it[2] = {{x, ldx, M, K, (__nv_bfloat16*)xh, ldxh}, {w, ldw, N, K, (__nv_bfloat16*)wh, ldwh}};
     launch_cast_rows(it, 2, s);
     if (M == 0) return launch_status();
     TcGemm g{};
     bf16_problem(M, N, K, xh, ldxh, 1, wh, ldwh, 1, y, N, bias, 0, &g);
-    int* err = tc_error_flag();
-    if (!err) return SQUINT_ECUDA;
     if (launch_tc_gemm(&g, 1, err, s) != 0) return SQUINT_EINVAL;
     return launch_status();
 }
@@ -531,6 +534,7 @@ int squint_op_mlp_head_fwd(int M, int kin, int nh, int H, int nout, const float*
         it[l + 1] = CastItem{w[l], ldw[l], rows, cols, (__nv_bfloat16*)wh[l], ldwh[l]};
         whc[l] = wh[l];
     }
+    if (!tc_error_flag()) return SQUINT_ECUDA;
     launch_cast_rows(it, nh + 2, (cudaStream_t)stream);
     return squint_op_mlp_bf16(M, kin, nh, H, nout, xh, ldxh, whc, ldwh, bias, g, beta, eps, out, nout, pre, post, post_bf,
                               mean, rstd, 0, stream);
@@ -578,9 +582,9 @@ int squint_op_mlp_head_bwd(int M, int kin, int nh, int H, int nout, const float*
     auto f32 = [&](size_t off) { return reinterpret_cast<float*>(base + off); };
     auto width = [&](int l) { return l == nh ? nout : H; };
     auto ldh = [&](int l) { return (int64_t)(width(l) + 7) / 8 * 8; };
+    ln_prepare();
     const CastItem top{dout, nout, M, nout, (__nv_bfloat16*)(base + p.dyh[nh]), ldh(nh)};
     launch_cast_colsum(top, db[nh], f32(p.part), s);
-    ln_prepare();
     TcGemm wg[kMlpMaxHidden + 1] = {};
     LnBwdProblem ln[kMlpMaxHidden] = {};
     for (int l = nh; l >= 0; --l) {
@@ -610,6 +614,7 @@ int squint_op_mlp_head_bwd(int M, int kin, int nh, int H, int nout, const float*
 int squint_op_conv32_layer_fwd(int nimg, int H, int W, const float* x, const float* w, const float* bias, int relu, void* xp,
                                void* w_fwd, void* w_bwd, float* y, void* stream) {
     if (nimg < 0 || H < 3 || W < 3 || !x || !w || !bias || !xp || !w_fwd || !w_bwd || !y) return SQUINT_EINVAL;
+    if (!tc_error_flag()) return SQUINT_ECUDA;
     launch_to_phwc_whole(x, nullptr, nimg, H, W, (__nv_bfloat16*)xp, (cudaStream_t)stream);
     launch_conv_weight_cast(w, (__nv_bfloat16*)w_fwd, (__nv_bfloat16*)w_bwd, (cudaStream_t)stream);
     return squint_op_conv32(0, nimg, H, W, xp, w_fwd, bias, relu, nullptr, nullptr, y, stream);
@@ -618,6 +623,7 @@ int squint_op_conv32_layer_fwd(int nimg, int H, int W, const float* x, const flo
 int squint_op_conv32_layer_bwd(int nimg, int H, int W, const float* dy, const float* y, const void* xp, const void* w_bwd,
                                void* dyp, float* dx, float* dw, float* db, void* work, size_t work_bytes, void* stream) {
     if (nimg < 1 || H < 3 || W < 3 || !dy || !xp || !w_bwd || !dyp || !dw || !db) return SQUINT_EINVAL;
+    if (!tc_error_flag()) return SQUINT_ECUDA;
     launch_to_phwc_whole(dy, y, nimg, H - 2, W - 2, (__nv_bfloat16*)dyp, (cudaStream_t)stream);
     if (dx) {
         const int rc = squint_op_conv32(1, nimg, H - 2, W - 2, dyp, w_bwd, nullptr, 0, nullptr, nullptr, dx, stream);
