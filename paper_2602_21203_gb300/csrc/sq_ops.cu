@@ -523,16 +523,22 @@ int squint_op_mlp_head_fwd(int M, int kin, int nh, int H, int nout, const float*
                            float eps, void* xh, int64_t ldxh, void* const* wh, const int64_t* ldwh, float* out,
                            float* const* pre, float* const* post, void* const* post_bf, float* const* mean,
                            float* const* rstd, void* stream) {
-    if (M < 0 || kin < 1 || nh < 1 || nh > kMlpMaxHidden || H < 1 || nout < 1 || !x || !w || !ldw || !xh || !wh || !ldwh)
+    if (M < 0 || kin < 1 || nh < 1 || nh > kMlpMaxHidden || H < 1 || nout < 1 || !x || !w || !ldw || !bias || !g || !beta ||
+        !xh || !wh || !ldwh || !out || ldx < kin || ldxh < kin)
         return SQUINT_EINVAL;
     CastItem it[kMlpMaxHidden + 2];
     it[0] = CastItem{x, ldx, M, kin, (__nv_bfloat16*)xh, ldxh};
     const void* whc[kMlpMaxHidden + 1];
     for (int l = 0; l <= nh; ++l) {
         const int rows = l == nh ? nout : H, cols = l == 0 ? kin : H;
-        if (!w[l] || !wh[l] || ldw[l] < cols || ldwh[l] < cols) return SQUINT_EINVAL;
+        if (!w[l] || !wh[l] || !bias[l] || (l < nh && (!g[l] || !beta[l])) || ldw[l] < cols || ldwh[l] < cols)
+            return SQUINT_EINVAL;
         it[l + 1] = CastItem{w[l], ldw[l], rows, cols, (__nv_bfloat16*)wh[l], ldwh[l]};
         whc[l] = wh[l];
+    }
+    if (!mlp_tc_supported(nh, H, nout, kin)) {   // (refused before anything is cast)
+        g_last_error = "fused MLP: shape outside the kernel's range";
+        return SQUINT_EINVAL;
     }
     if (!tc_error_flag()) return SQUINT_ECUDA;
     launch_cast_rows(it, nh + 2, (cudaStream_t)stream);

@@ -103,3 +103,21 @@ def test_invalid_configs_are_rejected_without_a_device(lib):
     assert L.squint_update(None, 1, None, None) == lib.EINVAL
     assert L.squint_set_debug(None, b"wait_cycles", 100) == lib.EINVAL
     assert L.squint_strerror(lib.ETIMEOUT).decode() == "timed out"
+
+
+# (argument, value): what the single casts and the fused head refuse, the one-call layer refuses before it launches anything
+@pytest.mark.parametrize("arg,value", [("ldx", 17), ("ldx", 0), ("ldxh", 17), ("kin", 0), ("H", 33), ("nout", 257), ("nh", 4), ("M", -1),
+                                       ("ldw", (17, 32)), ("ldwh", (24, 31)), ("bias", (None, 64)), ("g", (None,)), ("beta", None),
+                                       ("x", None), ("out", None)])
+def test_mlp_head_layer_checks_its_arguments(lib, arg, value):
+    L = lib.load()
+    P, I64 = ctypes.c_void_p, ctypes.c_int64
+    a = dict(M=4, kin=18, nh=1, H=32, nout=5, x=64, ldx=18, w=(64, 64), ldw=(18, 32), bias=(64, 64), g=(64,), beta=(64,), xh=64,
+             ldxh=24, wh=(64, 64), ldwh=(24, 32), out=64)
+    a[arg] = value
+    arr = lambda t, v: None if v is None else (t * len(v))(*v)
+    rc = L.squint_op_mlp_head_fwd(a["M"], a["kin"], a["nh"], a["H"], a["nout"], a["x"], a["ldx"], arr(P, a["w"]), arr(I64, a["ldw"]),
+                                  arr(P, a["bias"]), arr(P, a["g"]), arr(P, a["beta"]), 1e-5, a["xh"], a["ldxh"], arr(P, a["wh"]),
+                                  arr(I64, a["ldwh"]), a["out"], None, None, None, None, None, None)
+    assert rc == L.squint_op_cast_bf16(4, 18, 64, 17, 64, 24, None)     # SQUINT_EINVAL: rows that overlap
+    assert rc != 0
