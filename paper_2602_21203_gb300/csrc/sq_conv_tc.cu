@@ -235,12 +235,13 @@ __global__ void __launch_bounds__(kConvThreads) conv32_tc_kernel(const __grid_co
         for (int j = 0; j < kCh; ++j) bias_r[j] = a.bias ? a.bias[j] : 0.f;
         for (int i = 0; i < n_local; ++i) {
             const int b = i & 1;
-            const bool have = mbar_wait(tfull0 + 8 * b, (i >> 1) & 1, a.err, 12);
+            const bool have = __all_sync(0xffffffffu, mbar_wait(tfull0 + 8 * b, (i >> 1) & 1, a.err, 12));
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int img = (int)blockIdx.x + i * (int)gridDim.x;
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
                 if (t >= a.n_tiles || !have) break;
+                __syncwarp();   // (the lanes without a pixel in the tile before)
                 uint32_t r0[16], r1[16];
                 const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + b * (uint32_t)a.tmem_cols + t * kCh;
                 tmem_ld16(taddr, r0);
@@ -745,7 +746,7 @@ __global__ void __launch_bounds__(128, PL == 4 ? 5 : 2) conv0_tc_kernel(const __
         if (i > 0 && ok) {
             // the MMAs of tile i - 1 (and so of tile i - 2, which read buffer b) are complete
             const int pb = b ^ 1;
-            ok = mbar_wait(bar0 + 8 * pb, ((i - 1) >> 1) & 1, a.err, 17);
+            ok = __all_sync(0xffffffffu, mbar_wait(bar0 + 8 * pb, ((i - 1) >> 1) & 1, a.err, 17));
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (ok) drain(t - (int)gridDim.x, pb);
         }
@@ -765,7 +766,7 @@ __global__ void __launch_bounds__(128, PL == 4 ? 5 : 2) conv0_tc_kernel(const __
     }
     if (n_local > 0) {
         const int i = n_local - 1, b = i & 1;
-        if (mbar_wait(bar0 + 8 * b, (i >> 1) & 1, a.err, 18) && ok) {
+        if (__all_sync(0xffffffffu, mbar_wait(bar0 + 8 * b, (i >> 1) & 1, a.err, 18)) && ok) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             drain((int)blockIdx.x + i * (int)gridDim.x, b);
         }
@@ -962,9 +963,9 @@ __global__ void __launch_bounds__(128 * kEncGroups, 1) encoder_tc_kernel(const _
                             for (int j = 0; j < 16; ++j) a.z_bf[base + j * px] = __float2bfloat16_rn(v[j]);
                         }
                     }
+                }
+                __syncwarp();   // tensor memory is read by whole warps: lanes without a pixel wait for the others
             }
-            }
-            __syncwarp();
         }
     };
 

@@ -158,6 +158,7 @@ __device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
 // The end of a kernel: no CTA passes before all have arrived.  Orders no memory: what peers sent
 // has completed on this CTA's barriers.
 __device__ __forceinline__ void cluster_leave() {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.relaxed.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
@@ -573,6 +574,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) mlp_tc_kernel(const __grid_con
                             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                         }
                     }
+                    __syncwarp();   // (the next slab's tensor-memory load takes the whole warp)
                 }
             } else {
                 // ------------------------------------------------------------ output layer epilogue
@@ -1044,6 +1046,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
                             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                         }
                     }
+                    __syncwarp();   // (the next slab's tensor-memory load takes the whole warp)
                 }
                 if (s_col) {   // this row block's column sums of the slice, warps added in order
                     for (int i = threadIdx.x; i < 3 * NS; i += BM) {

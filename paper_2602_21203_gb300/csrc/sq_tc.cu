@@ -817,6 +817,7 @@ __global__ void __launch_bounds__(128) tc_gemm64_kernel(const __grid_constant__ 
             acc[i] = make_float4(b.x + x.x, b.y + x.y, b.z + x.z, b.w + x.w);
         }
         finish_rows(acc, nv > 0 ? rows_left : 0, row0, col, nv, out);
+        __syncwarp();   // (lanes at the tile's edge part there; the next load takes the whole warp)
     }
     // copies issued but not consumed (after a wait gave up) still land here before the CTA leaves
     __syncthreads();
