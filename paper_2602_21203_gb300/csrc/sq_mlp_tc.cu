@@ -475,6 +475,10 @@ __global__ void __launch_bounds__(kFwdThreads, 1) mlp_tc_kernel(const __grid_con
                         }
                     }
                 }
+                // the previous layer's TMA stores have read this CTA's slabs: before this CTA rewrites them,
+                // and before thread 0 sends its row's statistics, without which no peer gets as far as
+                // its partial outputs, which land where the slabs of the layer before lie
+                if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                 // the whole row's statistics: every CTA sends (mean, M2) of its slice to every
                 // CTA of the cluster; they are combined in rank order (Chan et al.'s pairwise
                 // update for equal counts: M2 = sum M2_q + NS sum (mean_q - mean)^2)
@@ -502,8 +506,6 @@ __global__ void __launch_bounds__(kFwdThreads, 1) mlp_tc_kernel(const __grid_con
                     buf[2 * r] = mean;
                     buf[2 * r + 1] = var;
                 }
-                // the previous layer's TMA store has read this CTA's slabs before they are rewritten
-                if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                 fwd_bar();
                 if (CL == 1 && set) {
                     mean = buf[2 * r];
@@ -982,6 +984,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
                     tmem_st32(trow + 2 * NS + c, t);
                 }
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                // the previous layer's TMA stores have read this CTA's slabs: before this CTA rewrites them,
+                // and before thread 0 sends its row's sums, without which no peer gets as far as
+                // its partial results, which land where the slabs of the step before lie
+                if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                 if (CL > 1) {
                     const int b = st & 1;
                     float* buf = xbuf + b * CL * BM * 2;
@@ -997,8 +1003,6 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
                     }
                 }
                 const float m1 = s1 / (float)H, m2 = s2 / (float)H;
-                // the previous layer's TMA store has read this CTA's slabs before they are rewritten
-                if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                 epi_bar();
                 const bool last_hidden = lh == 0;
                 // dpre_0 feeds the final step: every CTA needs all of it when that step splits
