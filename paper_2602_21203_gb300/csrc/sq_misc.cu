@@ -457,23 +457,26 @@ __global__ void __launch_bounds__(32 * kHeadRows) ce_kernel(CeArgs a) {
     }
 }
 
+// Each value is scaled by a power of two to at most 1 / n before it is added (exactly, but for
+// subnormal results), so that the sum does not overflow where the mean does not.
 __global__ void __launch_bounds__(512) mean_kernel(const float* __restrict__ v, int n, float* __restrict__ out) {
     SQ_KERNEL_ENTRY();
     __shared__ float part[16];
+    const float unit = __uint_as_float((127u - (n > 1 ? 32 - __clz(n - 1) : 0)) << 23);
     float s = 0.f;
     for (int i0 = threadIdx.x; i0 < n; i0 += 4 * 512) {   // four loads in flight, added in order
         float x[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) x[u] = i0 + 512 * u < n ? v[i0 + 512 * u] : 0.f;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) s += x[u];
+        for (int u = 0; u < 4; ++u) s += unit * x[u];
     }
     s = warp_sum(s);
     if (threadIdx.x % 32 == 0) part[threadIdx.x / 32] = s;
     __syncthreads();
     if (threadIdx.x >= 32) return;
     s = warp_sum(threadIdx.x < 16 ? part[threadIdx.x] : 0.f);
-    if (threadIdx.x == 0) *out = s / (float)n;
+    if (threadIdx.x == 0) *out = s / (unit * (float)n);
 }
 
 // Actor objective through the critics, one warp per sample over all critics:

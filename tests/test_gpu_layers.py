@@ -148,3 +148,11 @@ def test_linear_bf16_backward_over_many_rows():
 
 def test_mlp_head_backward_over_many_rows():
     test_mlp_head_layer(MANY, 8, 32, 1, 3)
+
+
+def test_ce_mean_of_losses_whose_sum_overflows():
+    from paper_2602_21203_gb300 import ops
+    rows = 600
+    logits, m = torch.zeros(rows, 3, device="cuda"), torch.zeros(rows, 3, device="cuda")
+    logits[:, 1], m[:, 1] = -3e36, 1.0      # every row's loss is 3e36 + log 2
+    assert abs(float(ops.ce_mean(logits, m)) / 3e36 - 1) <= (rows + 4) * U
