@@ -284,9 +284,12 @@ __device__ float block_sum(float v, float* sh) {
 // (1-d)(Q_bar - alpha log pi') with Q_bar the average (or, with clipped double Q, the
 // minimum) of the target outputs.  Softmax statistics by warp shuffles, no block barrier.
 constexpr int kHeadRows = 8;   // samples a block of the other per-sample kernels
-// The target's projection walks all K atoms for each of a lane's V: one warp a scheduler, and one
-// read of an atom for the V of them (512 rows of 101 atoms, two critics, in the update, waiting for
-// its inputs included: 13.0 us with eight rows a block and a walk for each, 11.8 now).
+// The target's projection walks all K atoms for each of a lane's V: one read of an atom for the V
+// of them, and V no more than K needs, because lanes beyond K multiply too (100,000 rows of 51 atoms, two
+// critics: 87 us; 126 with V = 4 for every K up to 128, 98 with a walk for each atom; of 139 atoms 337,
+// 484 with V = 8 and 421).  Four rows a block, one warp a scheduler for a batch's worth of rows (512
+// rows of 101 atoms in the update, waiting for its inputs included: 13.0 us with eight rows a block and
+// a walk for each, 11.8 now).
 constexpr int kC51Rows = 4;
 
 template <int V>
@@ -1031,12 +1034,22 @@ void launch_actor_head(const ActorHeadArgs& a, cudaStream_t s) {
 void launch_actor_head_bwd(const ActorHeadBwdArgs& a, cudaStream_t s) {
     launch_k(actor_head_bwd_kernel, dim3((unsigned)(((int64_t)a.B * a.A + 127) / 128)), dim3(128), 0, s, a);
 }
-// atoms per lane: 4 up to 128 atoms, 8 up to 256 (the most a configuration takes)
+// atoms per lane: as many as K needs, up to the 8 of 256 atoms (the most a configuration takes)
 void launch_c51_target(const C51TargetArgs& a, cudaStream_t s) {
     const dim3 g((a.B + kC51Rows - 1) / kC51Rows), t(32 * kC51Rows);
-    if (a.K <= 128) launch_k(c51_target_kernel<4>, g, t, 0, s, a);
-    else launch_k(c51_target_kernel<8>, g, t, 0, s, a);
+    switch ((a.K + 31) / 32) {
+        case 0:   // (scalar critics: K = 1 takes the branch without atoms)
+        case 1: launch_k(c51_target_kernel<1>, g, t, 0, s, a); break;
+        case 2: launch_k(c51_target_kernel<2>, g, t, 0, s, a); break;
+        case 3: launch_k(c51_target_kernel<3>, g, t, 0, s, a); break;
+        case 4: launch_k(c51_target_kernel<4>, g, t, 0, s, a); break;
+        case 5: launch_k(c51_target_kernel<5>, g, t, 0, s, a); break;
+        case 6: launch_k(c51_target_kernel<6>, g, t, 0, s, a); break;
+        case 7: launch_k(c51_target_kernel<7>, g, t, 0, s, a); break;
+        default: launch_k(c51_target_kernel<8>, g, t, 0, s, a); break;
+    }
 }
+// atoms per lane: 4 up to 128 atoms, 8 up to 256
 void launch_ce(const CeArgs& a, cudaStream_t s) {
     const dim3 g((a.E * a.B + kHeadRows - 1) / kHeadRows), t(32 * kHeadRows);
     if (a.K <= 128) launch_k(ce_kernel<4>, g, t, 0, s, a);

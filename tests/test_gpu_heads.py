@@ -59,3 +59,9 @@ def test_categorical_target(rows, E, K):
     tol = (8 * (2 * K) * U * 4 + (16 + K) * U) * 1.0
     assert float((m.double() - want).abs().max()) <= tol
     assert float((m.double().sum(1) - 1).abs().max()) <= K * tol
+
+
+# both ends of every count of atoms a lane
+@pytest.mark.parametrize("K", [32, 64, 65, 96, 97, 160, 161, 192, 193, 224, 225])
+def test_categorical_target_atoms_a_lane(K):
+    test_categorical_target(13, 2, K)
