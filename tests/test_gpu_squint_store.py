@@ -35,3 +35,10 @@ def test_squint_store_bit_exact(n, c, h, w, f, off_src, off_ring):
         want[(torch.arange(n, device="cuda") + slot0) % slots] = _ref(frames, f)
         assert torch.equal(ring, want)
         assert bool((rbuf[:off_ring] == 99).all()) and bool((rbuf[off_ring + slots * per:] == 99).all())
+
+
+# rows just too short and just long enough for the staged kernel
+@pytest.mark.parametrize("w,f", [(12, 2), (14, 2), (24, 4), (28, 4), (36, 6), (2, 2), (4, 4)])
+def test_squint_store_short_rows(w, f):
+    test_squint_store_bit_exact(37, 3, 5 * f, w, f, 3, 1)
+    test_squint_store_bit_exact(37, 3, 5 * f, w, f, 0, 0)
