@@ -297,17 +297,44 @@ void launch_layout(GemmF32Batch& gb, cudaStream_t s) {
     else launch_tiles<16, 32, 2, 2, 32, A_K, B_K>(gb, s);
 }
 
+// Where gemm_kernel (sq_gemm.cu) is the faster of the two (the bits are the same): grids of more than
+// three CTAs an SM whose CTAs have little K to pipeline over.  It pads K to 16 steps, not 32, and more of
+// its threads fit an SM; and a stage of the ring costs more where an operand contiguous in K has rows
+// that are copied 4 or 8 bytes at a time.  Ring against gemm_kernel in us, M 6000, N 1800 (5,358 tiles of
+// 32 x 64): K 16 45 and 31, 48 58 and 54, 52 57 and 66; with both operands' rows of odd length K 33 84 and
+// 52, 97 131 and 102, 161 176 and 152, 257 242 and 225 (within 5 % on smaller grids: left to the ring),
+// 513 409 and 424; with B's alone K 33 78 and 52, 129 141 and 127, 161 162 and 152.  456 tiles or fewer are
+// never slower in the ring (M = N = 512: 6.4 and 11.5); between 641 and 1,000 it fills its second wave
+// and gemm_kernel does not, and only the shortest narrow rows lose (K 17: 1.2 times); just above 456 it has
+// a nearly empty second wave, and K up to 32, where that is short, stays.
+bool general_is_faster(int64_t tiles, int64_t K, bool a_k, bool b_k, int va, int vb) {
+    if (tiles <= 456) return false;
+    const bool na = a_k && va < 4, nb = b_k && vb < 4;   // K-contiguous rows in narrow copies
+    int limit = nb ? (na ? 100 : 70) : na ? 65 : 48;
+    if (tiles <= 640) return K > 32 && K <= limit;
+    if (tiles <= 1000) return nb && K <= 33;
+    if (nb && tiles > 2400) limit = na ? (va == 1 && vb == 1 ? 200 : 130) : vb == 1 ? 140 : 100;
+    return K <= limit;
+}
+
 }  // namespace
 
 bool launch_gemm_f32(const GemmProblem* probs, int n_probs, cudaStream_t s) {
     GemmF32Batch gb;
     if (n_probs < 1) return false;
     const bool a_k = probs[0].sa_k == 1, b_k = probs[0].sb_k == 1;
+    int64_t tiles = 0, steps = 0;   // of the call; the longest chain over K
+    int va = 4, vb = 4;             // the narrowest copies
     for (int i = 0; i < n_probs; ++i) {
         const GemmProblem& p = probs[i];
         if ((p.sa_k == 1) != a_k || (p.sb_k == 1) != b_k || (!a_k && p.sa_m != 1) || (!b_k && p.sb_n != 1)) return false;
         if (!copy_width(p.A, 0, 0) || !copy_width(p.B, 0, 0)) return false;
+        tiles += (int64_t)((p.M + 31) / 32) * ((p.N + 63) / 64);
+        steps = std::max(steps, (int64_t)p.K * std::max(1, p.n_sum));
+        va = std::min(va, copy_width(p.A, a_k ? p.sa_m : p.sa_k, p.n_sum > 1 ? p.a_sum : 0));
+        vb = std::min(vb, copy_width(p.B, b_k ? p.sb_n : p.sb_k, p.n_sum > 1 ? p.b_sum : 0));
     }
+    if (general_is_faster(tiles, steps, a_k, b_k, va, vb)) return false;
     for (int base = 0; base < n_probs; base += kMaxGroup) {
         gb.n = std::min(kMaxGroup, n_probs - base);
         for (int i = 0; i < gb.n; ++i) {

@@ -50,3 +50,13 @@ def test_gemm_f32_non_finite_values_stay_in_their_rows():
     out = ops.gemm(A, B)
     assert bool(torch.isfinite(out[:32, :64]).all())
     assert torch.equal(torch.nan_to_num(out, 7.0), torch.nan_to_num(ops.gemm(_general(A), _general(B)), 7.0))
+
+
+# both sides of the lines between this kernel and the general one: grids of 465, 496, 722, 1,170 and 2,574 tiles, the last
+# K that changes sides and the next, rows copied 16, 8 and 4 bytes at a time
+@pytest.mark.parametrize("M,N,K", [(992, 960, 33), (992, 1024, 48), (992, 1024, 49), (992, 1024, 101), (1200, 1200, 33), (1200, 1200, 34),
+                                   (2080, 1100, 16), (2080, 1100, 48), (2080, 1100, 49), (2080, 1100, 71), (2081, 2494, 130),
+                                   (2081, 2494, 141), (2081, 2494, 201)])
+@pytest.mark.parametrize("a_k,b_k", [(True, True), (True, False), (False, True), (False, False)])
+def test_gemm_f32_large_grids(M, N, K, a_k, b_k):
+    test_gemm_f32_unit_strides(M, N, K, a_k, b_k)
