@@ -505,6 +505,13 @@ bool launch_conv_fwd_f32(const ConvShape& sh, const float* x, const float* w, co
     a.M = sh.nimg * sh.OH * sh.OW; a.N = sh.Cout; a.R = sh.Cin;
     a.in_img = sh.x_img_stride; a.in_plane = (int64_t)sh.H * sh.W; a.out_img = sh.y_img_stride;
     a.relu = relu ? 1 : 0; a.stride = sh.stride;
+    // Whole planes are staged where a stride reads parts of them, and a stage holds kChan of them: with one
+    // input channel, or few and a stride of 3 or more, conv_fwd_kernel's gather is cheaper once its CTAs fill
+    // the chip.  1,024 images of 40 x 40, here and there in us: 1 channel to 8, stride 2 32.9 and 25.4, 2 to
+    // 8 34 and 39; 3 channels to 32, stride 3 28.9 and 23.6, 9 to 48 102 and 101.
+    if ((int64_t)((a.M + 127) / 128) * ((a.N + 31) / 32) >= 800 &&
+        ((sh.Cin == 1 && sh.stride >= 2) || (sh.Cin <= 8 && sh.Cout > 8 && sh.stride >= 3)))
+        return false;
     return launch_conv<false>(a, s);
 }
 

@@ -54,3 +54,10 @@ def test_conv_f32_images_do_not_mix():
     keep = [0, 1, 2, 4]
     assert torch.equal(torch.relu(y[keep]), clean[keep])
     assert bool(torch.isnan(y[3, :, 2:5, 2:5]).all()) and not bool(torch.isnan(y[3, :, :2]).any())
+
+
+# grids on both sides of the line from which one input channel, or few and a wide stride, take the general kernel
+@pytest.mark.parametrize("n,cin,cout,h,w,s", [(1032, 1, 8, 21, 22, 2), (1020, 1, 8, 21, 22, 2), (1030, 2, 8, 21, 22, 2),
+                                              (530, 8, 40, 30, 32, 3), (500, 8, 40, 30, 32, 3), (530, 9, 40, 30, 32, 3)])
+def test_conv_f32_few_channels(n, cin, cout, h, w, s):
+    test_conv_f32_matches_fp64(n, cin, cout, h, w, s)
