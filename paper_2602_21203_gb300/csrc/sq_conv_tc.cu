@@ -138,7 +138,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-__global__ void __launch_bounds__(kConvThreads) conv32_tc_kernel(const __grid_constant__ ConvArgs a) {
+__device__ __forceinline__ void conv32_tc(const ConvArgs& a) {
     SQ_KERNEL_WAIT();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -306,6 +306,14 @@ __global__ void __launch_bounds__(kConvThreads) conv32_tc_kernel(const __grid_co
         tmem_dealloc(tmem, cols);
     }
 }
+
+// The two are one kernel compiled twice.  Bounded to two CTAs an SM (what fits), the compiler keeps
+// the bias and the pixel places in registers, 136 of them; left to itself it takes 80.  Alone the first is
+// the faster: 2,228 images of 11 x 9 16.2 us and 17.7, 4,096 of 9 x 9 24.5 and 27.4, 512 of 15 x 15 (data
+// gradient) 9.2 and 9.7.  Beside the kernels of the update's other branches, at 512 images, its registers
+// are missed there: 303.1 us an update and 301.8.
+__global__ void __launch_bounds__(kConvThreads) conv32_tc_kernel(const __grid_constant__ ConvArgs a) { conv32_tc(a); }
+__global__ void __launch_bounds__(kConvThreads, 2) conv32_tc_alone_kernel(const __grid_constant__ ConvArgs a) { conv32_tc(a); }
 
 // ---------------------------------------------------------------- weight gradient
 // D_tap[co, ci] += sum_q dy[q, co] x[q + origin(tap), ci] over the virtual grid of
@@ -1172,7 +1180,9 @@ int launch_conv32_tc(const ConvTc& c, int* err, cudaStream_t s) {
     a.out_chw = c.out_chw; a.out_chw_bf = c.out_chw_bf; a.err = err;
     const size_t smem = conv_smem(a.load_rows);
     const int ctas = std::min(c.nimg, g_num_sms * kConvCtasPerSm);
-    launch_k(conv32_tc_kernel, dim3(ctas), dim3(kConvThreads), smem, s, a);
+    // more than two images a CTA: the chip is this kernel's
+    if (c.nimg > 2 * g_num_sms * kConvCtasPerSm) launch_k(conv32_tc_alone_kernel, dim3(ctas), dim3(kConvThreads), smem, s, a);
+    else launch_k(conv32_tc_kernel, dim3(ctas), dim3(kConvThreads), smem, s, a);
     return 0;
 }
 
@@ -1224,6 +1234,7 @@ void conv_tc_prepare() {
         sms > 0)
         g_num_sms = sms;
     cudaFuncSetAttribute(conv32_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(conv32_tc_alone_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(wgrad32_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
     cudaFuncSetAttribute(encoder_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncSmem);
     cudaFuncSetAttribute(conv0_tc_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);

@@ -156,3 +156,9 @@ def test_ce_mean_of_losses_whose_sum_overflows():
     logits, m = torch.zeros(rows, 3, device="cuda"), torch.zeros(rows, 3, device="cuda")
     logits[:, 1], m[:, 1] = -3e36, 1.0      # every row's loss is 3e36 + log 2
     assert abs(float(ops.ce_mean(logits, m)) / 3e36 - 1) <= (rows + 4) * U
+
+
+# on both sides of two images a CTA
+@pytest.mark.parametrize("n", [607, 609, 1300])
+def test_conv32_layer_of_many_images(n):
+    test_conv32_layer(n, 7, 6, True)
