@@ -61,3 +61,37 @@ def test_conv_f32_images_do_not_mix():
                                               (530, 8, 40, 30, 32, 3), (500, 8, 40, 30, 32, 3), (530, 9, 40, 30, 32, 3)])
 def test_conv_f32_few_channels(n, cin, cout, h, w, s):
     test_conv_f32_matches_fp64(n, cin, cout, h, w, s)
+
+
+SMEM = 48 * 1024
+
+
+def _plan(n, channels, oh, ow, rs, pw):
+    """Pixels a thread and stages of launch_conv (sq_conv_f32.cu) for n images of oh x ow outputs read from rows pw wide."""
+    m, p = n * oh * ow, 4
+    while p > 1 and -(-m // (32 * p)) * -(-channels // 32) < 2 * 152:
+        p //= 2
+    px = 32 * p
+    words = ((-(-(px - 1) // ow) + 1) * rs + max(0, 3 - rs) * (-(-(px - 1) // (oh * ow)) + 1)) * pw
+    stage, table = 4 * (4 * 9 * 36 + 4 * words), 4 * words
+    assert 2 * stage + table <= SMEM
+    return p, 3 if 3 * stage + table <= SMEM else 2
+
+
+# four pixels a thread, forward and data gradient, where the multiplying warps stage too: the training layer; output
+# channels that are no multiple of 8 and one warp of input channels; stride 2 with an input row that no tap reads;
+# rows so wide that two stages fit; last tiles of one to four pixels a lane
+@pytest.mark.parametrize("n,cin,cout,h,w,s,stages", [(300, 32, 32, 15, 15, 1, (3, 3)), (200, 5, 44, 17, 13, 1, (3, 3)),
+                                                     (700, 3, 20, 18, 21, 2, (2, 3)), (12, 6, 9, 30, 120, 1, (2, 2)),
+                                                     (4325, 7, 32, 5, 5, 1, (3, 3))])
+def test_conv_f32_four_pixels_a_thread(n, cin, cout, h, w, s, stages):
+    oh, ow = (h - 3) // s + 1, (w - 3) // s + 1
+    assert _plan(n, cout, oh, ow, s, w) == (4, stages[0]) and _plan(n, cin, h, w, 1, w + 2) == (4, stages[1])
+    test_conv_f32_matches_fp64(n, cin, cout, h, w, s)
+
+
+@pytest.mark.parametrize("n,cin,cout,h,w,s,p", [(150, 12, 32, 15, 15, 1, 2), (100, 32, 7, 21, 19, 2, 1), (3, 40, 33, 11, 12, 1, 1)])
+def test_conv_f32_fewer_pixels_a_thread(n, cin, cout, h, w, s, p):
+    oh, ow = (h - 3) // s + 1, (w - 3) // s + 1
+    assert _plan(n, cout, oh, ow, s, w)[0] == p
+    test_conv_f32_matches_fp64(n, cin, cout, h, w, s)
