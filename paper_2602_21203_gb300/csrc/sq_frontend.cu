@@ -341,8 +341,7 @@ struct StoreArgs {
 // to, a warp sums a row, and the packed result leaves by 4-byte stores.  Bound by HBM: 4,096
 // frames of 3 x 128 x 128 at f = 4 (214 MB) 50 us, 164 us with a byte load per pixel; of 3 x 108 x
 // 108 40 us.
-// Rows too long for shared memory or too short for a warp, and other f than 1, 2 and 4, take
-// squint_store_wide_kernel.
+// Rows too long for shared memory, or that leave most of a warp idle, take squint_store_wide_kernel.
 __global__ void __launch_bounds__(256) squint_store_kernel(StoreArgs a) {
     SQ_KERNEL_ENTRY();
     extern __shared__ __align__(16) uint8_t buf[];
@@ -483,11 +482,16 @@ void launch_squint_store(const uint8_t* src, int n, int C, int H, int W, int f, 
     }
     a.block_rows = (int)std::max<int64_t>(1, std::min(12288 / row_in, (rows + 303) / 304));
     const int64_t in = (16 + a.block_rows * row_in + 15) / 16 * 16, bytes = in + (f > 1 ? a.block_rows * (W / f) + 4 : 4);
-    // Staged where a lane reads its pixels as words and a warp's lanes have outputs.  Byte reads of f x f
-    // pixels cost more from shared memory than from cache (683 frames of 3 x 120 x 24 at f = 3 18.3 us and
-    // 9.2, 506 at f = 6 14.5 and 7.9, 500 of 3 x 128 x 128 at f = 8 12.0 and 9.1), and so do rows of few
-    // outputs (2,000 frames, 40 output rows a plane at f = 2, 4 wide 24 us and 12, 6 19 and 17, 7 14 and 20).
-    if ((f == 1 || ((f == 2 || f == 4) && W / f >= 7)) && bytes <= 48 * 1024 && (rows + a.block_rows - 1) / a.block_rows < (1LL << 31)) {
+    // Staged where the lanes of a row's warp have work.  At f = 2 and 4 a lane reads its pixels as words:
+    // from 7 outputs a row on (2,000 frames, 40 output rows a plane at f = 2, here and in the wide kernel: 4
+    // wide 24 and 12 us, 6 19 and 17, 7 14 and 20).  At other f it reads bytes: where at least 5 of 8 lanes
+    // have an output, half at f = 3, and at least four of the eight warps a row (1,500 frames of some 100
+    // rows: f = 3 16 wide 26 and 29.5, f = 6 16 26 and 21, 24 29 and 30, 32 33 and 42, f = 10 30 46 and 52,
+    // 32, three rows a block, 1.1 times).
+    const int ws = W / f, lanes = (ws + 31) / 32 * 32;
+    const bool staged = f == 1 || (f == 2 || f == 4 ? ws >= 7
+                                                    : (f == 3 ? 2 * ws >= lanes : 8 * ws >= 5 * lanes) && 4 * row_in <= 12288);
+    if (staged && bytes <= 48 * 1024 && (rows + a.block_rows - 1) / a.block_rows < (1LL << 31)) {
         launch_k(squint_store_kernel, dim3((unsigned)((rows + a.block_rows - 1) / a.block_rows)), dim3(256), (size_t)bytes,
                  s, a);
         return;

@@ -42,3 +42,10 @@ def test_squint_store_bit_exact(n, c, h, w, f, off_src, off_ring):
 def test_squint_store_short_rows(w, f):
     test_squint_store_bit_exact(37, 3, 5 * f, w, f, 3, 1)
     test_squint_store_bit_exact(37, 3, 5 * f, w, f, 0, 0)
+
+
+# other factors on both sides of the share of a warp that a row has to fill
+@pytest.mark.parametrize("ws,f", [(15, 3), (16, 3), (31, 3), (33, 3), (19, 5), (20, 6), (39, 7), (40, 7), (22, 8), (30, 10), (31, 10)])
+def test_squint_store_share_of_a_warp(ws, f):
+    test_squint_store_bit_exact(11, 3, 4 * f, ws * f, f, 5, 2)
+    test_squint_store_bit_exact(11, 3, 4 * f, ws * f, f, 0, 0)
