@@ -162,3 +162,28 @@ def test_ce_mean_of_losses_whose_sum_overflows():
 @pytest.mark.parametrize("n", [607, 609, 1300])
 def test_conv32_layer_of_many_images(n):
     test_conv32_layer(n, 7, 6, True)
+
+
+def test_layer_calls_under_capture():
+    """Every one-call layer operation captured into a graph gives the bits of the same calls made at once."""
+    from paper_2602_21203_gb300 import ops
+    x, w, b, dy = _rand(40, 18, seed=1), _rand(13, 18, seed=2), _rand(13, seed=3), _rand(40, 13, seed=4)
+    hw = [_rand(64, 18, seed=5), _rand(64, 64, seed=6) / 8, _rand(13, 64, seed=7) / 8]
+    hb, hg, ht = [_rand(n, seed=8) for n in (64, 64, 13)], [1 + 0.1 * _rand(64, seed=9)] * 2, [0.1 * _rand(64, seed=10)] * 2
+    cx, cw, cb, cd = _rand(3, 32, 7, 9, seed=11), _rand(32, 32, 3, 3, seed=12) * 0.06, _rand(32, seed=13), _rand(3, 32, 5, 7, seed=14)
+    m, up = torch.softmax(_rand(40, 13, seed=15), 1), torch.full((), 0.5, device="cuda")
+
+    def calls():
+        y, xh, wh = ops.linear_bf16_fwd(x, w, b)
+        out, saved = ops.mlp_head_fwd(x, hw, hb, hg, ht)
+        cy, xp, wb = ops.conv32_layer_fwd(cx, cw, cb)
+        dx, *grads = ops.mlp_head_bwd(dy, hg, saved, 18)
+        return [y, *ops.linear_bf16_bwd(dy, xh, wh), *ops.linear_bwd(dy, x, w), out, dx, *[g for gs in grads for g in gs], cy,
+                *ops.conv32_layer_bwd(cd, cy, xp, wb), ops.ce_mean(out, m), ops.ce_mean_bwd(out, m, up)]
+    want = calls()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = calls()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert len(got) == len(want) and all(torch.equal(a, b) for a, b in zip(got, want))
