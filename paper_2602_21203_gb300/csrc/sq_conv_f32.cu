@@ -1,7 +1,10 @@
 // FP32 valid 3x3 convolutions on CUDA cores: forward, data gradient and weight gradient of
 // the plain FP32 path's encoder.
 //
-// What bounds them: the FP32 FMA rate.  The input rows of a tile of output pixels are copied
+// What bounds them: forward and data gradient the shared-memory read path (60-73 % busy beside an FMA
+// pipe at 45-55 %: the two broadcast weight reads and the input reads of a tap take more of its cycles
+// than the products take of theirs), the weight gradient the one multiplying warp a scheduler that its
+// splits leave.  The FMA rate is the floor.  The input rows of a tile of output pixels are copied
 // once into shared memory, plane by plane (cp.async, in a ring, so that the copies overlap
 // the arithmetic), and every tap reads them there: no per-tap index arithmetic, no nine-fold
 // gather.  A tile's pixels may cross rows and images: each image it touches brings the rows

@@ -657,7 +657,7 @@ __global__ void __launch_bounds__(128, PL == 4 ? 5 : 2) conv0_tc_kernel(const __
     const int opix = sh.OH * sh.OW;
 
     // inputs are read, and tensor memory taken, only once the previous kernel has finished,
-    // as in every tcgen05 kernel of the library: a kernel lets its dependents launch before
+    // as in every tcgen05 kernel of the library: a kernel may let its dependents launch before
     // it allocates, so one that allocated before its wait could hold columns its primary needs
     SQ_KERNEL_ENTRY();
     if (warp == 0) tmem_alloc(smem_u32(tmem_slot), 64);

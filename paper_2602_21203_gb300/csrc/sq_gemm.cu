@@ -572,7 +572,7 @@ void launch_conv_wgrad(const ConvShape& sh, const T* dy, const T* x, T* dw, T* d
         // the encoder's first layer: 21 us here, 37 us in sq_conv_f32.cu (512 images, 3 x 32 x 32, stride 2)
         if (sh.Cout == 32 && N <= 32) {
             // The full grid, two CTAs an SM, is not let in early: it would pack where there is room
-            // (1,024 images of 3 x 40 x 40, stride 1, after its own reduction 257 us, 201 on an even
+            // (1,024 images of 3 x 40 x 40, stride 1, after its own reduction 258 us, 206 on an even
             // chip; 512 of 3 x 20 x 20 after a ReLU backward 68 us with the forward, 55).
             launch_with(splits < 2 * 152, conv_wgrad_c32_kernel<false>, dim3(splits), dim3(128), 0, s, sh, (const void*)dy,
                         (const float*)x, (float*)work, chunk);

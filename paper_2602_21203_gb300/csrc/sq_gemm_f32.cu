@@ -10,12 +10,12 @@
 // where K is contiguous, four rows of a K step where it is not.  Every output is one
 // chain of fused multiply-adds over k ascending (no split of K), so its bits depend neither
 // on the tile nor on the rest of the batch, and equal those of gemm_kernel (sq_gemm.cu),
-// which stages synchronously: M = N = K = 512 twice 50.4 us there, 22.6 here (floor 6.7 at
-// one FMA per lane and cycle), the projections' 2048 x 256 x 2592 244 and 94 us (floor 33.7),
-// M 32, N 256, K 412 twice 39.7 and 5.7 us.  Where B's rows are contiguous in n, a read brings
+// which stages synchronously: M = N = K = 512 twice 50.4 us there, 22.5 here (floor 6.7 at
+// one FMA per lane and cycle), the projections' 2048 x 256 x 2592 244 and 88 us (floor 33.7),
+// M 32, N 256, K 412 twice 39.7 and 5.6 us.  Where B's rows are contiguous in n, a read brings
 // column pairs and products are issued in pairs: M 512, N 2592, K 256 32.8 us one by one and
-// 24.7 in pairs, N = K = 512 twice 22.6 and 20.6 (where they are contiguous in k the pairs would
-// have to be put together: 22.6 and 28.8).
+// 24.6 in pairs, N = K = 512 twice 22.5 and 20.5 (where they are contiguous in k the pairs would
+// have to be put together: 22.5 and 28.8).
 #include "sq_kernels.cuh"
 
 #include <algorithm>
@@ -100,7 +100,7 @@ struct TileCopy {
 // Row i of thread t's T rows of a tile of R.
 template <bool KMAJ, int R, int T>
 __device__ __forceinline__ int tile_row(int t, int i) {
-    return KMAJ ? t + (R / T) * i : T == 8 ? (i / 4) * (R / 2) + t * 4 + i % 4 : t * T + i;
+    return KMAJ ? t + (R / T) * i : t * T + i;
 }
 
 // T fragments of four k steps: f[i][kk].
@@ -286,10 +286,12 @@ int count_tiles(const GemmF32Batch& gb, int bm, int bn) {
 
 // The tile: the largest that still gives most of the 152 SMs a CTA.  A 32 x 64 tile (128
 // threads of 4 x 4) multiplies at the best rate, M = N = K = 512 twice in 20.5 us (64 x 64:
-// 21.4, 32 x 32: 26.9, 16 x 32: 27.0, all let in early, which launch_tiles does not do now); where it leaves SMs idle, one CTA's own pass over K
+// 21.4, 32 x 32: 26.9, 16 x 32: 27.0); where it leaves SMs idle, one CTA's own pass over K
 // is what takes the time, and smaller tiles of smaller fragments are shorter: M 512, N 101,
 // K 512 twice 12.5 us by 32 x 64 (64 CTAs) and 9.3 by 32 x 32 (128), M 32, N 256, K 412
-// twice 11.1, 8.1 and 5.9 us by 32 x 64, 32 x 32 and 16 x 32.
+// twice 11.1, 8.1 and 5.9 us by 32 x 64, 32 x 32 and 16 x 32.  (The choice was measured with every
+// grid let in at its primary's start; as launched now, one such call after another, the chosen tiles
+// take 22.5, 11.6 and 5.6.)
 template <bool A_K, bool B_K>
 void launch_layout(GemmF32Batch& gb, cudaStream_t s) {
     if (count_tiles(gb, 32, 64) >= 100) launch_tiles<32, 64, 4, 4, 32, A_K, B_K>(gb, s);
