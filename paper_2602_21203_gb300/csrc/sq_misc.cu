@@ -374,12 +374,13 @@ __global__ void __launch_bounds__(32 * kC51Rows) c51_target_kernel(C51TargetArgs
             if (lane + 32 * k < K) pb[k] += expf(l[k] - mx) / s;
     }
     const float n_used = pick >= 0 ? 1.f : (float)a.E;
+    const float ent = __fmul_rn(alpha, lp);   // rounded as it is where several atoms share it, for one atom a lane too
 #pragma unroll
     for (int k = 0; k < V; ++k) {
         const int j = lane + 32 * k;
         if (j >= K) break;
         const float zj = a.v_min + (float)j * dz;
-        float tz = r + a.gamma * nd * (zj - alpha * lp);
+        float tz = r + a.gamma * nd * (zj - ent);
         tz = fminf(fmaxf(tz, a.v_min), a.v_max);
         spb[warp][j] = make_float2(pb[k] / n_used, fminf(fmaxf((tz - a.v_min) / dz, 0.f), (float)(K - 1)));
     }
