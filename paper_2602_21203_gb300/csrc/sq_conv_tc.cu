@@ -907,17 +907,25 @@ __global__ void __launch_bounds__(128 * kEncGroups, 1) encoder_tc_kernel(const _
         asm volatile("bar.sync %0, 128;" ::"r"(g + 1) : "memory");
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     };
-    // one thread's bulk copy of an image's input, and all threads' first-layer operand from it
+    // one thread's bulk copy of an image's input, and all threads' first-layer operand from it; nothing
+    // is copied or gathered once a wait has given up
+    uint32_t iphase = 0;      // parity of the next copy to be waited for
+    bool in_flight = false;   // (of the thread that copies)
     auto fetch = [&](int img) {
+        if (!ok) return;
         mbar_expect_tx(ibar, a.ibytes);
         bulk_load(smem_u32(bi), a.x + (int64_t)img * sh.x_img_stride, a.ibytes, ibar);
+        in_flight = true;
     };
-    uint32_t iphase = 0;
     auto gather = [&] {
-        if (!mbar_wait(ibar, iphase, a.err, 44)) ok = false;
-        iphase ^= 1;
-        gather_conv0<0>(a, reinterpret_cast<const float*>(bi), tg, hw, opix, bx, plane0);
-        gather_conv0<1>(a, reinterpret_cast<const float*>(bi), tg, hw, opix, bx, plane0);
+        ok = ok && mbar_wait(ibar, iphase, a.err, 44);
+        if (ok) {
+            iphase ^= 1;
+            in_flight = false;
+            gather_conv0<0>(a, reinterpret_cast<const float*>(bi), tg, hw, opix, bx, plane0);
+            gather_conv0<1>(a, reinterpret_cast<const float*>(bi), tg, hw, opix, bx, plane0);
+        }
+        __syncwarp();
     };
     // this thread's pixels of a layer's output, tile by tile as the MMAs complete: bias, ReLU,
     // BF16, into `dst` (planes of oh ow pixels; unused for the last layer) and to global memory.
@@ -1033,7 +1041,9 @@ __global__ void __launch_bounds__(128 * kEncGroups, 1) encoder_tc_kernel(const _
     if (quarter == 0 && elect_one()) {   // every MMA this group issued has completed before the tensor memory is freed
         mma_commit(bar);
         mbar_wait(bar, phase & 1, a.err, 43);
+        if (in_flight) mbar_wait(ibar, iphase, a.err, 45);   // (after a wait that gave up: copies land before the CTA ends)
     }
+    if (threadIdx.x == 0 && !ok) mbar_wait(wbar, 0, a.err, 45);
     __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
