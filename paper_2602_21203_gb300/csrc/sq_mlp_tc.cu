@@ -630,10 +630,12 @@ __global__ void __launch_bounds__(kFwdThreads, 1) mlp_tc_kernel(const __grid_con
         (void)dead;
     }
     __syncthreads();
-    // after a wait gave up: weight copies issued but never consumed still land in this
+    // after a wait gave up: input and weight copies issued but never consumed still land in this
     // CTA's shared memory; wait for them (bounded) before the CTA can leave
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0) {
+        mbar_wait(x_full, 0, err, 37, wlim);
         for (int i = (int)slot[2]; i < (int)slot[1]; ++i) mbar_wait(full(i % S), (i / S) & 1, err, 37, wlim);
+    }
     // no CTA of the cluster leaves while a peer may still write into its shared memory
     if (CL > 1) cluster_leave();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1106,8 +1108,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_tc_kernel(const __grid_co
         (void)dead;
     }
     __syncthreads();
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0) {
+        mbar_wait(a0_full, 0, err, 47, wlim);
         for (int i = (int)slot[2]; i < (int)slot[1]; ++i) mbar_wait(full(i % S), (i / S) & 1, err, 47, wlim);
+    }
     if (CL > 1) cluster_leave();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
